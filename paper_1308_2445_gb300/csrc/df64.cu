@@ -12,101 +12,46 @@
 
 #include "common.h"
 #include "df64.h"
+#include "gram_tile.h"
 
 namespace hbsd {
 
 namespace {
 
+using df::Seg2d;
 using df::split_d;
 using df::dfma;
 using df::renorm;
 using df::to_d;
 
-struct Seg2d {
-    const double* p0;
-    int64_t ld0;
-    int q0;
-    const double* p1;
-    int64_t ld1;
-    __device__ __forceinline__ double at(int64_t i, int c) const {
-        return c < q0 ? p0[i * ld0 + c] : p1[i * ld1 + (c - q0)];
+// One CTA: a tile (a-block <= b-block, tw = 4 nb columns wide) of Z^T H Z (warps 0-1) and Z^T S Z
+// (warps 2-3) over a chunk of rows.  Bound by the FP32 pipe (10 instructions per multiply-add of
+// pairs, on two packed lanes).  32-wide tiles of 4 x 4 outputs per thread keep the padding of the
+// triangle at 8% for q = 538 (64-wide tiles: 27%) and the warps of a CTA equally loaded; one matrix
+// per warp pair keeps a thread at 128 registers without spills (both matrices in one thread: 24
+// bytes spilled, 49 ms).  Stages of 4 rows, the next one's loads in flight during the sums; FP64
+// sums in shared memory, flushed every 64 rows (with the 10-instruction multiply-add 64 rows are at
+// least as accurate as 128 rows with the 12-instruction one).  n = 334,272, q = 538: 40.6 ms (FP32
+// pipe 2.4e12 pairs/s) against 64.4 ms for 2 x 2 outputs per thread and scalar instructions;
+// n = 47,620, q = 149: 0.64 against 0.89 ms.
+__global__ void __launch_bounds__(GTHREADS, GCTAS) k_gram_df64(Seg2d Z, Seg2d ZH, Seg2d ZS, int q, int64_t n,
+                                                           int64_t rows_per_chunk, int ntile, int nb, df::f32x2 nz,
+                                                           double* __restrict__ partial) {
+    __shared__ GramTile sm;
+    // tile pair: the off-diagonal ones first, then the diagonal ones (half the work)
+    const int noff = ntile * (ntile - 1) / 2;
+    int ta, tb;
+    if ((int)blockIdx.x < noff) {
+        tri_index((int)blockIdx.x, tb, ta);   // ta <= tb of the strict triangle
+        ++tb;
+    } else {
+        ta = tb = (int)blockIdx.x - noff;
     }
-};
-
-constexpr int GT = 32;          // output tile edge
-constexpr int GR = 32;          // rows per shared-memory stage
-constexpr int GFLUSH = 4;       // stages per FP64 flush (128 rows)
-
-// One CTA: a 32 x 32 tile (a-block <= b-block) of Z^T H Z and Z^T S Z over a chunk of rows.
-__global__ void __launch_bounds__(256) k_gram_df64(Seg2d Z, Seg2d ZH, Seg2d ZS, int q,
-                                                   int64_t n, int64_t rows_per_chunk, double* __restrict__ partial) {
-    __shared__ float2 sz[GR][GT + 1], sh[GR][GT + 1], ss[GR][GT + 1];
-    // tile pair (ta <= tb) from the packed-triangle index of the block
-    const int pidx = blockIdx.x;
-    int tb = (int)((sqrtf(8.0f * (float)pidx + 1.0f) - 1.0f) * 0.5f);
-    while ((tb + 1) * (tb + 2) / 2 <= pidx) ++tb;
-    while (tb * (tb + 1) / 2 > pidx) --tb;
-    const int ta = pidx - tb * (tb + 1) / 2;
-    const int a0 = ta * GT, b0 = tb * GT;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;   // 16 x 16 threads, 2 x 2 outputs each
     const int64_t r0 = (int64_t)blockIdx.y * rows_per_chunk;
-    const int64_t r1 = min(n, r0 + rows_per_chunk);
-    double aH[2][2] = {{0, 0}, {0, 0}}, aS[2][2] = {{0, 0}, {0, 0}};
-    float hH[2][2], lH[2][2], hS[2][2], lS[2][2];
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int v = 0; v < 2; ++v) { hH[u][v] = lH[u][v] = hS[u][v] = lS[u][v] = 0.f; }
-    int stage = 0;
-    for (int64_t i0 = r0; i0 < r1; i0 += GR, ++stage) {
-        for (int t = threadIdx.x; t < GR * GT; t += 256) {
-            const int rr = t / GT, cc = t % GT;
-            const int64_t i = i0 + rr;
-            const bool ok = i < r1;
-            sz[rr][cc] = split_d((ok && a0 + cc < q) ? Z.at(i, a0 + cc) : 0.0);
-            sh[rr][cc] = split_d((ok && b0 + cc < q) ? ZH.at(i, b0 + cc) : 0.0);
-            ss[rr][cc] = split_d((ok && b0 + cc < q) ? ZS.at(i, b0 + cc) : 0.0);
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int rr = 0; rr < GR; ++rr) {
-            const float2 z0 = sz[rr][ty * 2], z1 = sz[rr][ty * 2 + 1];
-            const float2 h0 = sh[rr][tx * 2], h1 = sh[rr][tx * 2 + 1];
-            const float2 s0 = ss[rr][tx * 2], s1 = ss[rr][tx * 2 + 1];
-            dfma(z0, h0, hH[0][0], lH[0][0]); dfma(z0, h1, hH[0][1], lH[0][1]);
-            dfma(z1, h0, hH[1][0], lH[1][0]); dfma(z1, h1, hH[1][1], lH[1][1]);
-            dfma(z0, s0, hS[0][0], lS[0][0]); dfma(z0, s1, hS[0][1], lS[0][1]);
-            dfma(z1, s0, hS[1][0], lS[1][0]); dfma(z1, s1, hS[1][1], lS[1][1]);
-            if ((rr & 7) == 7) {
-#pragma unroll
-                for (int u = 0; u < 2; ++u)
-#pragma unroll
-                    for (int v = 0; v < 2; ++v) { renorm(hH[u][v], lH[u][v]); renorm(hS[u][v], lS[u][v]); }
-            }
-        }
-        __syncthreads();
-        if ((stage % GFLUSH) == GFLUSH - 1 || i0 + GR >= r1) {
-#pragma unroll
-            for (int u = 0; u < 2; ++u)
-#pragma unroll
-                for (int v = 0; v < 2; ++v) {
-                    aH[u][v] += to_d(hH[u][v], lH[u][v]);
-                    aS[u][v] += to_d(hS[u][v], lS[u][v]);
-                    hH[u][v] = lH[u][v] = hS[u][v] = lS[u][v] = 0.f;
-                }
-        }
-    }
     const int64_t qq = (int64_t)q * q;
     double* ph = partial + (int64_t)blockIdx.y * 2 * qq;
-    double* ps = ph + qq;
-    for (int u = 0; u < 2; ++u)
-        for (int v = 0; v < 2; ++v) {
-            const int a = a0 + ty * 2 + u, b = b0 + tx * 2 + v;
-            if (a < q && b < q) {
-                ph[(int64_t)a * q + b] = aH[u][v];
-                ps[(int64_t)a * q + b] = aS[u][v];
-            }
-        }
+    gram_df64_tile(sm, Z, ZH, ZS, q, ta * 4 * nb, tb * 4 * nb, nb, ta == tb, r0, min(n, r0 + rows_per_chunk), nz,
+                   [&](int m, int a, int b, double v) { ph[m * qq + (int64_t)a * q + b] = v; });
 }
 
 // Sum the chunks in order; entry (a, b), a <= b, of Z^T X Z is used for both (a, b) and (b, a).
@@ -273,15 +218,17 @@ int gram2_df64(Session* s, const double* Z0, int64_t ld0, int q0, const double* 
                const double* S1, int64_t lds1, int64_t n, double* HR, double* SR, cudaStream_t st) {
     const int q = q0 + q1;
     if (q <= 0) return 0;
-    const int tb = ceil_div(q, GT);
-    const int ntile = tb * (tb + 1) / 2;
-    // chunks of rows: enough CTAs for every SM several times over, a multiple of the stage height
-    int nch = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, ceil_div(152 * 8, ntile)));
+    // tiles of equal width, a multiple of 4 columns up to GW
+    const int ntile = ceil_div(q, GW);
+    const int nb = ceil_div(ceil_div(q, ntile), 4);
+    const int npair = ntile * (ntile + 1) / 2;
+    // chunks of rows: several waves of CTAs, at least 128 rows each
+    int nch = (int)std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, ceil_div(GWAVES * 152 * GCTAS, npair)));
     int64_t rpc = round_up((n + nch - 1) / nch, GR);
     nch = (int)((n + rpc - 1) / rpc);
     HBSD_TRY(s->ws.alloc((size_t)nch * 2 * q * q + 64));
     Seg2d Z{Z0, ld0, q0, Z1, ld1}, ZH{H0, ldh0, q0, H1, ldh1}, ZS{S0, lds0, q0, S1, lds1};
-    k_gram_df64<<<dim3(ntile, nch), 256, 0, st>>>(Z, ZH, ZS, q, n, rpc, s->ws.p);
+    k_gram_df64<<<dim3(npair, nch), GTHREADS, 0, st>>>(Z, ZH, ZS, q, n, rpc, ntile, nb, df::NEG_ZERO2, s->ws.p);
     HBSD_LAUNCHED(s);
     const int64_t qq = (int64_t)q * q;
     k_gram_final_upper<<<ceil_div(qq, 32), 256, 0, st>>>(s->ws.p, nch, q, HR, SR);
