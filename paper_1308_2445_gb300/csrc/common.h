@@ -240,6 +240,10 @@ int rayleigh_ritz(Session* s, const double* HR, const double* SR, int q, int k, 
 int gram2_df64(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1,
                const double* H0, int64_t ldh0, const double* H1, int64_t ldh1, const double* S0, int64_t lds0,
                const double* S1, int64_t lds1, int64_t n, double* HR, double* SR, cudaStream_t st);
+// the Gram on the tensor cores by exact digit slices, at least as accurate (gram_tc.cu)
+int gram2_tc(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, const double* H0,
+             int64_t ldh0, const double* H1, int64_t ldh1, const double* S0, int64_t lds0, const double* S1, int64_t lds1,
+             int64_t n, double* HR, double* SR, cudaStream_t st);
 int update2_df64(Session* s, double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, int64_t n,
                  const double* W, int k, cudaStream_t st, bool split_w);
 // Y = [Z0 Z1] W on the tensor cores by exact bf16 slices (oz.cu); Y must not alias Z0 or Z1

@@ -31,9 +31,8 @@ using df::to_d;
 // per warp pair keeps a thread at 128 registers without spills (both matrices in one thread: 24
 // bytes spilled, 49 ms).  Stages of 4 rows, the next one's loads in flight during the sums; FP64
 // sums in shared memory, flushed every 64 rows (with the 10-instruction multiply-add 64 rows are at
-// least as accurate as 128 rows with the 12-instruction one).  n = 334,272, q = 538: 40.6 ms (FP32
-// pipe 2.4e12 pairs/s) against 64.4 ms for 2 x 2 outputs per thread and scalar instructions;
-// n = 47,620, q = 149: 0.64 against 0.89 ms.
+// least as accurate as 128 rows with the 12-instruction one).  n = 47,620, q = 149: 0.64 ms against
+// 0.89 ms for 2 x 2 outputs per thread and scalar instructions; n = 646, q = 35: 33 against 64 us.
 __global__ void __launch_bounds__(GTHREADS, GCTAS) k_gram_df64(Seg2d Z, Seg2d ZH, Seg2d ZS, int q, int64_t n,
                                                            int64_t rows_per_chunk, int ntile, int nb, df::f32x2 nz,
                                                            double* __restrict__ partial) {
@@ -218,6 +217,12 @@ int gram2_df64(Session* s, const double* Z0, int64_t ld0, int q0, const double* 
                const double* S1, int64_t lds1, int64_t n, double* HR, double* SR, cudaStream_t st) {
     const int q = q0 + q1;
     if (q <= 0) return 0;
+    // Tensor cores from n q^2 = 8e7 on: below it the exponent pass, the lists and the fix-up launch (50 us at
+    // the least) outweigh the products.  Measured on both sides, us (this kernel / tensor cores): q = 71,
+    // n = 6,000: 51 / 59, n = 20,000: 125 / 89; q = 149, n = 2,000: 51 / 61, n = 6,000: 103 / 65; q = 19,
+    // n = 150,000: 145 / 202; q = 35, n = 150,000: 344 / 323; q = 538, n = 646: 121 / 95.
+    if ((double)n * q * q >= 8e7)
+        return gram2_tc(s, Z0, ld0, q0, Z1, ld1, q1, H0, ldh0, H1, ldh1, S0, lds0, S1, lds1, n, HR, SR, st);
     // tiles of equal width, a multiple of 4 columns up to GW
     const int ntile = ceil_div(q, GW);
     const int nb = ceil_div(ceil_div(q, ntile), 4);

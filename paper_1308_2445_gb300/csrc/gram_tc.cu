@@ -1,0 +1,633 @@
+// Gram products of step 8 on the tensor cores, by exact digit slices, with the accuracy of the
+// double-float form guaranteed entry by entry (mixed form: H_R = Z^T ZH, S_R = Z^T ZS, entries a <= b).
+//
+// The splitting idea is that of Ozaki, Ogita, Oishi and Rump ("Error-free transformations of matrix
+// multiplication by using fast routines of matrix multiplication", Numer. Algorithms 59, 2012), in the
+// fixed point of one chunk of rows:
+//  - row i of Z is scaled by 2^-r_i and row i of ZH, ZS by 2^r_i, r_i the exponent of the row's largest
+//    |Z| entry (the rows of an enriched basis span tens of decades, inversely in Z and in ZH, ZS);
+//  - column a of the scaled Z is written as a 62-bit integer against its largest entry of the chunk, and
+//    cut into 8 balanced base-256 digits d_s in [-128, 127] (the leading one in [-64, 64]), each exact in
+//    FP16: slice s holds the digits d_s.  ZH and ZS likewise.
+//  - digit products of equal weight 2^(-8 L), L = s + t <= 7, are summed by tcgen05.mma into one FP32
+//    accumulator per level; over 256 rows the sums of levels 0-4 stay within 2^24, so they are exact, and
+//    the rounding of levels 5-7 is far below the last bit kept.  Levels above 7 are dropped.
+//  - every 256 rows the levels are added in 64-bit integers (unit 2^-37 of the leading digit product),
+//    which hold the whole chunk (at most 8192 rows) without overflow.
+// The truncations leave an error of about sqrt(rows) 2^-61.7 of max|z| max|h| of the scaled columns in the
+// chunk.  That is below the double-float form's rounding, 2^-48 sum|z||h|, wherever
+//     sum|z||h| >= sqrt(rows) 2^-13 max|z| max|h|,
+// which search blocks meet with bits to spare although a few rows dominate their columns (16^3 case: at
+// least 2^-3.8 max|z| max|h|).  The kernel checks it for every entry: it first sums |z||h| (FP16, one MMA
+// per step) over one row in 16, the one with the largest scaled ZH entry of its group, a lower bound
+// within one or two bits on such blocks.  Entries that fail (none to some dozens of a million on the 32^3
+// case) are put on a list and computed in FP64 by k_gram_tc_fixup; a unit (tile and chunk) with more than
+// TG_UNIT_FIX of them, or with a non-finite input, is computed there in double-float (gram_df64_tile).
+//
+// Digit slices are laid out so that one MMA covers several levels: the B slices t = 0, 1, ... of the
+// tile's 32 + 32 columns are adjacent along N and level L's accumulator begins at TMEM column 64 L, so
+// A_s times the window B_0..B_(7-s) accumulates levels s..7 in MMAs of N up to 256 (measured 1176 clocks
+// for the 36 digit products of 16 rows, of which 1152 are the tensor core's minimum; one MMA per product
+// would take at least 50 clocks each).
+//
+// Bound: the integer pipe of the slicers (about 30 integer instructions per value and tile it meets; the
+// tensor core waits for them).  n = 334,272, q = 538: 9.7 ms against 40.5 ms for the FP32 pipes;
+// n = 47,620, q = 149: 0.27 against 0.64 ms.  Error against 64 bits on such blocks 2e-16, float pairs 2e-15.
+#include <algorithm>
+#include <mutex>
+#include <string>
+
+#include "common.h"
+#include "df64.h"
+#include "gram_tile.h"
+#include "tc.h"
+
+namespace hbsd {
+namespace {
+
+using df::Seg2d;
+
+constexpr int TG_M = 128;                       // columns a of a tile (M of every MMA)
+constexpr int TG_B = 32;                        // columns b of a tile, once of ZH and once of ZS
+constexpr int TG_DIG = 8;                       // base-256 digits per operand
+constexpr int TG_BLK = 256;                     // rows per flush of the accumulators
+constexpr int TG_STEPS = TG_BLK / 16;           // MMA steps per flush
+constexpr int TG_MAX_BLKS = 32;                 // flushes per chunk: 8192 rows keep the sums below 2^62
+constexpr int TG_NS = 3;                        // stage buffers
+constexpr int TG_A_SLICE = TG_M * 16 * 2;       // bytes of one 128 x 16 bf16 slice
+constexpr int TG_B_SLICE = 2 * TG_B * 16 * 2;   // bytes of one 64 x 16 bf16 slice
+constexpr int TG_STAGE = TG_DIG * (TG_A_SLICE + TG_B_SLICE);
+constexpr int TG_ACC = 2 * TG_B * TG_M;         // 64-bit sums per unit
+constexpr int TG_ATHREADS = 256;                // warps 0-7: slices of Z, flush
+constexpr int TG_SLICERS = TG_ATHREADS + 128;   // warps 8-11: slices of ZH and ZS
+constexpr int TG_THREADS = TG_SLICERS + 32;     // warp 12: MMA issue
+constexpr size_t TG_SMEM = (size_t)TG_NS * TG_STAGE + (size_t)TG_ACC * 8 + 1024;
+constexpr uint64_t TG_WAIT_NS = 2000000000ull;
+constexpr int TG_BAD_EXP = 0x40000000;          // column exponent of a chunk with a non-finite entry
+constexpr int TG_UNIT_FIX = 256;                // failing entries of a unit that are computed one by one
+constexpr int TG_FRAC = 37;                     // fraction bits of the integer sums
+constexpr int TG_EXP_ROWS = 32;                 // rows per CTA of the exponent pass
+
+__device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
+
+// rexp[i] = exponent field of max_a |Z(i, a)|; cexp[chunk][0][c] = max over the chunk's rows of the
+// exponent field of Z(i, c) minus rexp[i]; cexp[chunk][1..2][c] the same of ZH, ZS plus rexp[i] (memset
+// below every real value before); sel[g] = the row of group g (16 rows) with the largest scaled ZH entry, by
+// exponent.  One pass over the three blocks; a CTA's second read of its Z rows comes from L1.  32 rows
+// per CTA and 16 loads in flight per thread: bound by the latency of the loads (n = 47,620, q = 149:
+// 50 us; with 64 rows and 8 loads 78 us).
+__global__ void __launch_bounds__(256) k_gram_tc_exps(Seg2d Z, Seg2d ZH, Seg2d ZS, int q, int64_t n, int64_t chunk_rows,
+                                                      int* __restrict__ rexp, int* __restrict__ cexp, int* __restrict__ sel) {
+    __shared__ int sr[TG_EXP_ROWS], skey[TG_EXP_ROWS / 16];
+    const int64_t i0 = (int64_t)blockIdx.x * TG_EXP_ROWS;
+    const int rows = (int)min((int64_t)TG_EXP_ROWS, n - i0);
+    if (threadIdx.x < TG_EXP_ROWS) sr[threadIdx.x] = 0;
+    if (threadIdx.x < TG_EXP_ROWS / 16) skey[threadIdx.x] = 0;
+    __syncthreads();
+    for (int c = threadIdx.x; c < ((q + 31) & ~31); c += 256) {   // whole warps
+        int64_t ld;
+        const double* p = Z.column(min(c, q - 1), ld);
+        p += i0 * ld;
+        for (int r0 = 0; r0 < rows; r0 += 16) {
+            int e[16];
+#pragma unroll
+            for (int r = 0; r < 16; ++r) e[r] = r0 + r < rows ? exp_field(p[(r0 + r) * ld]) : 0;
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                const int m = __reduce_max_sync(0xffffffffu, e[r]);
+                if ((threadIdx.x & 31) == r && m > 0) atomicMax(&sr[r0 + r], m);
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < rows) rexp[i0 + threadIdx.x] = sr[threadIdx.x];
+    int* ce = cexp + (i0 / chunk_rows) * 3 * q;
+    for (int t = threadIdx.x; t < ((3 * q + 31) & ~31); t += 256) {
+        const int m = min(t, 3 * q - 1) / q, c = min(t, 3 * q - 1) - m * q;
+        int64_t ld;
+        const double* p = m == 0 ? Z.column(c, ld) : (m == 1 ? ZH.column(c, ld) : ZS.column(c, ld));
+        p += i0 * ld;
+        int e = (int)0x80808080;
+        for (int r0 = 0; r0 < rows; r0 += 16) {
+            int x[16];
+#pragma unroll
+            for (int r = 0; r < 16; ++r) x[r] = r0 + r < rows ? exp_field(p[(r0 + r) * ld]) : 0;
+            int key = 0;
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                const int re = sr[(r0 + r) & (TG_EXP_ROWS - 1)];
+                const int v = x[r] == 2047 ? TG_BAD_EXP : (m == 0 ? x[r] - re : x[r] + re);
+                if (x[r] != 0) {
+                    e = max(e, v);
+                    if (m == 1) key = max(key, ((x[r] + re) << 4) | (15 - r));   // the first of equal rows
+                }
+            }
+            key = __reduce_max_sync(0xffffffffu, key);
+            if ((threadIdx.x & 31) == 0 && key > 0) atomicMax(&skey[r0 / 16], key);
+        }
+        if (t < 3 * q && e > __ldcg(ce + t)) atomicMax(ce + t, e);   // the value only grows: most CTAs need no atomic
+    }
+    __syncthreads();
+    if (threadIdx.x < TG_EXP_ROWS / 16 && threadIdx.x * 16 < rows)
+        sel[i0 / 16 + threadIdx.x] = (int)(threadIdx.x * 16) + 15 - (skey[threadIdx.x] & 15);   // relative to i0
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
+    asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(tc::smem_u32(mbar)) : "memory");
+}
+template <int ACC>
+__device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+                 "l"(a), "l"(b), "r"(idesc), "n"(ACC));
+}
+// slice s of A times the B slices 0 .. 7 - s into levels s .. 7
+template <int S, int ACC>
+__device__ __forceinline__ void mma_window(uint32_t tbase, uint64_t a, uint64_t b) {
+    constexpr int N = (TG_DIG - S) * 2 * TG_B, N0 = N > 256 ? 256 : N;
+    mma<ACC>(tbase + S * 2 * TG_B, a + S * (TG_A_SLICE >> 4), b, tc::idesc_f16_f32(TG_M, N0));
+    if constexpr (N > 256)
+        mma<ACC>(tbase + S * 2 * TG_B + 256, a + S * (TG_A_SLICE >> 4), b + 4 * (TG_B_SLICE >> 4), tc::idesc_f16_f32(TG_M, N - 256));
+}
+
+// |x| as a 62-bit fixed-point integer plus 0x8080808080808080: byte 7 - s is the digit d_s of |x| plus
+// 128.  off: the column's exponent plus or minus the row's; off - exponent field >= 0 is the shift below
+// the maximum.  About 12 integer instructions; the digits of the sign are taken in digits2.
+__device__ __forceinline__ unsigned long long fixed62(double x, int off) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const int ex = (int)((hi >> 20) & 0x7FFu);
+    const unsigned sh = ex ? (unsigned)(off - ex) : 64u;   // zeros and subnormals enter as zero
+    const unsigned mh = __funnelshift_l(lo, (hi & 0xFFFFFu) | 0x100000u, 9), ml = lo << 9;
+    const unsigned t = __funnelshift_rc(ml, mh, sh);   // shifts by at most 32
+    unsigned rl;
+    asm("shr.b32 %0, %1, %2;" : "=r"(rl) : "r"(t), "r"(sh > 32u ? sh - 32u : 0u));   // 0 from 32 on
+    const unsigned rh = __funnelshift_rc(mh, 0u, sh);
+    return (((unsigned long long)rh << 32) | rl) + 0x8080808080808080ull;
+}
+
+// FP16 digits of two values from one byte of each biased word: 1024 + byte by its bits, then
+// (1024 + byte) sg - 1152 sg = +-d exactly, with sg = +-1 the values' signs and csg = -1152 sg
+__device__ __forceinline__ uint32_t digits2(unsigned w0, unsigned w1, int byte, uint32_t sg, uint32_t csg) {
+    const unsigned z = (__byte_perm(w0, w1, (unsigned)(byte | ((4 + byte) << 8))) & 0x00FF00FFu) | 0x64006400u;
+    uint32_t d;
+    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(z), "r"(sg), "r"(csg));
+    return d;
+}
+__device__ __forceinline__ uint32_t signs2(double x0, double x1) {
+    return (__byte_perm((unsigned)__double2hiint(x0), (unsigned)__double2hiint(x1), 0x7030) & 0x80008000u) | 0x3C003C00u;
+}
+
+// The 8 slices of 8 values (consecutive rows of one column): 16 bytes per slice at dst + s * stride
+__device__ __forceinline__ void slice8(const double (&x)[8], const int (&off)[8], uint8_t* dst, int stride) {
+    uint32_t w[TG_DIG][4];
+#pragma unroll
+    for (int c = 0; c < 8; c += 2) {
+        const unsigned long long u0 = fixed62(x[c], off[c]), u1 = fixed62(x[c + 1], off[c + 1]);
+        const uint32_t sg = signs2(x[c], x[c + 1]);
+        uint32_t csg;
+        asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(csg) : "r"(sg), "r"(0xE480E480u));
+#pragma unroll
+        for (int s = 0; s < TG_DIG; ++s)
+            w[s][c >> 1] = digits2((unsigned)(s < 4 ? u0 >> 32 : u0), (unsigned)(s < 4 ? u1 >> 32 : u1), 3 - (s & 3), sg, csg);
+    }
+#pragma unroll
+    for (int s = 0; s < TG_DIG; ++s)
+        *reinterpret_cast<uint4*>(dst + s * stride) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+}
+
+// The guard slice: 8 values as FP16 magnitudes 1.m 2^-shift against the column's leading power of two
+// (m truncated; 0 below 2^-14 of it)
+__device__ __forceinline__ unsigned guard16(double x, int off) {
+    const unsigned hi = (unsigned)__double2hiint(x);
+    const int ex = (int)((hi >> 20) & 0x7FFu), sh = off - ex;
+    return ex != 0 && sh < 15 ? (unsigned)((15 - sh) << 10) | ((hi >> 10) & 0x3FFu) : 0u;
+}
+__device__ __forceinline__ void slice8_guard(const double (&x)[8], const int (&off)[8], uint8_t* dst) {
+    uint32_t w[4];
+#pragma unroll
+    for (int c = 0; c < 8; c += 2) w[c >> 1] = guard16(x[c], off[c]) | (guard16(x[c + 1], off[c + 1]) << 16);
+    *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// tile pair p -> (ta, tb): a-tile ta (128 columns) with the b-tiles tb >= 4 ta of nb, ta-major
+__device__ __forceinline__ void tg_pair(int p, int nb, int& ta, int& tb) {
+    ta = 0;
+    while (p >= nb - 4 * ta) {
+        p -= nb - 4 * ta;
+        ++ta;
+    }
+    tb = 4 * ta + p;
+}
+
+__device__ __forceinline__ void tmem_ld8(uint32_t addr, uint32_t (&v)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(addr));
+}
+
+// One unit: 128 columns a x 32 columns b of both products over one chunk of rows, in phases: phase 0 sums
+// the guard (one step of 16 selected rows per 256-row block), phase p the block p - 1 (16 steps).  Warps 0-11 cut the
+// operands into slices (one thread: 8 rows of one column per step), warp 12 issues the MMAs, warps 0-7
+// read the accumulators after each phase.  Three stages: full[s] completes when the slicers have filled
+// stage s, empty[s] when the MMAs that read it are done, phasedone when a phase's MMAs are done, accfree
+// when its accumulators have been read.  The reading of a phase waits until the slicers are two steps into
+// the next one, so that the MMAs find filled stages afterwards.  list[0] counts the units left to k_gram_tc_fixup
+// (a wait that gives up leaves its unit there too) and list[1] the single entries: units from list[2] on,
+// entries (unit << 13 | matrix << 12 | column b << 7 | column a) from list[2 + units] on.
+__global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Seg2d ZS, int q, int64_t n,
+                                                           int64_t chunk_rows, int nb, const int* __restrict__ rexp,
+                                                           const int* __restrict__ cexp, const int* __restrict__ sel,
+                                                           long long* __restrict__ part, int* __restrict__ list) {
+    extern __shared__ __align__(1024) uint8_t tg_smem[];
+    __shared__ __align__(8) uint64_t full[TG_NS], empty[TG_NS], phasedone, accfree;
+    __shared__ uint32_t tslot;
+    __shared__ int s_flag, s_cnt, s_base, s_ent[TG_UNIT_FIX];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    int ta, tb;
+    tg_pair(blockIdx.x, nb, ta, tb);
+    const int a0 = ta * TG_M, b0 = tb * TG_B;
+    const int64_t r0 = (int64_t)blockIdx.y * chunk_rows, r1 = min(n, r0 + chunk_rows);
+    const int steps = (int)((r1 - r0 + 15) / 16), nblk = (steps + TG_STEPS - 1) / TG_STEPS;
+    const int total = nblk + steps;
+    const int unit = (int)(blockIdx.y * gridDim.x + blockIdx.x);
+    const int* ce = cexp + (int64_t)blockIdx.y * 3 * q;
+    uint8_t* base = tg_smem + ((1024 - (tc::smem_u32(tg_smem) & 1023)) & 1023);
+    long long* sacc = reinterpret_cast<long long*>(base + TG_NS * TG_STAGE);   // [64 columns b][128 columns a]
+    if (tid == 0) {
+        for (int i = 0; i < TG_NS; ++i) {
+            tc::mbar_init(&full[i], TG_SLICERS / 32);
+            tc::mbar_init(&empty[i], 1);
+        }
+        tc::mbar_init(&phasedone, 1);
+        tc::mbar_init(&accfree, TG_ATHREADS / 32);
+        s_flag = 0;
+        s_cnt = 0;
+    }
+    // this thread's column: warps 0-7 column a (tid & 127) of Z, warps 8-11 column b of ZH or ZS
+    const bool isa = warp < TG_ATHREADS / 32;
+    const int bt = tid - TG_ATHREADS, bm = (bt >> 5) & 1;
+    const int col = isa ? a0 + (tid & 127) : b0 + (bt & 31);
+    const int half = isa ? tid >> 7 : (bt >> 6) & 1;
+    const bool live = tid < TG_SLICERS && col < q;
+    const int cmax = live ? ce[(isa ? 0 : (1 + bm) * q) + col] : 0;
+    __syncthreads();
+    if (live && cmax == TG_BAD_EXP) s_flag = 1;
+    if (warp == 0) tc::tmem_alloc(&tslot, 512);
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tbase = tslot;
+
+    if (s_flag != 0) {
+        // non-finite input: the whole unit goes to the fallback
+    } else if (warp == TG_SLICERS / 32) {   // ---- MMA issuer
+        if (lane == 0) {
+            bool ok = true;
+            int st = 0, t = 0;
+            uint32_t ph = 0;
+            for (int p = 0; ok && p <= nblk; ++p) {
+                const int end = p == 0 ? nblk : min(total, nblk + p * TG_STEPS);
+                // the accumulators of the phase before have been read
+                if (p > 0) ok = tc::mbar_wait(&accfree, (uint32_t)((p - 1) & 1), TG_WAIT_NS);
+                for (const int first = t; ok && t < end; ++t) {
+                    ok = tc::mbar_wait(&full[st], ph, TG_WAIT_NS);
+                    if (!ok) break;
+                    tc::fence_after_sync();
+                    const uint64_t a = tc::smem_desc(tc::smem_u32(base + st * TG_STAGE), 128, 256);
+                    const uint64_t b = a + (uint64_t)((TG_DIG * TG_A_SLICE) >> 4);
+                    if (p == 0) {
+                        if (t == first) mma<0>(tbase, a, b, tc::idesc_f16_f32(TG_M, 2 * TG_B));
+                        else mma<1>(tbase, a, b, tc::idesc_f16_f32(TG_M, 2 * TG_B));
+                    } else {
+                        if (t == first) mma_window<0, 0>(tbase, a, b);
+                        else mma_window<0, 1>(tbase, a, b);
+                        mma_window<1, 1>(tbase, a, b);
+                        mma_window<2, 1>(tbase, a, b);
+                        mma_window<3, 1>(tbase, a, b);
+                        mma_window<4, 1>(tbase, a, b);
+                        mma_window<5, 1>(tbase, a, b);
+                        mma_window<6, 1>(tbase, a, b);
+                        mma_window<7, 1>(tbase, a, b);
+                    }
+                    tc::mma_commit(&empty[st]);
+                    if (++st == TG_NS) { st = 0; ph ^= 1u; }
+                }
+                if (ok) tc::mma_commit(&phasedone);
+            }
+            if (!ok) s_flag = 1;
+        }
+    } else {   // ---- slicers, and (warps 0-7) the reading of the accumulators
+        // a thread without a column reads column 0 of its block, with an exponent that shifts it to zero
+        int64_t ld;
+        const int pc = live ? col : 0;
+        const double* p = isa ? Z.column(pc, ld) : (bm ? ZS.column(pc, ld) : ZH.column(pc, ld));
+        const int ebase = live ? cmax : 1 << 20;
+        const int row_in = isa ? tid & 127 : (bt & 31) + TG_B * bm;   // M or N index in the tile
+        const uint32_t soff = (uint32_t)((isa ? 0 : TG_DIG * TG_A_SLICE) + half * 128 + (row_in >> 3) * 256 + (row_in & 7) * 16);
+        const int stride = isa ? TG_A_SLICE : TG_B_SLICE;
+        const int frow = (warp & 3) * 32 + lane, fm = (warp >> 2) & 1;   // column a, matrix of the reading
+        const uint32_t taddr = tbase + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(fm * TG_B);
+        long long* facc = sacc + (int64_t)fm * TG_B * TG_M + frow;
+        if (isa)
+#pragma unroll 4
+            for (int c = 0; c < TG_B; ++c) facc[c * TG_M] = 0;
+        auto read_phase = [&](int ph) -> bool {
+            if (!tc::mbar_wait(&phasedone, (uint32_t)(ph & 1), TG_WAIT_NS)) return false;
+            tc::fence_after_sync();
+            if (ph == 0) {
+                // the guard sums against the chunk's rows (see the head of the file); a column without
+                // entries is exact
+                const float need = sqrtf((float)(r1 - r0)) * 0x1p-11f;   // in units of the columns' leading powers of two
+                const int a = a0 + frow;
+                const bool az = a < q && ce[a] >= -4096;
+#pragma unroll 1
+                for (int c0 = 0; c0 < TG_B; c0 += 8) {
+                    uint32_t v[8];
+                    tmem_ld8(taddr + (uint32_t)c0, v);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        const int b = b0 + c0 + c;
+                        if (az && b < q && a <= b && ce[(1 + fm) * q + b] >= -4096 && !(__uint_as_float(v[c]) >= need)) {
+                            const int k = atomicAdd(&s_cnt, 1);
+                            if (k < TG_UNIT_FIX) s_ent[k] = (fm << 12) | ((c0 + c) << 7) | frow;
+                        }
+                    }
+                }
+            } else {
+#pragma unroll 1
+                for (int c0 = 0; c0 < TG_B; c0 += 8) {
+                    uint32_t v[8][8];
+#pragma unroll
+                    for (int l = 0; l < 8; ++l) tmem_ld8(taddr + (uint32_t)(2 * TG_B * l + c0), v[l]);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        // levels 0 and 1 (within 2^22) by adding 1.5 * 2^23, whose bits then hold the integer;
+                        // levels 2-4 by conversion; levels 5-7 together, rounded to 2^-37 of level 0 (2^3 of level 5)
+                        const int m0 = __float_as_int(__fadd_rn(__uint_as_float(v[0][c]), 12582912.0f)) - 0x4B400000;
+                        const int m1 = __float_as_int(__fadd_rn(__uint_as_float(v[1][c]), 12582912.0f)) - 0x4B400000;
+                        const int m2 = __float2int_rn(__uint_as_float(v[2][c]));
+                        const int m3 = __float2int_rn(__uint_as_float(v[3][c]));
+                        const int m4 = __float2int_rn(__uint_as_float(v[4][c]));
+                        const float g = __fmaf_rn(__fmaf_rn(__uint_as_float(v[7][c]), 0.00390625f, __uint_as_float(v[6][c])),
+                                                  0.00390625f, __uint_as_float(v[5][c]));
+                        const int m5 = __float_as_int(__fmaf_rn(g, 0.125f, 12582912.0f)) - 0x4B400000;
+                        facc[(c0 + c) * TG_M] += (((long long)m0 << 37) + ((long long)m1 << 29)) + (long long)m2 * (1 << 21) +
+                                                 (long long)m3 * (1 << 13) + (long long)m4 * 32 + (long long)m5;
+                    }
+                }
+            }
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&accfree);
+            return true;
+        };
+        // the values and row exponents of the next two steps are on their way while one is sliced
+        double x[2][8];
+        int4 e[2][2];
+        auto fetch = [&](int t, double (&xs)[8], int4 (&es)[2]) {
+            if (t >= total) return;
+            if (t < nblk) {   // the selected rows of block t
+                const int64_t b = r0 + (int64_t)t * TG_BLK;
+                int ee[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const int64_t g = b + (half * 8 + c) * 16;
+                    const int64_t i = g < r1 ? (g & ~(int64_t)(TG_EXP_ROWS - 1)) + sel[g / 16] : r1;
+                    xs[c] = i < r1 ? p[i * ld] : 0.0;
+                    ee[c] = i < r1 ? rexp[i] : 0;
+                }
+                es[0] = make_int4(ee[0], ee[1], ee[2], ee[3]);
+                es[1] = make_int4(ee[4], ee[5], ee[6], ee[7]);
+                return;
+            }
+            const int64_t i = r0 + (int64_t)(t - nblk) * 16 + half * 8;   // rexp is padded to whole blocks
+            es[0] = __ldg(reinterpret_cast<const int4*>(rexp + i));
+            es[1] = __ldg(reinterpret_cast<const int4*>(rexp + i + 4));
+            const double* pi = p + i * ld;
+            if (i + 8 <= r1) {
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    xs[c] = __ldg(pi);
+                    pi += ld;
+                }
+            } else {
+#pragma unroll
+                for (int c = 0; c < 8; ++c) xs[c] = i + c < r1 ? p[(i + c) * ld] : 0.0;
+            }
+        };
+        fetch(0, x[0], e[0]);
+        fetch(1, x[1], e[1]);
+        int st = 0, done = 0, ended = 0, since = 0, next_end = nblk;
+        uint32_t ph = 1;
+        bool ok = true;
+        auto step = [&](int t, double (&xs)[8], int4 (&es)[2]) -> bool {
+            const int sg = isa ? 1 : -1;
+            const int off[8] = {ebase + sg * es[0].x, ebase + sg * es[0].y, ebase + sg * es[0].z, ebase + sg * es[0].w,
+                                ebase + sg * es[1].x, ebase + sg * es[1].y, ebase + sg * es[1].z, ebase + sg * es[1].w};
+            // the first pass over the stages finds them empty (parity 1 of a fresh barrier is complete)
+            if (!tc::mbar_wait(&empty[st], ph, TG_WAIT_NS)) return false;
+            if (t < nblk) slice8_guard(xs, off, base + st * TG_STAGE + soff);
+            else slice8(xs, off, base + st * TG_STAGE + soff, stride);
+            tc::fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&full[st]);   // one arrival per warp
+            fetch(t + 2, xs, es);
+            if (++st == TG_NS) { st = 0; ph ^= 1u; }
+            if (isa) {
+                ++since;
+                if (done < ended && since >= 2) {
+                    if (!read_phase(done)) return false;
+                    ++done;
+                }
+                if (t + 1 == next_end) {   // a phase's last step
+                    ++ended;
+                    since = 0;
+                    next_end = min(total, next_end + TG_STEPS);
+                }
+            }
+            return true;
+        };
+        for (int t = 0; ok && t < total; t += 2) {
+            ok = step(t, x[0], e[0]);
+            if (ok && t + 1 < total) ok = step(t + 1, x[1], e[1]);
+        }
+        if (isa)
+            while (ok && done < ended) {
+                ok = read_phase(done);
+                ++done;
+            }
+        if (!ok) s_flag = 1;
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    if (warp == 0) tc::tmem_dealloc(tbase, 512);
+    const int nfix = s_cnt;
+    if (s_flag || nfix > TG_UNIT_FIX) {
+        if (tid == 0) list[2 + atomicAdd(list, 1)] = unit;
+        return;
+    }
+    if (nfix > 0) {
+        if (tid == 0) s_base = atomicAdd(list + 1, nfix);
+        __syncthreads();
+        int* ents = list + 2 + gridDim.x * gridDim.y + s_base;
+        for (int t = tid; t < nfix; t += TG_THREADS) ents[t] = (unit << 13) | s_ent[t];
+    }
+    long long* out = part + (int64_t)unit * TG_ACC;
+    for (int t = tid; t < TG_ACC; t += TG_THREADS) out[t] = sacc[t];
+}
+
+// An FP64 value in place of a unit's integer: the leading 62 bits under the tag 01, which no sum has
+__device__ __forceinline__ long long tag_double(double v) {
+    return (long long)(0x4000000000000000ull | ((unsigned long long)__double_as_longlong(v) >> 2));
+}
+
+// The listed units in double-float, four 32 x 32 tiles each, and the listed entries in FP64, one CTA each
+__global__ void __launch_bounds__(GTHREADS, GCTAS) k_gram_tc_fixup(Seg2d Z, Seg2d ZH, Seg2d ZS, int q, int64_t n,
+                                                                   int64_t chunk_rows, int nb, int npair, int units,
+                                                                   df::f32x2 nz, long long* __restrict__ part,
+                                                                   const int* __restrict__ list) {
+    __shared__ GramTile sm;
+    const int cnt = list[0], nent = list[1];
+    for (int w = blockIdx.x; w < 4 * cnt; w += gridDim.x) {
+        const int unit = list[2 + (w >> 2)], sub = w & 3;
+        const int chunk = unit / npair;
+        int ta, tb;
+        tg_pair(unit - chunk * npair, nb, ta, tb);
+        const int a0 = ta * TG_M + sub * GW, b0 = tb * TG_B;
+        if (a0 >= q || a0 > b0) continue;   // tiles above the diagonal only (b0 is a multiple of 32)
+        const int64_t r0 = (int64_t)chunk * chunk_rows;
+        long long* out = part + (int64_t)unit * TG_ACC;
+        gram_df64_tile(sm, Z, ZH, ZS, q, a0, b0, GW / 4, false, r0, min(n, r0 + chunk_rows), nz,
+                       [&](int m, int a, int b, double v) { out[(m * TG_B + b - b0) * TG_M + (a - ta * TG_M)] = tag_double(v); });
+        __syncthreads();
+    }
+    double* red = &sm.acc[0][0];
+    for (int w = blockIdx.x; w < nent; w += gridDim.x) {
+        const int code = list[2 + units + w], unit = code >> 13, m = (code >> 12) & 1;
+        const int chunk = unit / npair;
+        int ta, tb;
+        tg_pair(unit - chunk * npair, nb, ta, tb);
+        const int cb = (code >> 7) & 31, ca = code & 127;
+        int64_t lz, lx;
+        const double* z = Z.column(ta * TG_M + ca, lz);
+        const double* x = m ? ZS.column(tb * TG_B + cb, lx) : ZH.column(tb * TG_B + cb, lx);
+        const int64_t r0 = (int64_t)chunk * chunk_rows, r1 = min(n, r0 + chunk_rows);
+        double acc = 0.0;
+        for (int64_t i = r0 + threadIdx.x; i < r1; i += GTHREADS) acc = fma(z[i * lz], x[i * lx], acc);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+        __syncthreads();
+        if (threadIdx.x == 0) part[(int64_t)unit * TG_ACC + (m * TG_B + cb) * TG_M + ca] = tag_double((red[0] + red[1]) + (red[2] + red[3]));
+        __syncthreads();
+    }
+}
+
+// v 2^e without the FP64 pipe (normalise, round to nearest, set the exponent); results outside the normal
+// range by ldexp; a tagged FP64 value as it is
+__device__ __forceinline__ double scaled_double(long long v, int e) {
+    if (v == 0) return 0.0;
+    if ((v >> 62) == 1) return __longlong_as_double(v << 2);
+    const unsigned long long m = (unsigned long long)(v < 0 ? -v : v);
+    const int z = __clzll((long long)m);
+    const int ex = 1023 + 63 - z + e;   // exponent field of the leading bit
+    if (ex < 1 || ex > 2045) return ldexp((double)v, e);
+    const unsigned long long f = m << z;   // leading bit 63; the fraction is the next 52, rounded half up
+    const unsigned long long bits = ((unsigned long long)ex << 52) + ((f << 1) >> 12) + ((f >> 10) & 1ull);
+    return __longlong_as_double((long long)(bits | (v < 0 ? 0x8000000000000000ull : 0ull)));
+}
+
+// Sum of the chunks in order; the entry (a, b), a <= b, is used for (b, a) too.
+__global__ void __launch_bounds__(256) k_gram_tc_final(const long long* __restrict__ part, const int* __restrict__ cexp,
+                                                       int nchunks, int npair, int nb, int q, double* __restrict__ HR,
+                                                       double* __restrict__ SR) {
+    __shared__ double rh[8][33], rs[8][33];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int64_t idx = (int64_t)blockIdx.x * 32 + lane;
+    const int b = (int)(idx / q), a = (int)(idx - (int64_t)b * q);   // lanes over the contiguous index a
+    const bool on = b < q && a <= b;
+    double h = 0.0, s = 0.0;
+    if (on) {
+        const int ta = a / TG_M, tb = b / TG_B;
+        const int pair = ta * nb - 2 * ta * (ta - 1) + tb - 4 * ta;
+        const int64_t o = (int64_t)(b - tb * TG_B) * TG_M + (a - ta * TG_M);
+        for (int c = g; c < nchunks; c += 8) {
+            const long long* p = part + ((int64_t)c * npair + pair) * TG_ACC + o;
+            const int* ce = cexp + (int64_t)c * 3 * q;
+            h += scaled_double(p[0], ce[a] + ce[q + b] - 2056 - TG_FRAC);
+            s += scaled_double(p[(int64_t)TG_B * TG_M], ce[a] + ce[2 * q + b] - 2056 - TG_FRAC);
+        }
+    }
+    rh[g][lane] = h;
+    rs[g][lane] = s;
+    __syncthreads();
+    if (g == 0 && on) {
+        double H = 0.0, S = 0.0;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            H += rh[t][lane];
+            S += rs[t][lane];
+        }
+        HR[(int64_t)a * q + b] = H;
+        SR[(int64_t)a * q + b] = S;
+        HR[(int64_t)b * q + a] = H;
+        SR[(int64_t)b * q + a] = S;
+    }
+}
+
+}  // namespace
+
+int gram2_tc(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, const double* H0,
+             int64_t ldh0, const double* H1, int64_t ldh1, const double* S0, int64_t lds0, const double* S1, int64_t lds1,
+             int64_t n, double* HR, double* SR, cudaStream_t st) {
+    const int q = q0 + q1;
+    const int nb = ceil_div(q, TG_B);
+    int npair = 0;
+    for (int ta = 0; ta * TG_M < q; ++ta) npair += nb - 4 * ta;
+    // chunks of whole 256-row blocks: the height that ends the last wave of units soonest
+    const int nblk = ceil_div(n, TG_BLK);
+    int bpc = 1;
+    double best = 1e300;
+    for (int k = 1; k <= std::min(nblk, TG_MAX_BLKS); ++k) {
+        const double cost = (double)ceil_div((int64_t)npair * ceil_div(nblk, k), 152) * (k + 0.4);
+        if (cost < best) {
+            best = cost;
+            bpc = k;
+        }
+    }
+    const int64_t chunk_rows = (int64_t)bpc * TG_BLK;
+    const int nch = ceil_div(n, chunk_rows);
+    const int64_t units = (int64_t)nch * npair;
+    const int64_t rpad = round_up(n, TG_BLK);
+    // workspace: integer sums | row exponents | column exponents | guard rows | lists
+    const size_t ints = (size_t)rpad + (size_t)nch * 3 * q + (size_t)rpad / 16 + 2 + (size_t)units * (1 + TG_UNIT_FIX);
+    HBSD_TRY(s->ws.alloc((size_t)units * TG_ACC + ints / 2 + 64));
+    long long* part = reinterpret_cast<long long*>(s->ws.p);
+    int* rexp = reinterpret_cast<int*>(part + units * TG_ACC);   // 16-byte aligned: TG_ACC is even
+    int* cexp = rexp + rpad;
+    int* sel = cexp + (size_t)nch * 3 * q;
+    int* list = sel + rpad / 16;
+    HBSD_CUDA(cudaMemsetAsync(cexp, 0x80, (size_t)nch * 3 * q * sizeof(int), st));
+    HBSD_CUDA(cudaMemsetAsync(list, 0, 2 * sizeof(int), st));
+    static std::once_flag once;
+    static cudaError_t attr = cudaSuccess;
+    std::call_once(once, [] {
+        attr = cudaFuncSetAttribute(k_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TG_SMEM);
+    });
+    HBSD_CUDA(attr);
+    Seg2d Z{Z0, ld0, q0, Z1, ld1}, ZH{H0, ldh0, q0, H1, ldh1}, ZS{S0, lds0, q0, S1, lds1};
+    k_gram_tc_exps<<<ceil_div(n, TG_EXP_ROWS), 256, 0, st>>>(Z, ZH, ZS, q, n, chunk_rows, rexp, cexp, sel);
+    HBSD_LAUNCHED(s);
+    k_gram_tc<<<dim3(npair, nch), TG_THREADS, TG_SMEM, st>>>(Z, ZH, ZS, q, n, chunk_rows, nb, rexp, cexp, sel, part, list);
+    HBSD_LAUNCHED(s);
+    k_gram_tc_fixup<<<152 * GCTAS, GTHREADS, 0, st>>>(Z, ZH, ZS, q, n, chunk_rows, nb, npair, (int)units, df::NEG_ZERO2, part,
+                                                      list);
+    HBSD_LAUNCHED(s);
+    k_gram_tc_final<<<ceil_div((int64_t)q * q, 32), 256, 0, st>>>(part, cexp, nch, npair, nb, q, HR, SR);
+    HBSD_LAUNCHED(s);
+    return 0;
+}
+
+}  // namespace hbsd

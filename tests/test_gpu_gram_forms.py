@@ -1,7 +1,9 @@
-"""The double-float Gram at the edges of its tiles, stages and chunks, against FP64 products.
+"""The two forms of the double-float Gram -- float pairs on the FP32 pipes, digit slices on the tensor
+cores from n q^2 = 8e7 on -- at the edges of their tiles, stages and chunks, against FP64 products.
 
-Bound: each entry within 2^-44 of |Z|^T |ZH|: pairs carry 48 bits and keep sums of 64 rows between FP64
-flushes.
+Bound: each entry within 2^-44 of |Z|^T |ZH|.  Pairs carry 48 bits and keep sums of 64 rows between FP64
+flushes; the slices' truncation is held to the same level by the guard and the fix-up of the entries that
+fail it.
 """
 import numpy as np
 import pytest
@@ -49,3 +51,53 @@ def check(Z, ZH, ZS, **kw):
 @pytest.mark.parametrize("q,n", [(1, 1), (4, 3), (31, 63), (32, 64), (33, 65), (64, 129), (97, 5003)])
 def test_gram_df64_tile_edges(q, n):
     check(*blocks(q, n, 100 + q))
+
+
+@pytest.mark.parametrize("q,n", [(538, 300), (129, 5003), (161, 3200), (97, 8705), (71, 17001), (33, 80001)])
+def test_gram_tensor_core_tile_edges(q, n):
+    check(*blocks(q, n, 300 + q))
+
+
+def test_gram_tensor_core_entries_below_the_guard():
+    """Columns whose large entries lie in disjoint rows: the sum of |z||h| is then far below the product of
+    the maxima, so these entries have to come from the fix-up (a few pairs) or the double-float tiles."""
+    q, n = 130, 6000
+    Z, ZH, ZS = blocks(q, n, 900)
+    half = np.arange(n) < n // 2
+    Z[half, 3] *= 1e-7          # one column against its counterparts in ZH, ZS
+    ZH[~half, 40] *= 1e-8
+    ZS[~half, 40] *= 1e-8
+    check(Z, ZH, ZS)
+    Z[half, :64] *= 1e-8        # half of the columns: whole tiles
+    ZH[~half, 64:] *= 1e-8
+    ZS[~half, 64:] *= 1e-8
+    check(Z, ZH, ZS)
+
+
+def test_gram_tensor_core_wild_magnitudes():
+    """Entries over 24 decades without any row or column structure, and zero rows and columns."""
+    q, n = 100, 9000
+    Z, ZH, ZS = (pi.seed_normal_block(70 + i, n, q) * 10.0 ** (24.0 * pi.uniform(80 + i, 9, n * q).reshape(n, q) - 12.0)
+                 for i in range(3))
+    Z[100:140] = 0.0
+    ZH[130:150] = 0.0
+    Z[:, 7] = 0.0
+    ZS[:, 8] = 0.0
+    check(Z, ZH, ZS)
+
+
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_gram_tensor_core_non_finite(bad):
+    """A non-finite entry reaches the entries of its column and leaves the others as they are."""
+    q, n = 130, 6000
+    Z, ZH, ZS = blocks(q, n, 950)
+    Z[4321, 50] = bad
+    HR, SR = gram(Z, ZH, ZS)
+    iu = np.triu_indices(q)
+    hit = (iu[0] == 50)
+    ok = Z.copy()
+    ok[4321, 50] = 0.0
+    for out, B in ((HR, ZH), (SR, ZS)):
+        assert not np.isfinite(out[iu][hit]).any()
+        bound = 2.0 ** -44 * (np.abs(ok).T @ np.abs(B)) + 1e-300
+        assert np.all((np.abs(out - ok.T @ B) <= bound)[iu][~hit])
