@@ -29,10 +29,13 @@
 #include <vector>
 
 #include "common.h"
+#include "rr_math.h"
 
 namespace cg = cooperative_groups;
 
 namespace hbsd {
+
+using namespace rrm;
 
 namespace {
 
@@ -48,42 +51,9 @@ __device__ __forceinline__ uint64_t gtimer() {
     return t;
 }
 
-__device__ __forceinline__ double wsum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// 1/d: an FP32 estimate refined by two Newton steps r <- r + r (1 - d r) (each roughly doubles
-// the correct bits, 24 -> 48 -> full precision); operands outside the FP32 normal range use the
-// IEEE division.
-__device__ __forceinline__ double rcp64(double d) {
-    const double ad = fabs(d);
-    if (!(ad > 1e-30 && ad < 1e30)) return 1.0 / d;
-    double r = (double)(1.0f / (float)d);
-    double e = fma(-d, r, 1.0);
-    r = fma(r, e, r);
-    e = fma(-d, r, 1.0);
-    return fma(r, e, r);
-}
-
 // cluster barrier in two halves: work placed between them overlaps the barrier's latency
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-
-// order-preserving integer key of a double (sorting on the integer pipe)
-__device__ __forceinline__ unsigned long long dkey(double x) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
-}
-
-// (a, b), b <= a, of the p-th entry of a packed lower triangle
-__device__ __forceinline__ void tri_index(int p, int& a, int& b) {
-    a = (int)((sqrtf(8.0f * (float)p + 1.0f) - 1.0f) * 0.5f);
-    while ((a + 1) * (a + 2) / 2 <= p) ++a;
-    while (a * (a + 1) / 2 > p) --a;
-    b = p - a * (a + 1) / 2;
-}
 
 struct RRWork {
     double *Lg, *LgT, *Tg, *Cg, *V, *Y, *Gpart, *d, *e, *lam, *lamr, *scratch;
@@ -561,10 +531,6 @@ __global__ void __launch_bounds__(RR_THREADS_C, 1)
     cluster.sync();
 
     // ---- 5a. eigenvectors of T; eigenvector j on CTA j % NC, warp j / NC ----
-    // Inverse iteration at the coarse shift from a fixed pseudo-random start, then one solve at
-    // the Rayleigh quotient theta = x^T T x.  Pivoted tridiagonal LU with reciprocal pivots,
-    // sequential on lane 0; pivots below eps ||T|| are raised to it, so that a shift on an
-    // eigenvalue amplifies the wanted direction by about 1/eps instead of overflowing.
     const int64_t goff = (int64_t)2 * rb * q + (int64_t)2 * rb * (q + 2);   // G in a global row region
     double* G = grows ? Rg + (int64_t)rank * rper + goff : big;   // phase-5 region
     double* Vr = G + (int64_t)k * k;
@@ -572,148 +538,13 @@ __global__ void __launch_bounds__(RR_THREADS_C, 1)
     double* scr_base = yw + (int64_t)RR_NW * k;
     {
         double* scr = scr_sm ? scr_base + (int64_t)warp * 6 * q : W.scratch + ((int64_t)rank * RR_NW + warp) * 6 * q;
-        double* fdv = scr;             // reciprocals of the U diagonal
-        double* fuv = scr + q;         // first super-diagonal
-        double* fu2v = scr + 2 * q;    // second super-diagonal
-        double* flv = scr + 3 * q;     // multipliers
-        double* fpv = scr + 4 * q;     // pivot flags
-        double* x = scr + 5 * q;       // iterate
-        const double ptd = fmax(DBL_EPSILON * tnorm, pivmin);
-        auto floor_piv = [&](double d) { return fabs(d) < ptd ? (d < 0.0 ? -ptd : ptd) : d; };
-        auto solve64 = [&](double sh) {   // x <- (T - sh I)^{-1} x
-            if (lane == 0) {
-                for (int i = 0; i < q; ++i) { fdv[i] = dd[i] - sh; fuv[i] = ee[i]; fu2v[i] = 0.0; }
-                for (int i = 0; i + 1 < q; ++i) {
-                    const double sub = ee[i];
-                    const double di = fdv[i];
-                    if (fabs(di) >= fabs(sub)) {
-                        const double ri = rcp64(floor_piv(di));
-                        const double f = sub * ri;
-                        fdv[i] = ri;
-                        flv[i] = f;
-                        fpv[i] = 0.0;
-                        fdv[i + 1] = fma(-f, fuv[i], fdv[i + 1]);
-                    } else {
-                        const double ri = rcp64(floor_piv(sub));
-                        const double f = di * ri;
-                        flv[i] = f;
-                        fpv[i] = 1.0;
-                        const double tmp = fuv[i];
-                        fuv[i] = fdv[i + 1];
-                        fdv[i] = ri;
-                        fdv[i + 1] = fma(-f, fdv[i + 1], tmp);
-                        if (i + 2 < q) { fu2v[i] = fuv[i + 1]; fuv[i + 1] = -f * fuv[i + 1]; }
-                    }
-                }
-                fdv[q - 1] = rcp64(floor_piv(fdv[q - 1]));
-                for (int i = 0; i + 1 < q; ++i) {
-                    double bi = x[i], bn = x[i + 1];
-                    if (fpv[i] != 0.0) { const double t2 = bi; bi = bn; bn = t2; }
-                    x[i] = bi;
-                    x[i + 1] = fma(-flv[i], bi, bn);
-                }
-                for (int i = q - 1; i >= 0; --i) {
-                    double sacc = x[i];
-                    if (i + 1 < q) sacc = fma(-fuv[i], x[i + 1], sacc);
-                    if (i + 2 < q) sacc = fma(-fu2v[i], x[i + 2], sacc);
-                    x[i] = sacc * fdv[i];
-                }
-            }
-            __syncwarp();
-        };
-        // x / ||x||; false (x untouched) when an entry of x is not finite or x is zero
-        // (fmax drops NaN, so the entries are tested one by one)
-        auto normalise = [&]() {
-            double mx = 0.0;
-            bool bad = false;
-            for (int i = lane; i < q; i += 32) {
-                bad |= !isfinite(x[i]);
-                mx = fmax(mx, fabs(x[i]));
-            }
-            if (__any_sync(0xffffffffu, bad)) return false;
-            for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-            if (!(mx > 0.0 && isfinite(mx))) return false;
-            const double sc = 1.0 / mx;
-            double n2 = 0.0;
-            for (int i = lane; i < q; i += 32) { x[i] *= sc; n2 = fma(x[i], x[i], n2); }
-            const double inr = rsqrt(wsum(n2));
-            for (int i = lane; i < q; i += 32) x[i] *= inr;
-            __syncwarp();
-            return true;
-        };
         for (int j = rank + NC * warp; j < k && warp < nwr; j += NC * nwr) {
-            for (int i = lane; i < q; i += 32) {
-                uint64_t h = 0x9E3779B97F4A7C15ull * (uint64_t)(j + 1) + 0xBF58476D1CE4E5B9ull * (uint64_t)(i + 1);
-                h ^= h >> 31;
-                h *= 0x94D049BB133111EBull;
-                h ^= h >> 29;
-                x[i] = 0.5 + (double)(h >> 11) * (1.0 / 9007199254740992.0);
-            }
-            __syncwarp();
-            solve64(W.lam[j]);
-            normalise();
-            for (int i = lane; i < q; i += 32) W.V[(int64_t)i * k + j] = x[i];   // kept if the next solve fails
-            double th = 0.0;
-            for (int i = lane; i < q; i += 32) {
-                th = fma(dd[i] * x[i], x[i], th);
-                if (i + 1 < q) th = fma(2.0 * ee[i] * x[i], x[i + 1], th);
-            }
-            th = wsum(th);
-            __syncwarp();
-            solve64(th);
-            bool ok2 = normalise();
-            if (ok2)
+            double th;
+            const int solves = tri_eigenvector(dd, ee, q, k, j, W.lam, tnorm, pivmin, scr, lane, [&](const double* x) {
                 for (int i = lane; i < q; i += 32) W.V[(int64_t)i * k + j] = x[i];
-            // Rayleigh-quotient iteration until the residual ||T x - theta x|| is below
-            // 1e-12 ||T|| (a start vector nearly orthogonal to the wanted eigenvector leaves a
-            // neighbour's component after the first solve): at most three more solves
-            // only for a separated eigenvalue: inside a cluster narrower than 1e-6 ||T|| further
-            // solves would pull several vectors onto one eigenvector, while the mixing they
-            // remove there costs almost nothing (it is weighted by the cluster width).  A vector
-            // is accepted only while its quotient stays in eigenvalue j's interval (midpoints to
-            // the neighbouring coarse eigenvalues): unguarded, the iteration can settle on a
-            // neighbour and duplicate its vector.
-            double gapj = DBL_MAX;
-            if (j > 0) gapj = fmin(gapj, fabs(W.lam[j] - W.lam[j - 1]));
-            if (j + 1 < k) gapj = fmin(gapj, fabs(W.lam[j + 1] - W.lam[j]));
-            const bool separated = gapj > 1e-6 * tnorm;
-            const double lo_j = j > 0 ? 0.5 * (W.lam[j - 1] + W.lam[j]) : -DBL_MAX;
-            const double hi_j = j + 1 < k ? 0.5 * (W.lam[j] + W.lam[j + 1]) : DBL_MAX;
-            auto rayleigh = [&]() {
-                double t2 = 0.0;
-                for (int i = lane; i < q; i += 32) {
-                    t2 = fma(dd[i] * x[i], x[i], t2);
-                    if (i + 1 < q) t2 = fma(2.0 * ee[i] * x[i], x[i + 1], t2);
-                }
-                return wsum(t2);
-            };
-            int extra = 0;
-            if (ok2 && separated) {
-                double th2 = rayleigh();
-                while (extra < 3 && th2 >= lo_j && th2 <= hi_j) {
-                    double r2 = 0.0;
-                    for (int i = lane; i < q; i += 32) {
-                        double ti = fma(dd[i] - th2, x[i], 0.0);
-                        if (i > 0) ti = fma(ee[i - 1], x[i - 1], ti);
-                        if (i + 1 < q) ti = fma(ee[i], x[i + 1], ti);
-                        r2 = fma(ti, ti, r2);
-                    }
-                    r2 = wsum(r2);
-                    __syncwarp();
-                    th = th2;
-                    if (r2 <= (1e-12 * tnorm) * (1e-12 * tnorm)) break;   // far below what the caller resolves
-                    solve64(th);
-                    ++extra;
-                    if (!normalise()) break;               // W.V keeps the last accepted vector
-                    th2 = rayleigh();
-                    __syncwarp();
-                    if (th2 < lo_j || th2 > hi_j) break;   // left the interval: rejected
-                    for (int i = lane; i < q; i += 32) W.V[(int64_t)i * k + j] = x[i];
-                    __syncwarp();
-                }
-            }
+            }, &th);
             if (lane == 0) {
-                vdiag[j] = ok2 ? 1.0 + extra : 0.0;
+                vdiag[j] = (double)solves;
                 vdiag[k + j] = th;
                 vdiag[2 * k + j] = W.lam[j];
             }
@@ -882,6 +713,8 @@ __global__ void __launch_bounds__(RR_THREADS_C, 1)
 
 namespace hbsd {
 
+constexpr int RR_GRID_MIN_Q = 20;
+
 static int cluster_size_for(int q) {
     // 16 CTAs halve each CTA's rows in the tridiagonal reduction; measured faster from q ~ 48
     if (q >= 48) return 16;
@@ -895,6 +728,11 @@ int rayleigh_ritz_cluster(Session* s, const double* HR, const double* SR, int q,
     if (q <= 0 || k <= 0 || k > q) return fail(HBSD_ERR_ARG, "rayleigh_ritz: need 0 < k <= q");
     HBSD_TRY(s->rr_ws.alloc((size_t)std::max<int64_t>(rr_cluster_ws_doubles(q, k, 16, 1), (int64_t)4 * q * q + 3 * q + 64)));
     HBSD_TRY(s->rr_info.alloc(4));
+    // over the whole GPU from 20 columns on, where it is no slower (us, this kernel / whole GPU: q = 20: 349 /
+    // 334, 35: 514 / 471, 64: 847 / 654, 149: 2,450 / 1,396, 538: 44,700 / 8,020); this kernel below, for the
+    // column-dropping mode, and where a cluster of 16 cannot be scheduled
+    const bool grid = drop_tol == 0.0 && q >= RR_GRID_MIN_Q;
+    if (grid) HBSD_TRY(s->rr_ws.alloc(rr_grid_ws_doubles(q, k)));
     static const bool trace = std::getenv("HBSD_TRACE") != nullptr || std::getenv("HBSD_RRDBG") != nullptr;
     static thread_local cudaEvent_t tev[4];
     static thread_local bool tev_made = false;
@@ -909,8 +747,13 @@ int rayleigh_ritz_cluster(Session* s, const double* HR, const double* SR, int q,
     const int pref = cluster_size_for(q);
     // candidates: shared-memory rows on 16, 8, 4, 2, 1 CTAs, then global rows on 16 CTAs (large q)
     const int cands[6] = {16, 8, 4, 2, 1, 16};
-    bool launched = false;
+    bool launched = false, on_grid = false;
     int used_nc = 0, used_stage = 0;
+    if (grid) {
+        HBSD_TRY(rayleigh_ritz_grid(s, HR, SR, q, k, theta, W, s->rr_ws.p, s->rr_info.p, st, &launched));
+        on_grid = launched;
+        if (trace && launched) cudaEventRecord(tev[1], st);
+    }
     for (int ci = 0; ci < 6 && !launched; ++ci) {
         const int NC = cands[ci];
         const int grows = ci == 5 ? 1 : 0;
@@ -973,7 +816,7 @@ int rayleigh_ritz_cluster(Session* s, const double* HR, const double* SR, int q,
     HBSD_CUDA(cudaMemcpyAsync(info, s->rr_info.p, 4 * sizeof(int), cudaMemcpyDeviceToHost, st));
     {
         static const char* dbg = std::getenv("HBSD_RRDBG");
-        if (dbg && dbg[0] == '2') {
+        if (dbg && dbg[0] == '2' && !on_grid) {
             std::vector<double> vd(3 * (size_t)k);
             HBSD_CUDA(cudaMemcpyAsync(vd.data(), s->rr_ws.p + rr_cluster_ws_doubles(q, k, 16, 1) - 3 * k,
                                       3 * k * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -997,7 +840,11 @@ int rayleigh_ritz_cluster(Session* s, const double* HR, const double* SR, int q,
         if (std::getenv("HBSD_TRACE"))
             std::fprintf(stderr, "[hbsd]   RR events: memset+launch %.3f ms, after launch %.3f ms\n", a, b);
     }
-    if (std::getenv("HBSD_TRACE") && !info[3]) {
+    if (on_grid) {   // no column dropped
+        info[0] = 0;
+        info[1] = q;
+    }
+    if (std::getenv("HBSD_TRACE") && !info[3] && !on_grid) {
         uint64_t t[10];
         HBSD_CUDA(cudaMemcpy(t, s->rr_ws.p + rr_stamp_offset(q, k, used_nc), sizeof(t), cudaMemcpyDeviceToHost));
         double tpv[16 * 8];

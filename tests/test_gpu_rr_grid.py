@@ -1,0 +1,76 @@
+"""Rayleigh-Ritz over the whole GPU (from 20 columns on) at the edges of its 32-column blocks, 16 rows per
+cluster round and 16 x 16 tiles, against the oracle.
+
+Tolerances as for the other sizes: eigenvalues to 1e-11 of the largest (the solver's own bar is 1e-9),
+W^T S_R W = I and W^T H_R W = diag(theta) to 1e-10, which FP64 reaches with room on pencils whose scaled S_R
+has a condition number of up to 1e6 (1e-16 * 1e6).
+"""
+import numpy as np
+import pytest
+
+from oracle import labpsd as L
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def run(HR, SR, k):
+    from paper_1308_2445_gb300 import hbsd
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    th = torch.zeros(k, dtype=torch.float64, device="cuda")
+    W = torch.zeros(HR.shape[0], k, dtype=torch.float64, device="cuda")
+    info = torch.zeros(2, dtype=torch.int32, device="cuda")
+    hbsd.rayleigh_ritz(dev(HR), dev(SR), k, th, W, info)
+    torch.cuda.synchronize()
+    return th.cpu().numpy(), W.cpu().numpy(), info.cpu().numpy()
+
+
+def pencil(q, cond, seed):
+    """Spectrum of shells of up to 8 equal eigenvalues, S_R of the given condition, columns of many sizes."""
+    rng = np.random.default_rng(seed)
+    lam = np.repeat(np.cumsum(0.5 + rng.random(q)), rng.integers(1, 9, q))[:q]
+    U, V = (np.linalg.qr(rng.standard_normal((q, q)))[0] for _ in range(2))
+    G = (U * np.sqrt(np.logspace(0, -np.log10(cond), q))) @ V
+    G *= 10.0 ** rng.uniform(-3, 2, q)
+    HR, SR = G.T @ (lam[:, None] * G), G.T @ G
+    return 0.5 * (HR + HR.T), 0.5 * (SR + SR.T)
+
+
+@pytest.mark.parametrize("q,k", [(20, 1), (21, 21), (31, 7), (32, 32), (33, 20), (48, 47), (63, 33), (64, 16), (65, 65),
+                                 (97, 96), (129, 40), (161, 161), (260, 31)])
+def test_block_edges(q, k):
+    HR, SR = pencil(q, 1e3, q)
+    th, W, info = run(HR, SR, k)
+    g, _, fb = L.rayleigh_ritz(HR, SR, k)
+    assert info[0] == 0 and info[1] == q and not fb
+    scale = np.abs(g).max()
+    assert np.abs(th - g).max() <= 1e-11 * scale and np.all(np.diff(th) >= 0)
+    assert np.abs(W.T @ SR @ W - np.eye(k)).max() <= 1e-10
+    assert np.abs(W.T @ HR @ W - np.diag(th)).max() <= 1e-10 * scale
+
+
+def test_ill_conditioned_and_one_shell():
+    HR, SR = pencil(150, 1e6, 5)
+    th, W, info = run(HR, SR, 85)
+    g, _, _ = L.rayleigh_ritz(HR, SR, 85)
+    assert info[0] == 0 and np.abs(th - g).max() <= 1e-9 * np.abs(g).max()
+    assert np.abs(W.T @ SR @ W - np.eye(85)).max() <= 1e-8
+    # every eigenvalue the same: T is diagonal, the vectors are anything orthonormal
+    q = 70
+    th, W, _ = run(3.0 * np.eye(q), np.eye(q), 40)
+    assert np.abs(th - 3.0).max() <= 1e-13
+    assert np.abs(W.T @ W - np.eye(40)).max() <= 1e-12
+
+
+@pytest.mark.parametrize("q,k,ndep", [(64, 30, 2), (150, 85, 5)])
+def test_dependent_columns_reach_the_rank_revealing_branch(q, k, ndep):
+    HR, SR = pencil(q, 10.0, 3 * q)
+    C = np.eye(q)
+    for t in range(ndep):
+        C[:, q - 1 - t] = C[:, t] - 0.5 * C[:, t + 1]
+    HR, SR = C.T @ HR @ C, C.T @ SR @ C
+    HR, SR = 0.5 * (HR + HR.T), 0.5 * (SR + SR.T)
+    th, _, info = run(HR, SR, k)
+    g, _, fb = L.rayleigh_ritz(HR, SR, k)
+    assert fb and info[0] == 1 and info[1] == q - ndep
+    assert np.abs(th - g).max() <= 1e-8 * np.abs(g).max()
