@@ -246,6 +246,16 @@ int gram2_tc(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1
              int64_t n, double* HR, double* SR, cudaStream_t st);
 int update2_df64(Session* s, double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, int64_t n,
                  const double* W, int k, cudaStream_t st, bool split_w);
+// the update on the tensor cores by exact digit slices, at least as accurate (update_tc.cu): in place, 16-byte
+// aligned blocks with even leading dimensions, k <= UPDATE_TC_MAX_K
+constexpr int UPDATE_TC_MAX_K = 512;
+bool update_tc_fits(const double* Z0, int64_t ld0, const double* Z1, int64_t ld1, int q1, int k);
+int update2_tc(Session* s, double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, int64_t n, const double* W,
+               int k, cudaStream_t st);
+// Y = [Z0 Z1] W in double-float (df64.cu); with cnt, only when *cnt > cap on the device
+int update_df64_rows(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, int64_t n,
+                     const double* W, int k, double* Y, int64_t ldy, const unsigned* cnt, unsigned cap, cudaStream_t st,
+                     bool split_w = true);
 // Y = [Z0 Z1] W on the tensor cores by exact bf16 slices (oz.cu); Y must not alias Z0 or Z1
 // status: device int that a timed-out MMA wait sets to 1 (the call is then asynchronous), or NULL
 // (the call checks its own flag and synchronises)
@@ -344,6 +354,7 @@ struct Session {
     DBuf<int> mr_any, mr_steps; // grid barrier + error flag; per-column step counts
     DBuf<unsigned long long> mr_stamps;   // MINRES phase times when tracing
     DBuf<int64_t> mr_blk;       // per-block SELL slot ranges of the fused MINRES kernel
+    DBuf<double> ut_ws;         // tensor-core update (update_tc.cu): slab results, slices of W, exponents, list
     DBuf<float2> df_w;          // double-float copy of the Rayleigh-Ritz coefficients W
     DBuf<double> oz_ws;         // split-slice update: exponents and bf16 slices of W (oz.cu)
     DBuf<int> oz_status;        // set by a timed-out MMA wait of the solve's tensor-core updates

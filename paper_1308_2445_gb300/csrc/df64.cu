@@ -89,12 +89,15 @@ __global__ void __launch_bounds__(256) k_gram_final_upper(const double* __restri
 }
 
 // W (q x k, FP64) -> pairs
-__global__ void k_split_w(const double* __restrict__ W, int64_t cnt, float2* __restrict__ W2) {
+__global__ void k_split_w(const double* __restrict__ W, int64_t cnt, float2* __restrict__ W2, const unsigned* gate,
+                          unsigned cap) {
+    if (gate && __ldcg(gate) <= cap) return;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * blockDim.x)
         W2[t] = split_d(W[t]);
 }
 
-// Z0(:, 0:k) <- [Z0 Z1] W.  Threads are flattened over (row group, column): kc = min(k, 256)
+// Y(:, 0:k) <- [Z0 Z1] W, Y = Z0 allowed (a CTA writes only the rows it has staged).  With gate, only when *gate >
+// cap.  Threads are flattened over (row group, column): kc = min(k, 256)
 // columns per pass, ng = min(256 / kc, 8) row groups of UR rows, so a CTA covers ng * UR rows;
 // the rows (split) and W (q x k pairs) are staged in shared memory, W shared by the row groups.
 // Every output sums its q terms in column order, the running pair renormalised after each
@@ -102,9 +105,11 @@ __global__ void k_split_w(const double* __restrict__ W, int64_t cnt, float2* __r
 constexpr int UR = 8;
 constexpr int RN = 8;
 
-__global__ void __launch_bounds__(256) k_update_df64(double* __restrict__ Z0, int64_t ld0, int q0,
+__global__ void __launch_bounds__(256) k_update_df64(const double* Z0, int64_t ld0, int q0,
                                                      const double* __restrict__ Z1, int64_t ld1, int q1, int64_t n,
-                                                     const float2* __restrict__ W2, int k, int ng) {
+                                                     const float2* __restrict__ W2, int k, int ng, double* Y,
+                                                     int64_t ldy, const unsigned* gate, unsigned cap) {
+    if (gate && __ldcg(gate) <= cap) return;
     extern __shared__ __align__(16) float2 smu[];
     const int q = q0 + q1;
     const int rows = ng * UR;
@@ -150,7 +155,7 @@ __global__ void __launch_bounds__(256) k_update_df64(double* __restrict__ Z0, in
 #pragma unroll
         for (int u = 0; u < UR; ++u) {
             const int64_t i = i0 + g * UR + u;
-            if (i < n) Z0[i * ld0 + j] = to_d(ah[u], al[u]);
+            if (i < n) Y[i * ldy + j] = to_d(ah[u], al[u]);
         }
     }
 }
@@ -161,9 +166,11 @@ __global__ void __launch_bounds__(256) k_update_df64(double* __restrict__ Z0, in
 // time (no other thread of the CTA reads it, so staging it would buy nothing).  Same term order
 // and renormalisation as above.  In place: the outputs are written only after every row of the
 // CTA was staged, and only the staged copy is read.
-__global__ void __launch_bounds__(512) k_update_df64_kt(double* __restrict__ Z0, int64_t ld0, int q0,
+__global__ void __launch_bounds__(512) k_update_df64_kt(const double* Z0, int64_t ld0, int q0,
                                                         const double* __restrict__ Z1, int64_t ld1, int q1, int64_t n,
-                                                        const float2* __restrict__ W2, int k) {
+                                                        const float2* __restrict__ W2, int k, double* Y, int64_t ldy,
+                                                        const unsigned* gate, unsigned cap) {
+    if (gate && __ldcg(gate) <= cap) return;
     extern __shared__ __align__(16) float2 smu[];
     const int q = q0 + q1;
     const int nt = blockDim.x;
@@ -205,7 +212,7 @@ __global__ void __launch_bounds__(512) k_update_df64_kt(double* __restrict__ Z0,
 #pragma unroll
         for (int u = 0; u < UR; ++u) {
             const int64_t i = i0 + u;
-            if (i < n) Z0[i * ld0 + j] = to_d(ah[u], al[u]);
+            if (i < n) Y[i * ldy + j] = to_d(ah[u], al[u]);
         }
     }
 }
@@ -245,6 +252,22 @@ int update2_df64(Session* s, double* Z0, int64_t ld0, int q0, const double* Z1, 
                  const double* W, int k, cudaStream_t st, bool split_w) {
     const int q = q0 + q1;
     if (k > q0) return fail(HBSD_ERR_ARG, "update: k must not exceed the first segment width");
+    // On the tensor cores from here (us, pairs / digit slices; n, q, k): 20000, 149, 85: 187 / 157; 47620, 112, 56:
+    // 172 / 153; 6000, 538, 282: 459 / 328; 20000, 538, 282: 1,441 / 733.  Below, one CTA's chain of column tiles
+    // and the passes over Z for exponents and guard cost more: 20000, 128, 64: 106 / 117; 6000, 282, 150: 156 /
+    // 165; 646, 538, 282: 139 / 322; with half-empty column tiles 150000, 96, 48: 373 / 402.
+    if (n >= 6144 && k >= 56 && (double)n * q * k >= 2e8) {
+        if ((size_t)UR * q * sizeof(float2) <= 220 * 1024 && update_tc_fits(Z0, ld0, Z1, ld1, q1, k))
+            return update2_tc(s, Z0, ld0, q0, Z1, ld1, q1, n, W, k, st);
+        split_w = true;   // an earlier block of the same step may have gone the other way and left df_w alone
+    }
+    return update_df64_rows(s, Z0, ld0, q0, Z1, ld1, q1, n, W, k, Z0, ld0, nullptr, 0, st, split_w);
+}
+
+int update_df64_rows(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, int64_t n,
+                     const double* W, int k, double* Y, int64_t ldy, const unsigned* cnt, unsigned cap, cudaStream_t st,
+                     bool split_w) {
+    const int q = q0 + q1;
     // W staged whole when it fits with the rows (kernel k_update_df64), else read by each
     // thread from L2 (k_update_df64_kt: passes of nt <= 512 columns, as even as multiples of 32
     // allow, one pass for k <= 512)
@@ -269,12 +292,12 @@ int update2_df64(Session* s, double* Z0, int64_t ld0, int q0, const double* Z1, 
     }
     HBSD_TRY(s->df_w.alloc((size_t)q * k));
     if (split_w) {
-        const int64_t cnt = (int64_t)q * k;
-        k_split_w<<<ceil_div(cnt, 256), 256, 0, st>>>(W, cnt, s->df_w.p);
+        const int64_t wcnt = (int64_t)q * k;
+        k_split_w<<<ceil_div(wcnt, 256), 256, 0, st>>>(W, wcnt, s->df_w.p, cnt, cap);
         HBSD_LAUNCHED(s);
     }
-    if (whole) k_update_df64<<<ceil_div(n, rows), 256, smem, st>>>(Z0, ld0, q0, Z1, ld1, q1, n, s->df_w.p, k, ng);
-    else k_update_df64_kt<<<ceil_div(n, UR), nt, smem, st>>>(Z0, ld0, q0, Z1, ld1, q1, n, s->df_w.p, k);
+    if (whole) k_update_df64<<<ceil_div(n, rows), 256, smem, st>>>(Z0, ld0, q0, Z1, ld1, q1, n, s->df_w.p, k, ng, Y, ldy, cnt, cap);
+    else k_update_df64_kt<<<ceil_div(n, UR), nt, smem, st>>>(Z0, ld0, q0, Z1, ld1, q1, n, s->df_w.p, k, Y, ldy, cnt, cap);
     HBSD_LAUNCHED(s);
     return 0;
 }

@@ -40,35 +40,29 @@
 #include "common.h"
 #include "df64.h"
 #include "gram_tile.h"
+#include "slices.h"
 #include "tc.h"
 
 namespace hbsd {
 namespace {
 
 using df::Seg2d;
+using namespace slices;
 
 constexpr int TG_M = 128;                       // columns a of a tile (M of every MMA)
 constexpr int TG_B = 32;                        // columns b of a tile, once of ZH and once of ZS
-constexpr int TG_DIG = 8;                       // base-256 digits per operand
 constexpr int TG_BLK = 256;                     // rows per flush of the accumulators
-constexpr int TG_STEPS = TG_BLK / 16;           // MMA steps per flush
+constexpr int TG_STEPS = FLUSH_STEPS;           // MMA steps per flush
 constexpr int TG_MAX_BLKS = 32;                 // flushes per chunk: 8192 rows keep the sums below 2^62
 constexpr int TG_NS = 3;                        // stage buffers
-constexpr int TG_A_SLICE = TG_M * 16 * 2;       // bytes of one 128 x 16 bf16 slice
-constexpr int TG_B_SLICE = 2 * TG_B * 16 * 2;   // bytes of one 64 x 16 bf16 slice
-constexpr int TG_STAGE = TG_DIG * (TG_A_SLICE + TG_B_SLICE);
+constexpr int TG_STAGE = DIG * (A_SLICE + B_SLICE);
 constexpr int TG_ACC = 2 * TG_B * TG_M;         // 64-bit sums per unit
 constexpr int TG_ATHREADS = 256;                // warps 0-7: slices of Z, flush
 constexpr int TG_SLICERS = TG_ATHREADS + 128;   // warps 8-11: slices of ZH and ZS
 constexpr int TG_THREADS = TG_SLICERS + 32;     // warp 12: MMA issue
 constexpr size_t TG_SMEM = (size_t)TG_NS * TG_STAGE + (size_t)TG_ACC * 8 + 1024;
-constexpr uint64_t TG_WAIT_NS = 2000000000ull;
-constexpr int TG_BAD_EXP = 0x40000000;          // column exponent of a chunk with a non-finite entry
 constexpr int TG_UNIT_FIX = 256;                // failing entries of a unit that are computed one by one
-constexpr int TG_FRAC = 37;                     // fraction bits of the integer sums
 constexpr int TG_EXP_ROWS = 32;                 // rows per CTA of the exponent pass
-
-__device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
 
 // rexp[i] = exponent field of max_a |Z(i, a)|; cexp[chunk][0][c] = max over the chunk's rows of the
 // exponent field of Z(i, c) minus rexp[i]; cexp[chunk][1..2][c] the same of ZH, ZS plus rexp[i] (memset
@@ -116,7 +110,7 @@ __global__ void __launch_bounds__(256) k_gram_tc_exps(Seg2d Z, Seg2d ZH, Seg2d Z
 #pragma unroll
             for (int r = 0; r < 16; ++r) {
                 const int re = sr[(r0 + r) & (TG_EXP_ROWS - 1)];
-                const int v = x[r] == 2047 ? TG_BAD_EXP : (m == 0 ? x[r] - re : x[r] + re);
+                const int v = x[r] == 2047 ? BAD_EXP : (m == 0 ? x[r] - re : x[r] + re);
                 if (x[r] != 0) {
                     e = max(e, v);
                     if (m == 1) key = max(key, ((x[r] + re) << 4) | (15 - r));   // the first of equal rows
@@ -132,82 +126,6 @@ __global__ void __launch_bounds__(256) k_gram_tc_exps(Seg2d Z, Seg2d ZH, Seg2d Z
         sel[i0 / 16 + threadIdx.x] = (int)(threadIdx.x * 16) + 15 - (skey[threadIdx.x] & 15);   // relative to i0
 }
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
-    asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(tc::smem_u32(mbar)) : "memory");
-}
-template <int ACC>
-__device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc) {
-    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-                 "l"(a), "l"(b), "r"(idesc), "n"(ACC));
-}
-// slice s of A times the B slices 0 .. 7 - s into levels s .. 7
-template <int S, int ACC>
-__device__ __forceinline__ void mma_window(uint32_t tbase, uint64_t a, uint64_t b) {
-    constexpr int N = (TG_DIG - S) * 2 * TG_B, N0 = N > 256 ? 256 : N;
-    mma<ACC>(tbase + S * 2 * TG_B, a + S * (TG_A_SLICE >> 4), b, tc::idesc_f16_f32(TG_M, N0));
-    if constexpr (N > 256)
-        mma<ACC>(tbase + S * 2 * TG_B + 256, a + S * (TG_A_SLICE >> 4), b + 4 * (TG_B_SLICE >> 4), tc::idesc_f16_f32(TG_M, N - 256));
-}
-
-// |x| as a 62-bit fixed-point integer plus 0x8080808080808080: byte 7 - s is the digit d_s of |x| plus
-// 128.  off: the column's exponent plus or minus the row's; off - exponent field >= 0 is the shift below
-// the maximum.  About 12 integer instructions; the digits of the sign are taken in digits2.
-__device__ __forceinline__ unsigned long long fixed62(double x, int off) {
-    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    const int ex = (int)((hi >> 20) & 0x7FFu);
-    const unsigned sh = ex ? (unsigned)(off - ex) : 64u;   // zeros and subnormals enter as zero
-    const unsigned mh = __funnelshift_l(lo, (hi & 0xFFFFFu) | 0x100000u, 9), ml = lo << 9;
-    const unsigned t = __funnelshift_rc(ml, mh, sh);   // shifts by at most 32
-    unsigned rl;
-    asm("shr.b32 %0, %1, %2;" : "=r"(rl) : "r"(t), "r"(sh > 32u ? sh - 32u : 0u));   // 0 from 32 on
-    const unsigned rh = __funnelshift_rc(mh, 0u, sh);
-    return (((unsigned long long)rh << 32) | rl) + 0x8080808080808080ull;
-}
-
-// FP16 digits of two values from one byte of each biased word: 1024 + byte by its bits, then
-// (1024 + byte) sg - 1152 sg = +-d exactly, with sg = +-1 the values' signs and csg = -1152 sg
-__device__ __forceinline__ uint32_t digits2(unsigned w0, unsigned w1, int byte, uint32_t sg, uint32_t csg) {
-    const unsigned z = (__byte_perm(w0, w1, (unsigned)(byte | ((4 + byte) << 8))) & 0x00FF00FFu) | 0x64006400u;
-    uint32_t d;
-    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(z), "r"(sg), "r"(csg));
-    return d;
-}
-__device__ __forceinline__ uint32_t signs2(double x0, double x1) {
-    return (__byte_perm((unsigned)__double2hiint(x0), (unsigned)__double2hiint(x1), 0x7030) & 0x80008000u) | 0x3C003C00u;
-}
-
-// The 8 slices of 8 values (consecutive rows of one column): 16 bytes per slice at dst + s * stride
-__device__ __forceinline__ void slice8(const double (&x)[8], const int (&off)[8], uint8_t* dst, int stride) {
-    uint32_t w[TG_DIG][4];
-#pragma unroll
-    for (int c = 0; c < 8; c += 2) {
-        const unsigned long long u0 = fixed62(x[c], off[c]), u1 = fixed62(x[c + 1], off[c + 1]);
-        const uint32_t sg = signs2(x[c], x[c + 1]);
-        uint32_t csg;
-        asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(csg) : "r"(sg), "r"(0xE480E480u));
-#pragma unroll
-        for (int s = 0; s < TG_DIG; ++s)
-            w[s][c >> 1] = digits2((unsigned)(s < 4 ? u0 >> 32 : u0), (unsigned)(s < 4 ? u1 >> 32 : u1), 3 - (s & 3), sg, csg);
-    }
-#pragma unroll
-    for (int s = 0; s < TG_DIG; ++s)
-        *reinterpret_cast<uint4*>(dst + s * stride) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
-}
-
-// The guard slice: 8 values as FP16 magnitudes 1.m 2^-shift against the column's leading power of two
-// (m truncated; 0 below 2^-14 of it)
-__device__ __forceinline__ unsigned guard16(double x, int off) {
-    const unsigned hi = (unsigned)__double2hiint(x);
-    const int ex = (int)((hi >> 20) & 0x7FFu), sh = off - ex;
-    return ex != 0 && sh < 15 ? (unsigned)((15 - sh) << 10) | ((hi >> 10) & 0x3FFu) : 0u;
-}
-__device__ __forceinline__ void slice8_guard(const double (&x)[8], const int (&off)[8], uint8_t* dst) {
-    uint32_t w[4];
-#pragma unroll
-    for (int c = 0; c < 8; c += 2) w[c >> 1] = guard16(x[c], off[c]) | (guard16(x[c + 1], off[c + 1]) << 16);
-    *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-}
-
 // tile pair p -> (ta, tb): a-tile ta (128 columns) with the b-tiles tb >= 4 ta of nb, ta-major
 __device__ __forceinline__ void tg_pair(int p, int nb, int& ta, int& tb) {
     ta = 0;
@@ -216,12 +134,6 @@ __device__ __forceinline__ void tg_pair(int p, int nb, int& ta, int& tb) {
         ++ta;
     }
     tb = 4 * ta + p;
-}
-
-__device__ __forceinline__ void tmem_ld8(uint32_t addr, uint32_t (&v)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-                 : "r"(addr));
 }
 
 // One unit: 128 columns a x 32 columns b of both products over one chunk of rows, in phases: phase 0 sums
@@ -270,7 +182,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
     const bool live = tid < TG_SLICERS && col < q;
     const int cmax = live ? ce[(isa ? 0 : (1 + bm) * q) + col] : 0;
     __syncthreads();
-    if (live && cmax == TG_BAD_EXP) s_flag = 1;
+    if (live && cmax == BAD_EXP) s_flag = 1;
     if (warp == 0) tc::tmem_alloc(&tslot, 512);
     tc::fence_before_sync();
     __syncthreads();
@@ -287,13 +199,13 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
             for (int p = 0; ok && p <= nblk; ++p) {
                 const int end = p == 0 ? nblk : min(total, nblk + p * TG_STEPS);
                 // the accumulators of the phase before have been read
-                if (p > 0) ok = tc::mbar_wait(&accfree, (uint32_t)((p - 1) & 1), TG_WAIT_NS);
+                if (p > 0) ok = tc::mbar_wait(&accfree, (uint32_t)((p - 1) & 1), WAIT_NS);
                 for (const int first = t; ok && t < end; ++t) {
-                    ok = tc::mbar_wait(&full[st], ph, TG_WAIT_NS);
+                    ok = tc::mbar_wait(&full[st], ph, WAIT_NS);
                     if (!ok) break;
                     tc::fence_after_sync();
                     const uint64_t a = tc::smem_desc(tc::smem_u32(base + st * TG_STAGE), 128, 256);
-                    const uint64_t b = a + (uint64_t)((TG_DIG * TG_A_SLICE) >> 4);
+                    const uint64_t b = a + (uint64_t)((DIG * A_SLICE) >> 4);
                     if (p == 0) {
                         if (t == first) mma<0>(tbase, a, b, tc::idesc_f16_f32(TG_M, 2 * TG_B));
                         else mma<1>(tbase, a, b, tc::idesc_f16_f32(TG_M, 2 * TG_B));
@@ -322,8 +234,8 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
         const double* p = isa ? Z.column(pc, ld) : (bm ? ZS.column(pc, ld) : ZH.column(pc, ld));
         const int ebase = live ? cmax : 1 << 20;
         const int row_in = isa ? tid & 127 : (bt & 31) + TG_B * bm;   // M or N index in the tile
-        const uint32_t soff = (uint32_t)((isa ? 0 : TG_DIG * TG_A_SLICE) + half * 128 + (row_in >> 3) * 256 + (row_in & 7) * 16);
-        const int stride = isa ? TG_A_SLICE : TG_B_SLICE;
+        const uint32_t soff = (uint32_t)((isa ? 0 : DIG * A_SLICE) + half * 128 + (row_in >> 3) * 256 + (row_in & 7) * 16);
+        const int stride = isa ? A_SLICE : B_SLICE;
         const int frow = (warp & 3) * 32 + lane, fm = (warp >> 2) & 1;   // column a, matrix of the reading
         const uint32_t taddr = tbase + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(fm * TG_B);
         long long* facc = sacc + (int64_t)fm * TG_B * TG_M + frow;
@@ -331,7 +243,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
 #pragma unroll 4
             for (int c = 0; c < TG_B; ++c) facc[c * TG_M] = 0;
         auto read_phase = [&](int ph) -> bool {
-            if (!tc::mbar_wait(&phasedone, (uint32_t)(ph & 1), TG_WAIT_NS)) return false;
+            if (!tc::mbar_wait(&phasedone, (uint32_t)(ph & 1), WAIT_NS)) return false;
             tc::fence_after_sync();
             if (ph == 0) {
                 // the guard sums against the chunk's rows (see the head of the file); a column without
@@ -362,18 +274,8 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
                     asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
-                        // levels 0 and 1 (within 2^22) by adding 1.5 * 2^23, whose bits then hold the integer;
-                        // levels 2-4 by conversion; levels 5-7 together, rounded to 2^-37 of level 0 (2^3 of level 5)
-                        const int m0 = __float_as_int(__fadd_rn(__uint_as_float(v[0][c]), 12582912.0f)) - 0x4B400000;
-                        const int m1 = __float_as_int(__fadd_rn(__uint_as_float(v[1][c]), 12582912.0f)) - 0x4B400000;
-                        const int m2 = __float2int_rn(__uint_as_float(v[2][c]));
-                        const int m3 = __float2int_rn(__uint_as_float(v[3][c]));
-                        const int m4 = __float2int_rn(__uint_as_float(v[4][c]));
-                        const float g = __fmaf_rn(__fmaf_rn(__uint_as_float(v[7][c]), 0.00390625f, __uint_as_float(v[6][c])),
-                                                  0.00390625f, __uint_as_float(v[5][c]));
-                        const int m5 = __float_as_int(__fmaf_rn(g, 0.125f, 12582912.0f)) - 0x4B400000;
-                        facc[(c0 + c) * TG_M] += (((long long)m0 << 37) + ((long long)m1 << 29)) + (long long)m2 * (1 << 21) +
-                                                 (long long)m3 * (1 << 13) + (long long)m4 * 32 + (long long)m5;
+                        const uint32_t l[8] = {v[0][c], v[1][c], v[2][c], v[3][c], v[4][c], v[5][c], v[6][c], v[7][c]};
+                        facc[(c0 + c) * TG_M] += fold_levels(l);
                     }
                 }
             }
@@ -426,7 +328,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
             const int off[8] = {ebase + sg * es[0].x, ebase + sg * es[0].y, ebase + sg * es[0].z, ebase + sg * es[0].w,
                                 ebase + sg * es[1].x, ebase + sg * es[1].y, ebase + sg * es[1].z, ebase + sg * es[1].w};
             // the first pass over the stages finds them empty (parity 1 of a fresh barrier is complete)
-            if (!tc::mbar_wait(&empty[st], ph, TG_WAIT_NS)) return false;
+            if (!tc::mbar_wait(&empty[st], ph, WAIT_NS)) return false;
             if (t < nblk) slice8_guard(xs, off, base + st * TG_STAGE + soff);
             else slice8(xs, off, base + st * TG_STAGE + soff, stride);
             tc::fence_proxy_async();
@@ -525,18 +427,9 @@ __global__ void __launch_bounds__(GTHREADS, GCTAS) k_gram_tc_fixup(Seg2d Z, Seg2
     }
 }
 
-// v 2^e without the FP64 pipe (normalise, round to nearest, set the exponent); results outside the normal
-// range by ldexp; a tagged FP64 value as it is
-__device__ __forceinline__ double scaled_double(long long v, int e) {
-    if (v == 0) return 0.0;
-    if ((v >> 62) == 1) return __longlong_as_double(v << 2);
-    const unsigned long long m = (unsigned long long)(v < 0 ? -v : v);
-    const int z = __clzll((long long)m);
-    const int ex = 1023 + 63 - z + e;   // exponent field of the leading bit
-    if (ex < 1 || ex > 2045) return ldexp((double)v, e);
-    const unsigned long long f = m << z;   // leading bit 63; the fraction is the next 52, rounded half up
-    const unsigned long long bits = ((unsigned long long)ex << 52) + ((f << 1) >> 12) + ((f >> 10) & 1ull);
-    return __longlong_as_double((long long)(bits | (v < 0 ? 0x8000000000000000ull : 0ull)));
+// A unit's sum, or a tagged FP64 value
+__device__ __forceinline__ double unit_value(long long v, int e) {
+    return (v >> 62) == 1 ? __longlong_as_double(v << 2) : scaled_double(v, e);
 }
 
 // Sum of the chunks in order; the entry (a, b), a <= b, is used for (b, a) too.
@@ -556,8 +449,8 @@ __global__ void __launch_bounds__(256) k_gram_tc_final(const long long* __restri
         for (int c = g; c < nchunks; c += 8) {
             const long long* p = part + ((int64_t)c * npair + pair) * TG_ACC + o;
             const int* ce = cexp + (int64_t)c * 3 * q;
-            h += scaled_double(p[0], ce[a] + ce[q + b] - 2056 - TG_FRAC);
-            s += scaled_double(p[(int64_t)TG_B * TG_M], ce[a] + ce[2 * q + b] - 2056 - TG_FRAC);
+            h += unit_value(p[0], ce[a] + ce[q + b] - 2056 - FRAC);
+            s += unit_value(p[(int64_t)TG_B * TG_M], ce[a] + ce[2 * q + b] - 2056 - FRAC);
         }
     }
     rh[g][lane] = h;

@@ -176,8 +176,9 @@ struct StepTimer {
     }
 };
 
-// Gram and update of the loop: the mixed form computes them in double-float arithmetic on the
-// FP32 pipes (FP64 accumulation across 128-row tiles for the Gram sums), the FP64 form in FP64.
+// Gram and update of the loop: the mixed form computes them in double-float arithmetic on the FP32 pipes (FP64
+// accumulation across the rows for the Gram sums) or, from the sizes on where that is faster, from exact digit
+// slices on the tensor cores; the FP64 form in FP64.
 template <class T>
 static int gram_step(Session* S, bool df, const T* Z0, int64_t ld0, int q0, const T* Z1, int64_t ld1, int q1,
                      const T* H0, int64_t ldh0, const T* H1, int64_t ldh1, const T* S0, int64_t lds0, const T* S1,
