@@ -123,15 +123,15 @@ struct Sell {
     DBuf<double> dinv;          // D^-1
     std::vector<double> h_dscale;
     std::vector<int64_t> h_slice_ptr;
-    std::vector<int32_t> h_slot_row, h_cols;
+    std::vector<int32_t> h_slot_row;
     DBuf<int32_t> slot_row;     // original row of each slot (-1 for padding slots)
-    std::vector<int64_t> h_entry_of_csr;  // stored position of each CSR entry (host, for updates)
+    DBuf<int64_t> row_ptr;      // CSR row offsets, and CSR values on their way into hs: for updates of H
+    DBuf<double> val;
 };
 
 int sell_build(Sell& m, int64_t n, const int64_t* row_ptr, const int32_t* col_idx,
                const double* hval, const double* sval, double sigma0);
-int sell_update_h(Sell& m, const double* hval, const double* sval, double sigma0);
-int sell_fill_fp32(Sell& m, const double2* hs, const int32_t* cols, const int32_t* slot_row);
+int sell_update_h(Sell& m, const double* hval, double sigma0);
 
 // Y_h = Hs X, Y_s = S X for k columns; X, Y row-major.
 template <class T>
@@ -340,8 +340,6 @@ struct Session {
     bool has_factor = false;
     hbsd_stats stats{};
     int launches = 0;
-    // CSR kept on host for hbsd_update_H
-    std::vector<double> h_sval;
     // workspaces (FP64 driver)
     DBuf<double> ws;            // generic scratch for reductions
     DBuf<double> rr_ws;         // Rayleigh-Ritz workspace

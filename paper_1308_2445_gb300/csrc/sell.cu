@@ -20,6 +20,85 @@
 
 namespace hbsd {
 
+// D = diag(S)^{-1/2} and its inverse, a warp per row (the last positive diagonal entry; 1 without one)
+__global__ void __launch_bounds__(256) k_sell_dscale(int64_t n, const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
+                                                     const double* __restrict__ sval, double* __restrict__ dscale,
+                                                     double* __restrict__ dinv) {
+    const int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (r >= n) return;
+    const int64_t e0 = row_ptr[r];
+    const int len = (int)(row_ptr[r + 1] - e0);
+    int last = -1;
+    for (int j = lane; j < len; j += 32)
+        if (col_idx[e0 + j] == r && sval[e0 + j] > 0.0) last = j;
+    last = __reduce_max_sync(0xffffffffu, last);
+    if (lane == 0) {
+        const double d = last >= 0 ? __ddiv_rn(1.0, __dsqrt_rn(sval[e0 + last])) : 1.0;
+        dscale[r] = d;
+        dinv[r] = __ddiv_rn(1.0, d);
+    }
+}
+
+// A warp per slice, lanes over consecutive stored positions (8 rows x 4 entries at C = 8, so that the CSR reads
+// are whole sectors): column indices and S values; padding repeats the row's last column with zeros.
+__global__ void __launch_bounds__(256) k_sell_pattern(int64_t n_slices, int C, const int64_t* __restrict__ slice_ptr,
+                                                      const int32_t* __restrict__ slot_row, const int64_t* __restrict__ row_ptr,
+                                                      const int32_t* __restrict__ col_idx, const double* __restrict__ sval,
+                                                      int32_t* __restrict__ cols, double2* __restrict__ hs) {
+    const int64_t sl = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (sl >= n_slices) return;
+    const int64_t base = slice_ptr[sl];
+    const int count = (int)(slice_ptr[sl + 1] - base);
+    for (int i = threadIdx.x & 31; i < count; i += 32) {
+        const int j = i / C, r = slot_row[sl * C + i - j * C];
+        int col = 0;
+        double s = 0.0;
+        if (r >= 0) {
+            const int64_t e0 = row_ptr[r], e1 = row_ptr[r + 1];
+            if (e0 + j < e1) {
+                col = col_idx[e0 + j];
+                s = sval[e0 + j];
+            } else if (e1 > e0) {
+                col = col_idx[e1 - 1];
+            }
+        }
+        cols[base + i] = col;
+        hs[base + i] = make_double2(0.0, s);
+    }
+}
+
+// The H values in the same way, with the scaled pencil (D Hs D, D S D) in FP32 for the FP32 step entry points (FP32
+// works only on this pencil: the unscaled basis spans ~30 orders of magnitude) and as float pairs, the nearest
+// float and the nearest float to the remainder.  On the host this took 21 ms per matrix of 5.9 M entries, the copies
+// of the finished arrays included; here the copy of the CSR values is most of it.
+__global__ void __launch_bounds__(256) k_sell_values(int64_t n_slices, int C, const int64_t* __restrict__ slice_ptr,
+                                                     const int32_t* __restrict__ slot_row, const int64_t* __restrict__ row_ptr,
+                                                     const double* __restrict__ hval, double sigma0, const int32_t* __restrict__ cols,
+                                                     const double* __restrict__ dscale, double2* __restrict__ hs,
+                                                     float2* __restrict__ hs32, float4* __restrict__ hsdf) {
+    const int64_t sl = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (sl >= n_slices) return;
+    const int64_t base = slice_ptr[sl];
+    const int count = (int)(slice_ptr[sl + 1] - base);
+    for (int i = threadIdx.x & 31; i < count; i += 32) {
+        const int j = i / C, r = slot_row[sl * C + i - j * C];
+        const int64_t p = base + i;
+        const int64_t e = r >= 0 ? row_ptr[r] + j : 0;
+        if (r < 0 || e >= row_ptr[r + 1]) {
+            hs32[p] = make_float2(0.f, 0.f);
+            hsdf[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+            continue;
+        }
+        const double s = hs[p].y, h = fma(-sigma0, s, hval[e]), f = __dmul_rn(dscale[r], dscale[cols[p]]);
+        const double fh = __dmul_rn(f, h), fs = __dmul_rn(f, s);
+        const float h0 = (float)fh, s0 = (float)fs;
+        hs[p] = make_double2(h, s);
+        hs32[p] = make_float2(h0, s0);
+        hsdf[p] = make_float4(h0, (float)(fh - (double)h0), s0, (float)(fs - (double)s0));
+    }
+}
+
 int sell_build(Sell& m, int64_t n, const int64_t* row_ptr, const int32_t* col_idx,
                const double* hval, const double* sval, double sigma0) {
     const int C = m.C;
@@ -52,100 +131,43 @@ int sell_build(Sell& m, int64_t n, const int64_t* row_ptr, const int32_t* col_id
     m.stored = sptr[m.n_slices];
     m.h_slice_ptr = sptr;
     m.h_slot_row = slot_row;
-    // D = diag(S)^{-1/2} (the diagonal entry of each row of S)
-    m.h_dscale.assign(n, 1.0);
-    for (int64_t r = 0; r < n; ++r)
-        for (int64_t e = row_ptr[r]; e < row_ptr[r + 1]; ++e)
-            if (col_idx[e] == r && sval[e] > 0.0) m.h_dscale[r] = 1.0 / std::sqrt(sval[e]);
-    std::vector<int32_t> cols(m.stored, 0);
-    std::vector<double2> hs(m.stored, make_double2(0.0, 0.0));
-    m.h_entry_of_csr.assign(m.nnz, -1);
-    for (int64_t s = 0; s < m.n_slices; ++s) {
-        for (int t = 0; t < C; ++t) {
-            int32_t r = slot_row[s * C + t];
-            int64_t len = r >= 0 ? row_ptr[r + 1] - row_ptr[r] : 0;
-            int32_t pad_col = (r >= 0 && len > 0) ? col_idx[row_ptr[r + 1] - 1] : 0;
-            for (int64_t j = 0; j < slen[s]; ++j) {
-                int64_t pos = sptr[s] + j * C + t;
-                if (j < len) {
-                    int64_t e = row_ptr[r] + j;
-                    cols[pos] = col_idx[e];
-                    double hv = hval[e];
-                    double sv = sval[e];
-                    double shifted = hv - sigma0 * sv;
-                    hs[pos] = make_double2(shifted, sv);
-                    m.h_entry_of_csr[e] = pos;
-                } else {
-                    cols[pos] = pad_col;
-                }
-            }
-        }
-    }
     HBSD_TRY(m.slice_ptr.alloc(m.n_slices + 1));
     HBSD_TRY(m.slice_len.alloc(m.n_slices));
     HBSD_TRY(m.cols.alloc(m.stored));
     HBSD_TRY(m.hs.alloc(m.stored));
+    HBSD_TRY(m.hs32.alloc(m.stored));
+    HBSD_TRY(m.hsdf.alloc(m.stored));
     HBSD_TRY(m.slot_row.alloc(m.n_slots));
+    HBSD_TRY(m.row_ptr.alloc(n + 1));
+    HBSD_TRY(m.val.alloc(m.nnz));
+    HBSD_TRY(m.dscale.alloc(n));
+    HBSD_TRY(m.dinv.alloc(n));
     HBSD_CUDA(cudaMemcpy(m.slice_ptr.p, sptr.data(), sptr.size() * 8, cudaMemcpyHostToDevice));
     HBSD_CUDA(cudaMemcpy(m.slice_len.p, slen.data(), slen.size() * 4, cudaMemcpyHostToDevice));
-    HBSD_CUDA(cudaMemcpy(m.cols.p, cols.data(), cols.size() * 4, cudaMemcpyHostToDevice));
-    HBSD_CUDA(cudaMemcpy(m.hs.p, hs.data(), hs.size() * sizeof(double2), cudaMemcpyHostToDevice));
     HBSD_CUDA(cudaMemcpy(m.slot_row.p, slot_row.data(), slot_row.size() * 4, cudaMemcpyHostToDevice));
-    m.h_cols = cols;
-    HBSD_TRY(m.dscale.alloc(n));
-    HBSD_CUDA(cudaMemcpy(m.dscale.p, m.h_dscale.data(), n * 8, cudaMemcpyHostToDevice));
-    {
-        std::vector<double> dinv(n);
-        for (int64_t i = 0; i < n; ++i) dinv[i] = 1.0 / m.h_dscale[i];
-        HBSD_TRY(m.dinv.alloc(n));
-        HBSD_CUDA(cudaMemcpy(m.dinv.p, dinv.data(), n * 8, cudaMemcpyHostToDevice));
-    }
-    HBSD_TRY(m.hs32.alloc(m.stored));
-    return sell_fill_fp32(m, hs.data(), cols.data(), slot_row.data());
+    HBSD_CUDA(cudaMemcpy(m.row_ptr.p, row_ptr, (n + 1) * 8, cudaMemcpyHostToDevice));
+    int32_t* ci = reinterpret_cast<int32_t*>(m.hsdf.p);   // until the values are filled in
+    HBSD_CUDA(cudaMemcpy(ci, col_idx, m.nnz * 4, cudaMemcpyHostToDevice));
+    HBSD_CUDA(cudaMemcpy(m.val.p, sval, m.nnz * 8, cudaMemcpyHostToDevice));
+    const int gs = ceil_div(m.n_slices, 8);
+    k_sell_dscale<<<ceil_div(n, 8), 256>>>(n, m.row_ptr.p, ci, m.val.p, m.dscale.p, m.dinv.p);
+    HBSD_LAUNCHED((Session*)nullptr);
+    k_sell_pattern<<<gs, 256>>>(m.n_slices, m.C, m.slice_ptr.p, m.slot_row.p, m.row_ptr.p, ci, m.val.p, m.cols.p, m.hs.p);
+    HBSD_LAUNCHED((Session*)nullptr);
+    m.h_dscale.resize(n);
+    HBSD_CUDA(cudaMemcpy(m.h_dscale.data(), m.dscale.p, n * 8, cudaMemcpyDeviceToHost));
+    return sell_update_h(m, hval, sigma0);
 }
 
-// FP32 values of the diagonally scaled pencil (D Hs D, D S D), D = diag(S)^{-1/2}, for the FP32
-// step entry points: FP32 works only on this pencil, because the unscaled basis spans ~30 orders
-// of magnitude.
-int sell_fill_fp32(Sell& m, const double2* hs, const int32_t* cols, const int32_t* slot_row) {
-    std::vector<float2> hs32(m.stored, make_float2(0.f, 0.f));
-    std::vector<float4> hsdf(m.stored, make_float4(0.f, 0.f, 0.f, 0.f));
-    // double-float pair of a double: the nearest float, then the nearest float to the remainder
-    auto pair = [](double v, float& hi, float& lo) {
-        hi = (float)v;
-        lo = (float)(v - (double)hi);
-    };
-    for (int64_t sl = 0; sl < m.n_slices; ++sl) {
-        const int64_t len = (m.h_slice_ptr[sl + 1] - m.h_slice_ptr[sl]) / m.C;
-        for (int t = 0; t < m.C; ++t) {
-            const int32_t r = slot_row[sl * m.C + t];
-            if (r < 0) continue;
-            for (int64_t j = 0; j < len; ++j) {
-                const int64_t pos = m.h_slice_ptr[sl] + j * m.C + t;
-                const double f = m.h_dscale[r] * m.h_dscale[cols[pos]];
-                hs32[pos] = make_float2((float)(f * hs[pos].x), (float)(f * hs[pos].y));
-                float a, b, c, d;
-                pair(f * hs[pos].x, a, b);
-                pair(f * hs[pos].y, c, d);
-                hsdf[pos] = make_float4(a, b, c, d);
-            }
-        }
-    }
-    HBSD_CUDA(cudaMemcpy(m.hs32.p, hs32.data(), hs32.size() * sizeof(float2), cudaMemcpyHostToDevice));
-    HBSD_TRY(m.hsdf.alloc(m.stored));
-    HBSD_CUDA(cudaMemcpy(m.hsdf.p, hsdf.data(), hsdf.size() * sizeof(float4), cudaMemcpyHostToDevice));
+// The stored H values from CSR values in host memory; S, the pattern and the scaling stay.  On the legacy default
+// stream and complete on return, as the copies are.
+int sell_update_h(Sell& m, const double* hval, double sigma0) {
+    HBSD_CUDA(cudaMemcpy(m.val.p, hval, m.nnz * 8, cudaMemcpyHostToDevice));
+    k_sell_values<<<ceil_div(m.n_slices, 8), 256>>>(m.n_slices, m.C, m.slice_ptr.p, m.slot_row.p, m.row_ptr.p, m.val.p, sigma0,
+                                                    m.cols.p, m.dscale.p, m.hs.p, m.hs32.p, m.hsdf.p);
+    HBSD_LAUNCHED((Session*)nullptr);
+    HBSD_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
     return 0;
-}
-
-int sell_update_h(Sell& m, const double* hval, const double* sval, double sigma0) {
-    std::vector<double2> hs(m.stored, make_double2(0.0, 0.0));
-    for (int64_t e = 0; e < m.nnz; ++e) {
-        int64_t pos = m.h_entry_of_csr[e];
-        double shifted = hval[e] - sigma0 * sval[e];
-        hs[pos] = make_double2(shifted, sval[e]);
-    }
-    HBSD_CUDA(cudaMemcpy(m.hs.p, hs.data(), hs.size() * sizeof(double2), cudaMemcpyHostToDevice));
-    return sell_fill_fp32(m, hs.data(), m.h_cols.data(), m.h_slot_row.data());
 }
 
 // ---- kernels ------------------------------------------------------------------------

@@ -775,7 +775,6 @@ int hbsd_create(const hbsd_csr* H, const hbsd_csr* Sm, const hbsd_local_blocks* 
         }
         int rc = sell_build(S->A, S->n, row_ptr, col_idx, hval, sval, S->sigma0);
         if (rc < 0) { hbsd_destroy(h); return rc; }
-        S->h_sval.assign(sval, sval + S->nnz);
         std::vector<double> aval(S->nnz);
         for (int64_t e = 0; e < S->nnz; ++e) aval[e] = hval[e] - opt->sigma_bar * sval[e];
         if (opt->precond != HBSD_PRECOND_LOCAL) {   // the local-only mode has no global step
@@ -794,9 +793,9 @@ int hbsd_update_H(hbsd_handle* h, const double* H_val) {
         if (h->s.cplx) {   // 2 nnz interleaved (re, im) values of the complex pattern
             std::vector<double> v2;
             complex_realify_values(h->s.n_c, h->s.c_row_ptr.data(), H_val, v2);
-            return sell_update_h(h->s.A, v2.data(), h->s.h_sval.data(), h->s.sigma0);
+            return sell_update_h(h->s.A, v2.data(), h->s.sigma0);
         }
-        return sell_update_h(h->s.A, H_val, h->s.h_sval.data(), h->s.sigma0);
+        return sell_update_h(h->s.A, H_val, h->s.sigma0);
     });
 }
 
