@@ -348,7 +348,7 @@ struct Session {
     DBuf<double> mr_d;
     DBuf<double> mr_red;        // per-block partial sums of the fused MINRES kernel
     DBuf<float> mr_v32;         // D^-1 v in FP32 for the FP32 operator products of MINRES
-    DBuf<float2> x2;            // D^-1 X in double-float for spmm_pair_df64
+    DBuf<float4> x2;            // D^-1 X in double-float, per column pair, for spmm_pair_df64
     DBuf<int> mr_any, mr_steps; // grid barrier + error flag; per-column step counts
     DBuf<unsigned long long> mr_stamps;   // MINRES phase times when tracing
     DBuf<int64_t> mr_blk;       // per-block SELL slot ranges of the fused MINRES kernel

@@ -210,70 +210,65 @@ __device__ __forceinline__ void ldhs(const float2* hs, int64_t e, float& h, floa
     h = t.x; s = t.y;
 }
 
-// MODE 0: pair (HX, SX).  MODE 1: shifted, Y = HX - e_j SX.
-template <class T, int CH, int MODE>
+// MODE 0: pair (HX, SX).  MODE 1: shifted, Y = HX - e_j SX.  A row is worked by 1 << parts_log2 groups of
+// 1 << lpr_log2 lanes of one warp, a lane one vector, a group every 1 << parts_log2-th entry; blockIdx.y counts
+// passes of (1 << lpr_log2) vectors.
+// Bound by the FP64 pipe (a multiply-add of a warp takes it 64 clocks, idle lanes included) and on small
+// matrices by the chain of index and X loads.  One vector per lane: with up to four, 85 columns of the 32^3
+// problem (47,620 rows, 124 entries each) took 1,042 us instead of 988, 64 columns of the 16^3 one 72 instead of 52.
+template <class T, int MODE, bool SPLIT>
 __global__ void __launch_bounds__(256) k_spmm(
     const int64_t* __restrict__ slice_ptr, const int32_t* __restrict__ slice_len,
     const int32_t* __restrict__ cols, const typename VecOf<T>::P* __restrict__ hs,
     const int32_t* __restrict__ slot_row, int64_t n_slots, int C, const T* __restrict__ X,
-    int64_t ldx, int k, int lpr_log2, T* __restrict__ Y0, int64_t ld0, T* __restrict__ Y1,
-    int64_t ld1, const T* __restrict__ shifts) {
+    int64_t ldx, int k, int lpr_log2, int parts_log2, T* __restrict__ Y0, int64_t ld0,
+    T* __restrict__ Y1, int64_t ld1, const T* __restrict__ shifts) {
     constexpr int VW = VecOf<T>::W;
-    const int lpr = 1 << lpr_log2;
-    const int lane = threadIdx.x & (lpr - 1);
-    const int64_t slot = (int64_t)blockIdx.x * (blockDim.x >> lpr_log2) + (threadIdx.x >> lpr_log2);
-    if (slot >= n_slots) return;
-    const int64_t sl = slot / C;
-    const int t = (int)(slot - sl * C);
-    const int64_t base = slice_ptr[sl] + t;
-    const int len = slice_len[sl];
-    T ah[CH][VW], as[CH][VW];
+    const int lpr = 1 << lpr_log2, parts = SPLIT ? 1 << parts_log2 : 1, row_log2 = lpr_log2 + (SPLIT ? parts_log2 : 0);
+    const int lane = threadIdx.x & (lpr - 1), part = SPLIT ? (threadIdx.x >> lpr_log2) & (parts - 1) : 0;
+    const int64_t slot = (int64_t)blockIdx.x * (blockDim.x >> row_log2) + (threadIdx.x >> row_log2);
+    const int cc = VW * ((int)blockIdx.y * lpr + lane);
+    const bool on = slot < n_slots && cc < k;
+    const int64_t sl = on ? slot / C : 0;
+    const int64_t base = on ? slice_ptr[sl] + (slot - sl * C) : 0;
+    const int len = on ? slice_len[sl] : 0;
+    T ah[VW], as[VW];
 #pragma unroll
-    for (int c = 0; c < CH; ++c)
-#pragma unroll
-        for (int v = 0; v < VW; ++v) { ah[c][v] = T(0); as[c][v] = T(0); }
-    int col0[CH];
-#pragma unroll
-    for (int c = 0; c < CH; ++c) col0[c] = VW * (lane + c * lpr);
+    for (int v = 0; v < VW; ++v) { ah[v] = T(0); as[v] = T(0); }
 #pragma unroll 4
-    for (int j = 0; j < len; ++j) {
+    for (int j = part; j < len; j += parts) {
         const int64_t e = base + (int64_t)j * C;
         const int cj = __ldg(cols + e);
-        T hv, sv;
+        T hv, sv, x[VW];
         ldhs(hs, e, hv, sv);
-        const T* xr = X + (int64_t)cj * ldx;
+        vload<T>(X + (int64_t)cj * ldx + cc, x);
 #pragma unroll
-        for (int c = 0; c < CH; ++c) {
-            if (col0[c] < k) {
-                T x[VW];
-                vload<T>(xr + col0[c], x);
-#pragma unroll
-                for (int v = 0; v < VW; ++v) {
-                    ah[c][v] = fma(hv, x[v], ah[c][v]);
-                    as[c][v] = fma(sv, x[v], as[c][v]);
-                }
-            }
+        for (int v = 0; v < VW; ++v) {
+            ah[v] = fma(hv, x[v], ah[v]);
+            as[v] = fma(sv, x[v], as[v]);
         }
     }
-    const int row = slot_row[slot];
-    if (row < 0) return;
+    for (int o = lpr; SPLIT && o < (1 << row_log2); o <<= 1) {
 #pragma unroll
-    for (int c = 0; c < CH; ++c) {
-        const int cc = col0[c];
-        if (cc >= k) continue;
-        const int valid = min(VW, k - cc);
-        if (MODE == 0) {
-            vstore<T>(Y0 + (int64_t)row * ld0 + cc, ah[c], valid);
-            vstore<T>(Y1 + (int64_t)row * ld1 + cc, as[c], valid);
-        } else {
-            T y[VW];
-#pragma unroll
-            for (int v = 0; v < VW; ++v) {
-                T ev = (cc + v < k) ? shifts[cc + v] : T(0);
-                y[v] = ah[c][v] - ev * as[c][v];
-            }
-            vstore<T>(Y0 + (int64_t)row * ld0 + cc, y, valid);
+        for (int v = 0; v < VW; ++v) {
+            ah[v] += __shfl_xor_sync(0xffffffffu, ah[v], o);
+            as[v] += __shfl_xor_sync(0xffffffffu, as[v], o);
         }
+    }
+    const int row = on && part == 0 ? slot_row[slot] : -1;
+    if (row < 0) return;
+    const int valid = min(VW, k - cc);
+    if (MODE == 0) {
+        vstore<T>(Y0 + (int64_t)row * ld0 + cc, ah, valid);
+        vstore<T>(Y1 + (int64_t)row * ld1 + cc, as, valid);
+    } else {
+        T y[VW];
+#pragma unroll
+        for (int v = 0; v < VW; ++v) {
+            T ev = (cc + v < k) ? shifts[cc + v] : T(0);
+            y[v] = ah[v] - ev * as[v];
+        }
+        vstore<T>(Y0 + (int64_t)row * ld0 + cc, y, valid);
     }
 }
 
@@ -284,10 +279,24 @@ const double2* values_of<double>(const Sell& m) { return m.hs.p; }
 template <>
 const float2* values_of<float>(const Sell& m) { return m.hs32.p; }
 
+constexpr int64_t SPMM_SPLIT_ROWS = 8192;   // rows x groups up to which FP64 rows are split
+
 // most lanes per row: the autotuner's choice for the session, else 32
 static int spmm_lanes(const Session* s) {
     const int v = s ? s->tune_spmm_lpr : 0;
     return (v == 4 || v == 8 || v == 16) ? v : 32;
+}
+
+static int ceil_log2(int v) {
+    int g = 0;
+    while ((1 << g) < v) ++g;
+    return g;
+}
+
+// Small CTAs where large ones would leave SMs idle: 19 columns of the 16^3 problem 31 us with 64 threads, 39 with 256
+// (FP32, bound by latencies alone, 25 and 21)
+static int spmm_threads(int64_t n_slots, int row_log2, int passes) {
+    return ceil_div(n_slots, 256 >> row_log2) * passes < 8 * 152 ? 64 : 256;
 }
 
 template <class T, int MODE>
@@ -297,64 +306,72 @@ static int spmm_launch(Session* s, const Sell& m, const T* X, int64_t ldx, int k
     if (k <= 0) return 0;
     if ((ldx % VW) || (ld0 % VW) || (MODE == 0 && (ld1 % VW)))
         return fail(HBSD_ERR_ARG, "spmm: leading dimensions must be multiples of the vector width");
-    // columns are processed in passes of at most lpr_max lanes * VW * 4 chunks; each row gets the
-    // smallest power-of-two number of lanes (up to lpr_max, the autotuner's choice) that covers
-    // its vectors in at most 4 chunks
-    const int lpr_max = spmm_lanes(s);
-    const int pass_cols = lpr_max * VW * 4;
-    for (int c0 = 0; c0 < k; c0 += pass_cols) {
-        const int kk = std::min(pass_cols, k - c0);
-        int vecs = ceil_div(kk, VW);
-        int lpr = 1, lg = 0;
-        while (lpr < vecs && lpr < lpr_max) { lpr <<= 1; ++lg; }
-        const int ch = ceil_div(vecs, lpr);
-        const int rows_per_cta = 256 / lpr;
-        const int grid = ceil_div(m.n_slots, rows_per_cta);
-        const T* Xc = X + c0;
-        T* Y0c = Y0 + c0;
-        T* Y1c = Y1 ? Y1 + c0 : nullptr;
-        const T* ec = e ? e + c0 : nullptr;
-#define HBSD_SPMM_CASE(CHV)                                                                    \
-    case CHV:                                                                                  \
-        k_spmm<T, CHV, MODE><<<grid, 256, 0, st>>>(m.slice_ptr.p, m.slice_len.p, m.cols.p,      \
-                                                   values_of<T>(m), m.slot_row.p, m.n_slots,   \
-                                                   m.C, Xc, ldx, kk, lg, Y0c, ld0, Y1c, ld1, ec); \
-        break;
-        switch (ch) {
-            HBSD_SPMM_CASE(1)
-            HBSD_SPMM_CASE(2)
-            HBSD_SPMM_CASE(3)
-            HBSD_SPMM_CASE(4)
-            default:
-                return fail(HBSD_ERR_ARG, "spmm: internal chunking error");
-        }
-#undef HBSD_SPMM_CASE
-        HBSD_LAUNCHED(s);
+    // FP64 rows of a small matrix are split over 2 to 8 groups of lanes: 19 columns of the 8^3 problem (646 rows)
+    // took 28.7 us on one group, its 80 entries one after another, and 11 us on 8.  By the matrix alone, so that a
+    // column's sums do not depend on the block it is in; from 4,797 rows on (16^3) the pipe is busy without.
+    int parts_log2 = 0;
+    if (sizeof(T) == 8)
+        while (parts_log2 < 3 && (m.n_slots << (parts_log2 + 1)) <= SPMM_SPLIT_ROWS) ++parts_log2;
+    // lanes per row (4 or more, up to the session's limit) with the fewest idle over all passes, each pass worth half
+    // a lane: 24 columns of the 32^3 problem 307 us in 3 passes of 4 lanes, 371 in one of 16; 85 columns 988 in 3
+    // of 16, 1,335 in one of 32 with a second vector on every lane
+    const int vecs = ceil_div(k, VW), lmax = std::min(ceil_log2(spmm_lanes(s)), 5 - parts_log2);
+    int lg = std::min(lmax, ceil_log2(std::min(vecs, 4))), best = 0x7FFFFFFF;
+    for (int g = lg; g <= lmax; ++g) {
+        const int cost = ceil_div(vecs, 1 << g) * ((2 << g) + 1);
+        if (cost <= best) { best = cost; lg = g; }
     }
+    const int threads = sizeof(T) == 8 ? spmm_threads(m.n_slots, lg + parts_log2, ceil_div(vecs, 1 << lg)) : 256;
+    const dim3 grid(ceil_div(m.n_slots, threads >> (lg + parts_log2)), ceil_div(vecs, 1 << lg));
+    const auto kern = sizeof(T) == 8 && parts_log2 ? k_spmm<T, MODE, sizeof(T) == 8> : k_spmm<T, MODE, false>;
+    kern<<<grid, threads, 0, st>>>(m.slice_ptr.p, m.slice_len.p, m.cols.p, values_of<T>(m), m.slot_row.p, m.n_slots, m.C,
+                                   X, ldx, k, lg, parts_log2, Y0, ld0, Y1, ld1, e);
+    HBSD_LAUNCHED(s);
     return 0;
 }
 
 // ---- double-float SpMM on the scaled pencil (mixed form) ------------------------------------------
-// X2 = D^-1 X as double-float pairs (the FP64 scaling, then split_d's exact bit split)
+// X2 = D^-1 X as double-float pairs (the FP64 scaling, then split_d's exact bit split), per two columns the two high
+// parts and the two low parts: the packed operands of k_spmm_df64
 __global__ void k_split_scaled(const double* __restrict__ X, int64_t ldx, int k, int64_t n,
-                               const double* __restrict__ dinv, float2* __restrict__ X2, int64_t ld2) {
-    const int64_t total = n * k;
+                               const double* __restrict__ dinv, float4* __restrict__ X2, int pairs) {
+    const int64_t total = n * pairs;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = t / k;
-        const int j = (int)(t - i * k);
-        X2[i * ld2 + j] = df::split_d(X[i * ldx + j] * dinv[i]);
+        const int64_t i = t / pairs;
+        const int j = 2 * (int)(t - i * pairs);
+        const double d = dinv[i];
+        const float2 a = df::split_d(X[i * ldx + j] * d);
+        const float2 b = j + 1 < k ? df::split_d(X[i * ldx + j + 1] * d) : make_float2(0.f, 0.f);
+        X2[t] = make_float4(a.x, b.x, a.y, b.y);
     }
 }
 
-// Pair mode of k_spmm in double-float: per stored entry the (hi, lo) of D Hs D and of D S D, per
-// column pair one float4 of X2; sums by df::dfma, renormalised every 8 entries; the row result is
+// Pair mode of k_spmm in double-float: per stored entry the (hi, lo) of D Hs D and of D S D, per column pair one
+// float4 of X2.  Sums by df::dfma's steps on packed column pairs, renormalised every 8 entries; the row result is
 // scaled back by D^-1 in FP64.
+// Bound by the FP32 pipe: 24 packed instructions (48 pipe cycles of a warp) per entry and column pair.  Without the
+// loads an entry ahead, and with scalar instructions, 85 columns of the 32^3 problem took 583 us (now 404); packed
+// without them 517.
+// nax = -ax; the product is kept negated, which saves negating it for its rounding error
+__device__ __forceinline__ void dfma_packed(df::f32x2 ax, df::f32x2 nax, df::f32x2 ay, df::f32x2 bx, df::f32x2 by, df::f32x2& sh,
+                                            df::f32x2& sl, df::f32x2 nz) {
+    const df::f32x2 np = df::fma2(nax, bx, nz);   // minus the rounded product (df64.h: why not a multiplication)
+    const df::f32x2 t = df::sub2(sh, np);
+    const df::f32x2 bp = df::sub2(t, sh);
+    df::f32x2 e = df::fma2(ax, bx, np);
+    e = df::fma2(ax, by, e);
+    e = df::fma2(ay, bx, e);
+    const df::f32x2 err = df::sub2(df::sub2(sh, df::sub2(t, bp)), df::add2(np, bp));
+    sl = df::add2(sl, df::add2(err, e));
+    sh = t;
+}
+
 template <int CH>
-__global__ void __launch_bounds__(256) k_spmm_df64(
+__global__ void __launch_bounds__(256, CH <= 2 ? 3 : 2) k_spmm_df64(
     const int64_t* __restrict__ slice_ptr, const int32_t* __restrict__ slice_len, const int32_t* __restrict__ cols,
     const float4* __restrict__ hsdf, const int32_t* __restrict__ slot_row, int64_t n_slots, int C,
-    const float2* __restrict__ X2, int64_t ld2, int k, int lpr_log2, const double* __restrict__ dinv,
-    double* __restrict__ Y0, int64_t ld0, double* __restrict__ Y1, int64_t ld1) {
+    const float4* __restrict__ X2, int pairs, int k, int lpr_log2, const double* __restrict__ dinv,
+    double* __restrict__ Y0, int64_t ld0, double* __restrict__ Y1, int64_t ld1, df::f32x2 nz) {
     const int lpr = 1 << lpr_log2;
     const int lane = threadIdx.x & (lpr - 1);
     const int64_t slot = (int64_t)blockIdx.x * (blockDim.x >> lpr_log2) + (threadIdx.x >> lpr_log2);
@@ -363,39 +380,50 @@ __global__ void __launch_bounds__(256) k_spmm_df64(
     const int t = (int)(slot - sl * C);
     const int64_t base = slice_ptr[sl] + t;
     const int len = slice_len[sl];
-    float ah[CH][2][2], as[CH][2][2];   // [chunk][column of the pair][hi, lo]
+    const int v0 = (int)blockIdx.y * lpr * CH + lane;
+    df::f32x2 ah[CH][2], as[CH][2];   // [chunk][hi, lo] of two columns
 #pragma unroll
-    for (int c = 0; c < CH; ++c)
+    for (int c = 0; c < CH; ++c) ah[c][0] = ah[c][1] = as[c][0] = as[c][1] = 0;
+    // entry j + 1's values and X vectors are loaded before entry j's sums, entry j + 2's index with them
+    const float4* xv[CH];   // idle lanes repeat the last vector
 #pragma unroll
-        for (int v = 0; v < 2; ++v) { ah[c][v][0] = ah[c][v][1] = as[c][v][0] = as[c][v][1] = 0.f; }
-    int col0[CH];
+    for (int c = 0; c < CH; ++c) xv[c] = X2 + min(v0 + c * lpr, pairs - 1);
+    float4 hn = make_float4(0.f, 0.f, 0.f, 0.f), xn[CH];
+    int64_t e = base;
+    int cn = 0;
+    if (len > 0) {
+        hn = __ldg(hsdf + e);
+        cn = __ldg(cols + e);
 #pragma unroll
-    for (int c = 0; c < CH; ++c) col0[c] = 2 * (lane + c * lpr);
+        for (int c = 0; c < CH; ++c) xn[c] = __ldg(xv[c] + (int64_t)cn * pairs);
+        if (len > 1) cn = __ldg(cols + e + C);
+    }
     for (int j = 0; j < len; ++j) {
-        const int64_t e = base + (int64_t)j * C;
-        const int cj = __ldg(cols + e);
-        const float4 hv = __ldg(hsdf + e);
-        const float2 h2 = make_float2(hv.x, hv.y), s2 = make_float2(hv.z, hv.w);
-        const float2* xr = X2 + (int64_t)cj * ld2;
+        const float4 hv = hn;
+        float4 x[CH];
+#pragma unroll
+        for (int c = 0; c < CH; ++c) x[c] = xn[c];
+        e += C;
+        if (j + 1 < len) {
+            hn = __ldg(hsdf + e);
+#pragma unroll
+            for (int c = 0; c < CH; ++c) xn[c] = __ldg(xv[c] + (int64_t)cn * pairs);
+            if (j + 2 < len) cn = __ldg(cols + e + C);
+        }
+        const df::f32x2 hx = df::pack2(hv.x, hv.x), hnx = df::pack2(-hv.x, -hv.x), hy = df::pack2(hv.y, hv.y);
+        const df::f32x2 sx = df::pack2(hv.z, hv.z), snx = df::pack2(-hv.z, -hv.z), sy = df::pack2(hv.w, hv.w);
 #pragma unroll
         for (int c = 0; c < CH; ++c) {
-            if (col0[c] < k) {
-                const float4 x = __ldg(reinterpret_cast<const float4*>(xr + col0[c]));
-                const float2 x0 = make_float2(x.x, x.y), x1 = make_float2(x.z, x.w);
-                df::dfma(h2, x0, ah[c][0][0], ah[c][0][1]);
-                df::dfma(s2, x0, as[c][0][0], as[c][0][1]);
-                df::dfma(h2, x1, ah[c][1][0], ah[c][1][1]);
-                df::dfma(s2, x1, as[c][1][0], as[c][1][1]);
-            }
+            const df::f32x2 bx = df::pack2(x[c].x, x[c].y), by = df::pack2(x[c].z, x[c].w);
+            dfma_packed(hx, hnx, hy, bx, by, ah[c][0], ah[c][1], nz);
+            dfma_packed(sx, snx, sy, bx, by, as[c][0], as[c][1], nz);
         }
         if ((j & 7) == 7) {
 #pragma unroll
-            for (int c = 0; c < CH; ++c)
-#pragma unroll
-                for (int v = 0; v < 2; ++v) {
-                    df::renorm(ah[c][v][0], ah[c][v][1]);
-                    df::renorm(as[c][v][0], as[c][v][1]);
-                }
+            for (int c = 0; c < CH; ++c) {
+                df::renorm2(ah[c][0], ah[c][1]);
+                df::renorm2(as[c][0], as[c][1]);
+            }
         }
     }
     const int row = slot_row[slot];
@@ -403,13 +431,18 @@ __global__ void __launch_bounds__(256) k_spmm_df64(
     const double di = dinv[row];
 #pragma unroll
     for (int c = 0; c < CH; ++c) {
-        const int cc = col0[c];
+        const int cc = 2 * (v0 + c * lpr);
         if (cc >= k) continue;
-#pragma unroll
-        for (int v = 0; v < 2; ++v) {
-            if (cc + v >= k) break;
-            Y0[(int64_t)row * ld0 + cc + v] = df::to_d(ah[c][v][0], ah[c][v][1]) * di;
-            Y1[(int64_t)row * ld1 + cc + v] = df::to_d(as[c][v][0], as[c][v][1]) * di;
+        float h0, h1, l0, l1, s0, s1, m0, m1;
+        df::unpack2(ah[c][0], h0, h1);
+        df::unpack2(ah[c][1], l0, l1);
+        df::unpack2(as[c][0], s0, s1);
+        df::unpack2(as[c][1], m0, m1);
+        Y0[(int64_t)row * ld0 + cc] = df::to_d(h0, l0) * di;
+        Y1[(int64_t)row * ld1 + cc] = df::to_d(s0, m0) * di;
+        if (cc + 1 < k) {
+            Y0[(int64_t)row * ld0 + cc + 1] = df::to_d(h1, l1) * di;
+            Y1[(int64_t)row * ld1 + cc + 1] = df::to_d(s1, m1) * di;
         }
     }
 }
@@ -417,36 +450,41 @@ __global__ void __launch_bounds__(256) k_spmm_df64(
 int spmm_pair_df64(Session* s, const Sell& m, const double* X, int64_t ldx, int k, double* HX, int64_t ldhx,
                    double* SX, int64_t ldsx, cudaStream_t st) {
     if (k <= 0) return 0;
-    const int64_t ld2 = round_up(k, 2);
-    HBSD_TRY(s->x2.alloc((size_t)m.n * ld2));
+    const int pairs = ceil_div(k, 2);
+    HBSD_TRY(s->x2.alloc((size_t)m.n * pairs));
     {
-        const int64_t total = m.n * k;
-        const int g = (int)std::min<int64_t>(std::max<int64_t>(1, (total + 255) / 256), 8192);
-        k_split_scaled<<<g, 256, 0, st>>>(X, ldx, k, m.n, m.dinv.p, s->x2.p, ld2);
+        const int g = (int)std::min<int64_t>(ceil_div(m.n * pairs, 256), 8192);
+        k_split_scaled<<<g, 256, 0, st>>>(X, ldx, k, m.n, m.dinv.p, s->x2.p, pairs);
         HBSD_LAUNCHED(s);
     }
-    const int lpr_max = spmm_lanes(s);
-    const int pass_cols = lpr_max * 2 * 4;
-    for (int c0 = 0; c0 < k; c0 += pass_cols) {
-        const int kk = std::min(pass_cols, k - c0);
-        const int vecs = ceil_div(kk, 2);
-        int lpr = 1, lg = 0;
-        while (lpr < vecs && lpr < lpr_max) { lpr <<= 1; ++lg; }
-        const int ch = ceil_div(vecs, lpr);
-        const int rows_per_cta = 256 / lpr;
-        const int grid = ceil_div(m.n_slots, rows_per_cta);
-#define HBSD_SPMM_DF_CASE(CHV)                                                                                 case CHV:                                                                                                      k_spmm_df64<CHV><<<grid, 256, 0, st>>>(m.slice_ptr.p, m.slice_len.p, m.cols.p, m.hsdf.p, m.slot_row.p,                                                  m.n_slots, m.C, s->x2.p + c0, ld2, kk, lg, m.dinv.p, HX + c0, ldhx,                                                SX + c0, ldsx);                                                     break;
-        switch (ch) {
-            HBSD_SPMM_DF_CASE(1)
-            HBSD_SPMM_DF_CASE(2)
-            HBSD_SPMM_DF_CASE(3)
-            HBSD_SPMM_DF_CASE(4)
-            default:
-                return fail(HBSD_ERR_ARG, "spmm_df64: internal chunking error");
-        }
+    // 4 lanes per row and up to 4 column pairs per lane, in as many passes as that takes (each worth one more pair):
+    // 85 columns of the 32^3 problem 404 us in 3 passes of 4 x 4, 441 in one of 16 x 3, 552 in one of 16 x 2 and more;
+    // 64 columns 279 us against 311 (16 x 2).  Few rows keep to 2 pairs: 64 columns of the 16^3 problem (4,796
+    // rows) 33 us in 4 passes, 37 in 2
+    const int lg = std::min(2, ceil_log2(pairs)), cmax = m.n_slots >= 152 * 128 ? 4 : 2;
+    int ch = 1, best = 0x7FFFFFFF;
+    for (int c = 1; c <= cmax; ++c) {
+        const int cost = ceil_div(pairs, c << lg) * (c + 1);
+        if (cost <= best) { best = cost; ch = c; }
+    }
+    const int threads = spmm_threads(m.n_slots, lg, ceil_div(pairs, ch << lg));
+    const dim3 grid(ceil_div(m.n_slots, threads >> lg), ceil_div(pairs, ch << lg));
+#define HBSD_SPMM_DF_CASE(CHV)                                                                                      \
+    case CHV:                                                                                                       \
+        k_spmm_df64<CHV><<<grid, threads, 0, st>>>(m.slice_ptr.p, m.slice_len.p, m.cols.p, m.hsdf.p, m.slot_row.p,      \
+                                               m.n_slots, m.C, s->x2.p, pairs, k, lg, m.dinv.p, HX, ldhx, SX, ldsx, \
+                                               df::NEG_ZERO2);                                                      \
+        break;
+    switch (ch) {
+        HBSD_SPMM_DF_CASE(1)
+        HBSD_SPMM_DF_CASE(2)
+        HBSD_SPMM_DF_CASE(3)
+        HBSD_SPMM_DF_CASE(4)
+        default:
+            return fail(HBSD_ERR_ARG, "spmm_df64: internal chunking error");
+    }
 #undef HBSD_SPMM_DF_CASE
-        HBSD_LAUNCHED(s);
-    }
+    HBSD_LAUNCHED(s);
     return nl_apply_add<double>(s, X, ldx, k, HX, ldhx, st);
 }
 
