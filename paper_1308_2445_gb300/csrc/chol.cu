@@ -442,12 +442,17 @@ struct SolveItem {
     int64_t part_row;   // first partial row of this supernode's split block (level-relative)
 };
 
-template <class T, int RC, bool BWD>
+// 64 rows x 16 columns per CTA, rows in groups of 16 (one per thread and group; groups beyond the block are not
+// computed).  Bound by the FP64 pipe (64 clocks for a warp's multiply-add), so the panels are re-read per 16 columns
+// without cost, and wide blocks only idled lanes and left SMs without a CTA: with 64 columns per CTA and 32
+// right-hand sides, a solve with the 16^3 problem's factor took 1,704 us, now 621 (16 of them: 555, now 538).
+template <class T, bool BWD>
 __global__ void __launch_bounds__(256) k_solve_gemm(const SnDev* __restrict__ sn, const SolveItem* __restrict__ items,
                                                     const T* __restrict__ G, const int64_t* __restrict__ srows,
                                                     int p, T* __restrict__ fv, int64_t ldf,
                                                     T* __restrict__ Y, T* __restrict__ X, int64_t ldx,
                                                     T* __restrict__ part) {
+    constexpr int RC = 16;   // columns
     __shared__ T Gt[32][65];
     __shared__ T Zt[32][RC + 1];
     const SolveItem it = items[blockIdx.x];
@@ -456,13 +461,17 @@ __global__ void __launch_bounds__(256) k_solve_gemm(const SnDev* __restrict__ sn
     const int j0 = blockIdx.y * RC;
     const int kc = min(RC, p - j0);
     const int nout = BWD ? s.ns : nf;
-    constexpr int CPT = RC / 16;         // columns per thread
     const int tr = threadIdx.x % 16, tc = threadIdx.x / 16;
-    T acc[4][CPT];
+    const int groups = min(4, (nout - it.t0 + 15) / 16);
+    T acc[4] = {T(0), T(0), T(0), T(0)};
+    auto sum = [&](auto groups_c, int qn) {
+#pragma unroll 8
+        for (int q = 0; q < qn; ++q) {
+            const T b = Zt[q][tc];
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < CPT; ++v) acc[u][v] = T(0);
+            for (int u = 0; u < decltype(groups_c)::value; ++u) acc[u] = fma(Gt[q][tr + 16 * u], b, acc[u]);
+        }
+    };
     const T* Gs = G + s.L_off;
     for (int kk = it.k0; kk < it.k1; kk += 32) {
         if (!BWD) {
@@ -492,17 +501,12 @@ __global__ void __launch_bounds__(256) k_solve_gemm(const SnDev* __restrict__ sn
             }
         }
         __syncthreads();
-#pragma unroll 8
-        for (int q = 0; q < 32; ++q) {
-            T a[4], b[CPT];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) a[u] = Gt[q][tr + 16 * u];
-#pragma unroll
-            for (int v = 0; v < CPT; ++v) b[v] = Zt[q][tc + 16 * v];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < CPT; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
+        const int qn = min(32, it.k1 - kk);
+        switch (groups) {
+            case 1: sum(std::integral_constant<int, 1>{}, qn); break;
+            case 2: sum(std::integral_constant<int, 2>{}, qn); break;
+            case 3: sum(std::integral_constant<int, 3>{}, qn); break;
+            default: sum(std::integral_constant<int, 4>{}, qn);
         }
         __syncthreads();
     }
@@ -510,19 +514,16 @@ __global__ void __launch_bounds__(256) k_solve_gemm(const SnDev* __restrict__ sn
     for (int u = 0; u < 4; ++u) {
         const int o = it.t0 + tr + 16 * u;
         if (o >= nout) continue;
-#pragma unroll
-        for (int v = 0; v < CPT; ++v) {
-            const int j = tc + 16 * v;
-            if (j >= kc) continue;
-            if (it.nsplit > 1) {
-                part[(it.part_row + (int64_t)it.split * nout + o) * ldf + j0 + j] = acc[u][v];
-            } else if (BWD) {
-                X[(s.first + o) * ldx + j0 + j] = acc[u][v];
-            } else if (o < s.ns) {
-                Y[(s.first + o) * ldx + j0 + j] = acc[u][v];
-            } else {
-                fv[(s.fv_off + o) * ldf + j0 + j] += acc[u][v];
-            }
+        if (tc >= kc) continue;
+        const int j = j0 + tc;
+        if (it.nsplit > 1) {
+            part[(it.part_row + (int64_t)it.split * nout + o) * ldf + j] = acc[u];
+        } else if (BWD) {
+            X[(s.first + o) * ldx + j] = acc[u];
+        } else if (o < s.ns) {
+            Y[(s.first + o) * ldx + j] = acc[u];
+        } else {
+            fv[(s.fv_off + o) * ldf + j] += acc[u];
         }
     }
 }
@@ -1277,9 +1278,6 @@ int factor_solve(Session* s, Factor& f, const T* R, int64_t ldr, int k, T* P, in
     const SolveItem* items = reinterpret_cast<const SolveItem*>(f.items.p);
     const SolveItem* red = reinterpret_cast<const SolveItem*>(f.red_items.p);
     const int H = (int)f.levels.size() - 1;
-    const bool narrow = k <= 16;
-    const int rc = narrow ? 16 : 64;
-    const int rchunks = ceil_div(k, rc);
     // FP32: TN columns per thread, 32 TN per CTA, the smallest TN whose tile holds all k columns
     const int tn = std::min(8, ceil_div(k, 32));
     auto gemm = [&](int h, bool bwd) -> int {
@@ -1311,15 +1309,10 @@ int factor_solve(Session* s, Factor& f, const T* R, int64_t ldr, int k, T* P, in
             rc = bwd ? pick(std::true_type{}) : pick(std::false_type{});
             HBSD_TRY(rc);
         } else if (sw.n_items > 0) {
-            dim3 g(sw.n_items, rchunks);
+            dim3 g(sw.n_items, ceil_div(k, 16));
             const SolveItem* it = items + sw.item_off;
-            if (bwd) {
-                if (narrow) k_solve_gemm<T, 16, true><<<g, 256, 0, st>>>(dsn, it, G, f.d_struct.p, k, fv, ld, Y, X, ld, part);
-                else k_solve_gemm<T, 64, true><<<g, 256, 0, st>>>(dsn, it, G, f.d_struct.p, k, fv, ld, Y, X, ld, part);
-            } else {
-                if (narrow) k_solve_gemm<T, 16, false><<<g, 256, 0, st>>>(dsn, it, G, f.d_struct.p, k, fv, ld, Y, X, ld, part);
-                else k_solve_gemm<T, 64, false><<<g, 256, 0, st>>>(dsn, it, G, f.d_struct.p, k, fv, ld, Y, X, ld, part);
-            }
+            if (bwd) k_solve_gemm<T, true><<<g, 256, 0, st>>>(dsn, it, G, f.d_struct.p, k, fv, ld, Y, X, ld, part);
+            else k_solve_gemm<T, false><<<g, 256, 0, st>>>(dsn, it, G, f.d_struct.p, k, fv, ld, Y, X, ld, part);
             HBSD_LAUNCHED(s);
         }
         if (sw.n_red > 0) {
