@@ -211,22 +211,141 @@ __global__ void __launch_bounds__(256) k_gram_partial(Seg2<T> Z, Seg2<T> ZH, Seg
         }
 }
 
-// Sum the chunks in order and symmetrise: X_R = (A + A^T) / 2.
-__global__ void k_gram_final(const double* __restrict__ partial, int nchunks, int q,
-                             double* __restrict__ HR, double* __restrict__ SR) {
+// The same with 24 x 24 outputs per CTA of 64 threads, 3 x 3 per thread: for widths that leave 32 x 32 tiles too empty
+// (gram_plan).
+template <class T>
+__global__ void __launch_bounds__(64) k_gram_partial24(Seg2<T> Z, Seg2<T> ZH, Seg2<T> ZS, int q, int64_t n,
+                                                     int64_t rows_per_chunk, int tiles, double* __restrict__ partial) {
+    constexpr int U = 3, W = 8 * U;
+    __shared__ T sz[32][W + 1], sh[32][W + 1], ss[32][W + 1];
+    const int tile = blockIdx.x;
+    const int a0 = tile / tiles * W, b0 = tile % tiles * W;
+    const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
+    const int64_t r0 = (int64_t)blockIdx.y * rows_per_chunk;
+    const int64_t r1 = min(n, r0 + rows_per_chunk);
+    double accH[U][U], accS[U][U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int v = 0; v < U; ++v) accH[u][v] = accS[u][v] = 0.0;
+    for (int64_t i0 = r0; i0 < r1; i0 += 32) {
+        const int rows = (int)min((int64_t)32, r1 - i0);
+#pragma unroll 4
+        for (int t = threadIdx.x; t < 32 * W; t += 64) {
+            const int rr = t / W, cc = t - rr * W;
+            const int64_t i = i0 + rr;
+            const bool ok = rr < rows;
+            sz[rr][cc] = (ok && a0 + cc < q) ? Z.at(i, a0 + cc) : T(0);
+            sh[rr][cc] = (ok && b0 + cc < q) ? ZH.at(i, b0 + cc) : T(0);
+            ss[rr][cc] = (ok && b0 + cc < q) ? ZS.at(i, b0 + cc) : T(0);
+        }
+        __syncthreads();
+        T tH[U][U], tS[U][U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int v = 0; v < U; ++v) tH[u][v] = tS[u][v] = T(0);
+#pragma unroll 2
+        for (int rr = 0; rr < rows; ++rr) {
+            T z[U], h[U], s[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                z[u] = sz[rr][ty + 8 * u];
+                h[u] = sh[rr][tx + 8 * u];
+                s[u] = ss[rr][tx + 8 * u];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int v = 0; v < U; ++v) {
+                    tH[u][v] = fma(z[u], h[v], tH[u][v]);
+                    tS[u][v] = fma(z[u], s[v], tS[u][v]);
+                }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int v = 0; v < U; ++v) { accH[u][v] += (double)tH[u][v]; accS[u][v] += (double)tS[u][v]; }
+        __syncthreads();
+    }
     const int64_t qq = (int64_t)q * q;
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= qq) return;
+    double* ph = partial + (int64_t)blockIdx.y * 2 * qq;
+    double* ps = ph + qq;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int v = 0; v < U; ++v) {
+            const int a = a0 + ty + 8 * u, b = b0 + tx + 8 * v;
+            if (a < q && b < q) {
+                ph[(int64_t)a * q + b] = accH[u][v];
+                ps[(int64_t)a * q + b] = accS[u][v];
+            }
+        }
+}
+
+// Tiles and chunks of rows of one product.  The FP64 pipe bounds it (64 clocks for a warp's multiply-add), so
+// the width decides by padding: 24 x 24 tiles where they leave a tenth less than 32 x 32 ones -- q = 71, n = 20,613:
+// 405 us against 764; q = 35: 211 against 396.  Chunks of at least 32 rows, enough for 8 (16) CTAs per SM: with
+// 128 rows or more, q = 64 of 646 rows took 84 us, now 31.
+struct GramPlan {
+    int w, tiles, nch;
+    int64_t rpc;
+};
+static GramPlan gram_plan(int64_t n, int q, size_t most) {
+    GramPlan g;
+    const int64_t w24 = (int64_t)ceil_div(q, 24) * 24, w32 = (int64_t)ceil_div(q, 32) * 32;
+    g.w = 11 * w24 * w24 < 10 * w32 * w32 ? 24 : 32;
+    g.tiles = ceil_div(q, g.w);
+    int64_t nch = std::max<int64_t>(1, std::min<int64_t>((n + 31) / 32, ceil_div(g.w == 24 ? 2432 : 1216, g.tiles * g.tiles)));
+    nch = std::min<int64_t>(nch, (int64_t)most);
+    g.rpc = (n + nch - 1) / nch;
+    if (g.w == 32) g.rpc = round_up(g.rpc, 32);   // that kernel works in whole row tiles
+    g.nch = (int)((n + g.rpc - 1) / g.rpc);
+    return g;
+}
+template <class T>
+static void gram_partials(const GramPlan& g, Seg2<T> Z, Seg2<T> ZH, Seg2<T> ZS, int q, int64_t n, double* partial, cudaStream_t st) {
+    const dim3 grid(g.tiles * g.tiles, g.nch);
+    if (g.w == 24) k_gram_partial24<T><<<grid, 64, 0, st>>>(Z, ZH, ZS, q, n, g.rpc, g.tiles, partial);
+    else k_gram_partial<T><<<grid, 256, 0, st>>>(Z, ZH, ZS, q, n, g.rpc, g.tiles, partial);
+}
+
+// Sum the chunks, eight strands of them in order and the strands in order, and symmetrise: HR, SR = (A + A^T) / 2;
+// SKEW (the complex recovery): HR = (A - A^T) / 2, the antisymmetric part of Z^T V1.
+template <bool SKEW>
+__global__ void __launch_bounds__(256) k_gram_final(const double* __restrict__ partial, int nchunks, int q,
+                                                    double* __restrict__ HR, double* __restrict__ SR) {
+    __shared__ double red[4][8][33];
+    const int64_t qq = (int64_t)q * q;
+    const int l = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int64_t idx = (int64_t)blockIdx.x * 32 + l;
     const int a = (int)(idx / q), b = (int)(idx % q);
     double h_ab = 0, h_ba = 0, s_ab = 0, s_ba = 0;
-    for (int c = 0; c < nchunks; ++c) {
-        const double* ph = partial + (int64_t)c * 2 * qq;
-        h_ab += ph[(int64_t)a * q + b];
-        h_ba += ph[(int64_t)b * q + a];
-        s_ab += ph[qq + (int64_t)a * q + b];
-        s_ba += ph[qq + (int64_t)b * q + a];
+    if (idx < qq) {
+        const int64_t t = (int64_t)b * q + a;
+#pragma unroll 4
+        for (int c = g; c < nchunks; c += 8) {
+            const double* ph = partial + (int64_t)c * 2 * qq;
+            h_ab += ph[idx];
+            h_ba += ph[t];
+            s_ab += ph[qq + idx];
+            s_ba += ph[qq + t];
+        }
     }
-    HR[idx] = 0.5 * (h_ab + h_ba);
+    red[0][g][l] = h_ab;
+    red[1][g][l] = h_ba;
+    red[2][g][l] = s_ab;
+    red[3][g][l] = s_ba;
+    __syncthreads();
+    if (g != 0 || idx >= qq) return;
+#pragma unroll
+    for (int i = 1; i < 8; ++i) {
+        h_ab += red[0][i][l];
+        h_ba += red[1][i][l];
+        s_ab += red[2][i][l];
+        s_ba += red[3][i][l];
+    }
+    HR[idx] = SKEW ? 0.5 * (h_ab - h_ba) : 0.5 * (h_ab + h_ba);
     SR[idx] = 0.5 * (s_ab + s_ba);
 }
 
@@ -237,18 +356,14 @@ int gram2(Session* s, const T* Z0, int64_t ld0, int q0, const T* Z1, int64_t ld1
           cudaStream_t st) {
     const int q = q0 + q1;
     if (q <= 0) return 0;
-    const int tiles = ceil_div(q, 32);
-    int nch = (int)std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, ceil_div(1216, tiles * tiles)));
-    const int64_t rpc = (n + nch - 1) / nch;
-    nch = (int)((n + rpc - 1) / rpc);
-    const size_t need = (size_t)nch * 2 * q * q;
+    const GramPlan g = gram_plan(n, q, SIZE_MAX >> 1);
+    const size_t need = (size_t)g.nch * 2 * q * q;
     HBSD_TRY(s->ws.alloc(need + 64));
     Seg2<T> Z{Z0, ld0, q0, Z1, ld1}, ZH{H0, ldh0, q0, H1, ldh1}, ZS{S0, lds0, q0, S1, lds1};
-    dim3 grid(tiles * tiles, nch);
-    k_gram_partial<T><<<grid, 256, 0, st>>>(Z, ZH, ZS, q, n, rpc, tiles, s->ws.p);
+    gram_partials(g, Z, ZH, ZS, q, n, s->ws.p, st);
     HBSD_LAUNCHED(s);
     const int64_t qq = (int64_t)q * q;
-    k_gram_final<<<ceil_div(qq, 256), 256, 0, st>>>(s->ws.p, nch, q, HR, SR);
+    k_gram_final<false><<<ceil_div(qq, 32), 256, 0, st>>>(s->ws.p, g.nch, q, HR, SR);
     HBSD_LAUNCHED(s);
     return 0;
 }
@@ -260,39 +375,16 @@ template int gram2<float>(Session*, const float*, int64_t, int, const float*, in
                           double*, cudaStream_t);
 
 // ---- cross Gram of the complex recovery ----------------------------------------------------
-// Sum the chunks in order; A1 = (X - X^T) / 2 (the antisymmetric part of Z^T V1), A2 = (Y + Y^T) / 2.
-__global__ void k_gram_final_skew(const double* __restrict__ partial, int nchunks, int q,
-                                  double* __restrict__ A1, double* __restrict__ A2) {
-    const int64_t qq = (int64_t)q * q;
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= qq) return;
-    const int a = (int)(idx / q), b = (int)(idx % q);
-    double x_ab = 0, x_ba = 0, y_ab = 0, y_ba = 0;
-    for (int c = 0; c < nchunks; ++c) {
-        const double* px = partial + (int64_t)c * 2 * qq;
-        x_ab += px[(int64_t)a * q + b];
-        x_ba += px[(int64_t)b * q + a];
-        y_ab += px[qq + (int64_t)a * q + b];
-        y_ba += px[qq + (int64_t)b * q + a];
-    }
-    A1[idx] = 0.5 * (x_ab - x_ba);
-    A2[idx] = 0.5 * (y_ab + y_ba);
-}
-
 int gram_skew(Session* s, const double* Z, int64_t ldz, const double* V1, int64_t ldv1, const double* V2,
               int64_t ldv2, int64_t n, int q, double* A1, double* A2, cudaStream_t st) {
     if (q <= 0) return 0;
-    const int tiles = ceil_div(q, 32);
-    int nch = (int)std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, ceil_div(1216, tiles * tiles)));
-    const int64_t rpc = (n + nch - 1) / nch;
-    nch = (int)((n + rpc - 1) / rpc);
-    HBSD_TRY(s->ws.alloc((size_t)nch * 2 * q * q + 64));
+    const GramPlan g = gram_plan(n, q, SIZE_MAX >> 1);
+    HBSD_TRY(s->ws.alloc((size_t)g.nch * 2 * q * q + 64));
     Seg2<double> A{Z, ldz, q, nullptr, 0}, B1{V1, ldv1, q, nullptr, 0}, B2{V2, ldv2, q, nullptr, 0};
-    dim3 grid(tiles * tiles, nch);
-    k_gram_partial<double><<<grid, 256, 0, st>>>(A, B1, B2, q, n, rpc, tiles, s->ws.p);
+    gram_partials(g, A, B1, B2, q, n, s->ws.p, st);
     HBSD_LAUNCHED(s);
     const int64_t qq = (int64_t)q * q;
-    k_gram_final_skew<<<ceil_div(qq, 256), 256, 0, st>>>(s->ws.p, nch, q, A1, A2);
+    k_gram_final<true><<<ceil_div(qq, 32), 256, 0, st>>>(s->ws.p, g.nch, q, A1, A2);
     HBSD_LAUNCHED(s);
     return 0;
 }
@@ -335,18 +427,13 @@ int gram_noalloc(const double* Z, int64_t ldz, const double* ZH, int64_t ldzh, c
                                       " exceeds the static scratch (2 q^2 <= 2^21 doubles, q <= 1024)");
     double* scratch = nullptr;
     HBSD_TRY(gram_static_address(&scratch));
-    const int tiles = ceil_div(q, 32);
-    int nch = (int)std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, ceil_div(1216, tiles * tiles)));
-    nch = (int)std::min<size_t>((size_t)nch, GRAM_STATIC_DOUBLES / per_chunk);
-    const int64_t rpc = (n + nch - 1) / nch;
-    nch = (int)((n + rpc - 1) / rpc);
+    const GramPlan g = gram_plan(n, q, GRAM_STATIC_DOUBLES / per_chunk);
     // every partial element read by k_gram_final is written by k_gram_partial: nothing to clear
     Seg2<double> A{Z, ldz, q, nullptr, 0}, AH{ZH, ldzh, q, nullptr, 0}, AS{ZS, ldzs, q, nullptr, 0};
-    dim3 grid(tiles * tiles, nch);
-    k_gram_partial<double><<<grid, 256, 0, st>>>(A, AH, AS, q, n, rpc, tiles, scratch);
+    gram_partials(g, A, AH, AS, q, n, scratch, st);
     HBSD_LAUNCHED(nullptr);
     const int64_t qq = (int64_t)q * q;
-    k_gram_final<<<ceil_div(qq, 256), 256, 0, st>>>(scratch, nch, q, HR, SR);
+    k_gram_final<false><<<ceil_div(qq, 32), 256, 0, st>>>(scratch, g.nch, q, HR, SR);
     HBSD_LAUNCHED(nullptr);
     return 0;
 }

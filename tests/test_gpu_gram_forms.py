@@ -101,3 +101,23 @@ def test_gram_tensor_core_non_finite(bad):
         assert not np.isfinite(out[iu][hit]).any()
         bound = 2.0 ** -44 * (np.abs(ok).T @ np.abs(B)) + 1e-300
         assert np.all((np.abs(out - ok.T @ B) <= bound)[iu][~hit])
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 646, 5003])
+@pytest.mark.parametrize("q", [1, 23, 24, 25, 33, 48, 71, 73, 97])
+def test_gram_fp64_tiles_and_chunks(q, n):
+    """24 x 24 and 32 x 32 tiles, chunks of 32 rows and more: symmetric, and each entry within the rounding of its n
+    products summed in any order (and of the mean with its mirror image)."""
+    from paper_1308_2445_gb300 import hbsd
+    Z, ZH, ZS = blocks(q, n, 1000 + q)
+    bufs = []
+    for a in (Z, ZH, ZS):
+        t = torch.zeros(n, q + (q & 1), dtype=torch.float64, device="cuda")[:, :q]
+        t.copy_(torch.from_numpy(a))
+        bufs.append(t)
+    HR, SR = (torch.zeros(q, q, dtype=torch.float64, device="cuda") for _ in range(2))
+    hbsd.gram(*bufs, HR, SR)
+    for out, B in ((HR.cpu().numpy(), ZH), (SR.cpu().numpy(), ZS)):
+        assert np.array_equal(out, out.T)
+        exact, mag = Z.T @ B, np.abs(Z).T @ np.abs(B)
+        assert np.all(np.abs(out - 0.5 * (exact + exact.T)) <= 2.0 ** -53 * (n + 4) * (mag + mag.T))
