@@ -97,3 +97,16 @@ def test_update_non_finite(bad):
     out = update(Z, W)[:, :k]
     assert not np.isfinite(out[hit]).any()
     assert np.all((np.abs(out - exact) <= bound)[~hit])
+
+
+@pytest.mark.parametrize("n,q,k", [(1, 1, 1), (15, 3, 3), (17, 40, 16), (33, 70, 63), (16, 90, 64), (47, 66, 65), (100, 140, 130)])
+def test_update_fp64_columns(n, q, k):
+    """The FP64 form's items (four rows, a column) at the edges of warps, CTAs and rows: the rounding of q products."""
+    from paper_1308_2445_gb300 import hbsd
+    Z, W = blocks(n, q, k, 1100 + q)
+    t = torch.zeros(n, q + (q & 1), dtype=torch.float64, device="cuda")[:, :q]
+    t.copy_(torch.from_numpy(Z))
+    hbsd.update(t, torch.from_numpy(W).cuda(), k)
+    out = t.cpu().numpy()
+    assert np.array_equal(out[:, k:], Z[:, k:])
+    assert np.all(np.abs(out[:, :k] - Z @ W) <= 2.0 ** -53 * 2 * (q + 2) * (np.abs(Z) @ np.abs(W)))
