@@ -107,8 +107,8 @@ typedef struct {
     uint64_t seed;      /* seed of the SplitMix64 normals used when X0 is NULL                           */
     int local_solver;   /* HBSD_LOCAL_* (default MINRES)                                                */
     int tc_update;      /* mixed form, experimental: 1 runs steps 10-11 on the tensor cores from exact
-                           bf16 slices (as hbsd_update_oz) while q <= 640; 0 (default) in double-float
-                           on the FP32 pipes.  The slices are fixed point against each row's largest
+                           bf16 slices (as hbsd_update_oz) while q <= 640; 0 (default) as
+                           hbsd_update_df64 does.  The bf16 slices are fixed point against each row's largest
                            entry, and the rows of the search blocks span many orders of magnitude
                            across their columns: with 1 the solves of the synthetic workloads stall
                            above 1e-8.  The FP64 form ignores it.                                       */
@@ -483,8 +483,8 @@ void hbsd_server_destroy(hbsd_server* sv);
  * steps whose best shape depends on the problem's size, on seeded data on the session's stream,
  * and keeps the fastest for the session's later solves:
  *   - the fused SpMM of steps 3/7 (in the session's precision form; w columns): the most lanes
- *     per matrix row, 4, 8, 16 or 32 (fewer lanes per row put more rows in a CTA and more
- *     column chunks in a lane);
+ *     per matrix row, 4, 8, 16 or 32 (fewer lanes per row put more rows in a CTA and take more
+ *     passes over the columns; double-float products use at most 4 whatever the limit);
  *   - the cooperative MINRES launch of step 6(b) (min(w, 32) columns, 10 steps): its CTA count,
  *     the whole GPU or 1/2 ... 1/32 of it; the smallest count within 10% of the fastest is kept
  *     (cheaper grid barriers, and SMs left to the other sessions of a batch).

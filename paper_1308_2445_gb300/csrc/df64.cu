@@ -4,8 +4,8 @@
 // FP64 rate is the bound runs faster as pairs of floats (hi + lo, Dekker 1971; Knuth's
 // TwoSum): a product of two pairs is hi*hi exactly (TwoProd by FMA) plus the two cross terms,
 // and the running sum is a pair kept by TwoSum and renormalised every few terms.  About 48
-// significant bits per term; the Gram sums keep FP64 across 128-row tiles, so their long sums
-// carry FP64 accuracy.
+// significant bits per term; the Gram sums go over to FP64 every 64 rows, so their long sums
+// carry FP64 accuracy.  Large products run on the tensor cores instead (gram_tc.cu, update_tc.cu).
 //
 // The pair arithmetic (split, TwoProd + TwoSum, renormalisation) is in df64.h.
 #include <mutex>

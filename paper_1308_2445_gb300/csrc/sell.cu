@@ -9,7 +9,7 @@
 // load yields both.
 //
 // Block vectors are row-major, so the X-row that a nonzero needs is one contiguous vector.
-// A row is handled by lpr lanes; each lane owns VW consecutive columns per chunk (one 16-byte
+// A row is handled by lpr lanes; each lane owns VW consecutive columns per pass (one 16-byte
 // vector load), so the gather of an X row is coalesced and vectorised.
 #include <algorithm>
 #include <cmath>
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(256) k_sell_pattern(int64_t n_slices, int C, c
 
 // The H values in the same way, with the scaled pencil (D Hs D, D S D) in FP32 for the FP32 step entry points (FP32
 // works only on this pencil: the unscaled basis spans ~30 orders of magnitude) and as float pairs, the nearest
-// float and the nearest float to the remainder.  On the host this took 21 ms per matrix of 5.9 M entries, the copies
+// float and the nearest float to the remainder.  On the host this took 21 ms per matrix of 2.95 M entries, the copies
 // of the finished arrays included; here the copy of the CSR values is most of it.
 __global__ void __launch_bounds__(256) k_sell_values(int64_t n_slices, int C, const int64_t* __restrict__ slice_ptr,
                                                      const int32_t* __restrict__ slot_row, const int64_t* __restrict__ row_ptr,
@@ -215,7 +215,7 @@ __device__ __forceinline__ void ldhs(const float2* hs, int64_t e, float& h, floa
 // passes of (1 << lpr_log2) vectors.
 // Bound by the FP64 pipe (a multiply-add of a warp takes it 64 clocks, idle lanes included) and on small
 // matrices by the chain of index and X loads.  One vector per lane: with up to four, 85 columns of the 32^3
-// problem (47,620 rows, 124 entries each) took 1,042 us instead of 988, 64 columns of the 16^3 one 72 instead of 52.
+// problem (47,620 rows, 62 entries each) took 1,042 us instead of 988, 64 columns of the 16^3 one 72 instead of 52.
 template <class T, int MODE, bool SPLIT>
 __global__ void __launch_bounds__(256) k_spmm(
     const int64_t* __restrict__ slice_ptr, const int32_t* __restrict__ slice_len,
@@ -307,7 +307,7 @@ static int spmm_launch(Session* s, const Sell& m, const T* X, int64_t ldx, int k
     if ((ldx % VW) || (ld0 % VW) || (MODE == 0 && (ld1 % VW)))
         return fail(HBSD_ERR_ARG, "spmm: leading dimensions must be multiples of the vector width");
     // FP64 rows of a small matrix are split over 2 to 8 groups of lanes: 19 columns of the 8^3 problem (646 rows)
-    // took 28.7 us on one group, its 80 entries one after another, and 11 us on 8.  By the matrix alone, so that a
+    // took 28.7 us on one group, its 38 (up to 77) entries one after another, and 11 us on 8.  By the matrix alone, so that a
     // column's sums do not depend on the block it is in; from 4,797 rows on (16^3) the pipe is busy without.
     int parts_log2 = 0;
     if (sizeof(T) == 8)
