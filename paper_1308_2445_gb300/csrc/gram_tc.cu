@@ -1,23 +1,27 @@
-// Gram products of step 8 on the tensor cores, by exact digit slices, with the accuracy of the
-// double-float form guaranteed entry by entry (mixed form: H_R = Z^T ZH, S_R = Z^T ZS, entries a <= b).
+// Gram products of step 8 on the tensor cores, by exact digit slices, with the accuracy of the double-float
+// form checked entry by entry (mixed form: H_R = Z^T ZH, S_R = Z^T ZS, entries a <= b).
 //
 // The splitting idea is that of Ozaki, Ogita, Oishi and Rump ("Error-free transformations of matrix
 // multiplication by using fast routines of matrix multiplication", Numer. Algorithms 59, 2012), in the
 // fixed point of one chunk of rows:
 //  - row i of Z is scaled by 2^-r_i and row i of ZH, ZS by 2^r_i, r_i the exponent of the row's largest
 //    |Z| entry (the rows of an enriched basis span tens of decades, inversely in Z and in ZH, ZS);
-//  - column a of the scaled Z is written as a 62-bit integer against its largest entry of the chunk, and
+//  - column a of the scaled Z is rounded to a 62-bit integer against its largest entry of the chunk, and
 //    cut into 8 balanced base-256 digits d_s in [-128, 127] (the leading one in [-64, 64]), each exact in
 //    FP16: slice s holds the digits d_s.  ZH and ZS likewise.
 //  - digit products of equal weight 2^(-8 L), L = s + t <= 7, are summed by tcgen05.mma into one FP32
 //    accumulator per level; over 256 rows the sums of levels 0-4 stay within 2^24, so they are exact, and
 //    the rounding of levels 5-7 is far below the last bit kept.  Levels above 7 are dropped.
-//  - every 256 rows the levels are added in 64-bit integers (unit 2^-37 of the leading digit product),
-//    which hold the whole chunk (at most 8192 rows) without overflow.
-// The truncations leave an error of about sqrt(rows) 2^-61.7 of max|z| max|h| of the scaled columns in the
-// chunk.  That is below the double-float form's rounding, 2^-48 sum|z||h|, wherever
-//     sum|z||h| >= sqrt(rows) 2^-13 max|z| max|h|,
-// which search blocks meet with bits to spare although a few rows dominate their columns (16^3 case: at
+//  - every 256 rows the levels are added in 72-bit integers (unit 2^-45 of the leading digit product: 64 bits
+//    and a byte of fraction), which hold the whole chunk (at most 8192 rows) without overflow.
+// With P the product of the two columns' leading powers of two in the chunk and R its rows, the rounded operands and the
+// dropped levels leave about sqrt(R) 2^-60 P, and the rounding of levels 6 and 7 at most 2^-56 P per 256 rows.  That is
+// within the double-float form's rounding, 2^-48 sum|z||h|, wherever
+//     sum|z||h| >= sqrt(R) 2^-11 P
+// (random and same-signed columns on that line, emulated: at most 2^-47.8).  It takes the errors of different rows as
+// independent.  Columns that repeat the same digits row after row beside maxima in other rows add them up one way: up to
+// 2^-41 of sum|z||h| on the line at R = 8192, 2^-44 at R = 256; constant columns without such maxima lie far above it.
+// Search blocks meet the line with bits to spare although a few rows dominate their columns (16^3 case: at
 // least 2^-3.8 max|z| max|h|).  The kernel checks it for every entry: it first sums |z||h| (FP16, one MMA
 // per step) over one row in 16, the one with the largest scaled ZH entry of its group, a lower bound
 // within one or two bits on such blocks.  Entries that fail (none to some dozens of a million on the 32^3
@@ -31,8 +35,9 @@
 // would take at least 50 clocks each).
 //
 // Bound: the integer pipe of the slicers (about 30 integer instructions per value and tile it meets; the
-// tensor core waits for them).  n = 334,272, q = 538: 9.7 ms against 40.5 ms for the FP32 pipes;
-// n = 47,620, q = 149: 0.27 against 0.64 ms.  Error against 64 bits on such blocks 2e-16, float pairs 2e-15.
+// tensor core waits for them).  n = 334,272, q = 538: 9.9 ms against 40.5 ms for the FP32 pipes;
+// n = 47,620, q = 149: 0.28 against 0.64 ms.  Error against 64 bits on such blocks 5e-16 (q = 538: 1.9e-15, most of it the
+// 64-bit reference's own), float pairs 2e-15.
 #include <algorithm>
 #include <mutex>
 #include <string>
@@ -56,11 +61,11 @@ constexpr int TG_STEPS = FLUSH_STEPS;           // MMA steps per flush
 constexpr int TG_MAX_BLKS = 32;                 // flushes per chunk: 8192 rows keep the sums below 2^62
 constexpr int TG_NS = 3;                        // stage buffers
 constexpr int TG_STAGE = DIG * (A_SLICE + B_SLICE);
-constexpr int TG_ACC = 2 * TG_B * TG_M;         // 64-bit sums per unit
+constexpr int TG_ACC = 2 * TG_B * TG_M;         // sums per unit, 64 bits and a byte of fraction each
 constexpr int TG_ATHREADS = 256;                // warps 0-7: slices of Z, flush
 constexpr int TG_SLICERS = TG_ATHREADS + 128;   // warps 8-11: slices of ZH and ZS
 constexpr int TG_THREADS = TG_SLICERS + 32;     // warp 12: MMA issue
-constexpr size_t TG_SMEM = (size_t)TG_NS * TG_STAGE + (size_t)TG_ACC * 8 + 1024;
+constexpr size_t TG_SMEM = (size_t)TG_NS * TG_STAGE + (size_t)TG_ACC * 9 + 1024;
 constexpr int TG_UNIT_FIX = 256;                // failing entries of a unit that are computed one by one
 constexpr int TG_EXP_ROWS = 32;                 // rows per CTA of the exponent pass
 
@@ -148,7 +153,7 @@ __device__ __forceinline__ void tg_pair(int p, int nb, int& ta, int& tb) {
 __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Seg2d ZS, int q, int64_t n,
                                                            int64_t chunk_rows, int nb, const int* __restrict__ rexp,
                                                            const int* __restrict__ cexp, const int* __restrict__ sel,
-                                                           long long* __restrict__ part, int* __restrict__ list) {
+                                                           double* __restrict__ part, int* __restrict__ list) {
     extern __shared__ __align__(1024) uint8_t tg_smem[];
     __shared__ __align__(8) uint64_t full[TG_NS], empty[TG_NS], phasedone, accfree;
     __shared__ uint32_t tslot;
@@ -164,6 +169,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
     const int* ce = cexp + (int64_t)blockIdx.y * 3 * q;
     uint8_t* base = tg_smem + ((1024 - (tc::smem_u32(tg_smem) & 1023)) & 1023);
     long long* sacc = reinterpret_cast<long long*>(base + TG_NS * TG_STAGE);   // [64 columns b][128 columns a]
+    uint32_t* slow = reinterpret_cast<uint32_t*>(sacc + TG_ACC);               // [16][128]: fractions, four columns b in a word
     if (tid == 0) {
         for (int i = 0; i < TG_NS; ++i) {
             tc::mbar_init(&full[i], TG_SLICERS / 32);
@@ -238,10 +244,14 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
         const int stride = isa ? A_SLICE : B_SLICE;
         const int frow = (warp & 3) * 32 + lane, fm = (warp >> 2) & 1;   // column a, matrix of the reading
         const uint32_t taddr = tbase + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(fm * TG_B);
-        long long* facc = sacc + (int64_t)fm * TG_B * TG_M + frow;
+        long long* facc = sacc + fm * TG_B * TG_M + frow;
+        uint32_t* flow = slow + fm * (TG_B / 4) * TG_M + frow;
         if (isa)
 #pragma unroll 4
-            for (int c = 0; c < TG_B; ++c) facc[c * TG_M] = 0;
+            for (int c = 0; c < TG_B; ++c) {
+                facc[c * TG_M] = 0;
+                if (c < TG_B / 4) flow[c * TG_M] = 0;
+            }
         auto read_phase = [&](int ph) -> bool {
             if (!tc::mbar_wait(&phasedone, (uint32_t)(ph & 1), WAIT_NS)) return false;
             tc::fence_after_sync();
@@ -273,9 +283,15 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
                     for (int l = 0; l < 8; ++l) tmem_ld8(taddr + (uint32_t)(2 * TG_B * l + c0), v[l]);
                     asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const uint32_t l[8] = {v[0][c], v[1][c], v[2][c], v[3][c], v[4][c], v[5][c], v[6][c], v[7][c]};
-                        facc[(c0 + c) * TG_M] += fold_levels(l);
+                    for (int c = 0; c < 8; c += 4) {
+                        uint32_t w = flow[(c0 + c) / 4 * TG_M];
+#pragma unroll
+                        for (int d = 0; d < 4; ++d) {
+                            const uint32_t l[8] = {v[0][c + d], v[1][c + d], v[2][c + d], v[3][c + d],
+                                                   v[4][c + d], v[5][c + d], v[6][c + d], v[7][c + d]};
+                            facc[(c0 + c + d) * TG_M] += fold_levels(l, w, d);
+                        }
+                        flow[(c0 + c) / 4 * TG_M] = w;
                     }
                 }
             }
@@ -376,19 +392,17 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
         int* ents = list + 2 + gridDim.x * gridDim.y + s_base;
         for (int t = tid; t < nfix; t += TG_THREADS) ents[t] = (unit << 13) | s_ent[t];
     }
-    long long* out = part + (int64_t)unit * TG_ACC;
-    for (int t = tid; t < TG_ACC; t += TG_THREADS) out[t] = sacc[t];
-}
-
-// An FP64 value in place of a unit's integer: the leading 62 bits under the tag 01, which no sum has
-__device__ __forceinline__ long long tag_double(double v) {
-    return (long long)(0x4000000000000000ull | ((unsigned long long)__double_as_longlong(v) >> 2));
+    double* out = part + (int64_t)unit * TG_ACC;
+    for (int t = tid; t < TG_ACC; t += TG_THREADS) {
+        const int a = a0 + (t & (TG_M - 1)), c = t / TG_M, b = b0 + (c & (TG_B - 1));
+        if (a < q && b < q) out[t] = scaled_sum(sacc[t], slow[c / 4 * TG_M + (t & (TG_M - 1))], c & 3, ce[a] + ce[(1 + c / TG_B) * q + b] - 2056 - FRAC);
+    }
 }
 
 // The listed units in double-float, four 32 x 32 tiles each, and the listed entries in FP64, one CTA each
 __global__ void __launch_bounds__(GTHREADS, GCTAS) k_gram_tc_fixup(Seg2d Z, Seg2d ZH, Seg2d ZS, int q, int64_t n,
                                                                    int64_t chunk_rows, int nb, int npair, int units,
-                                                                   df::f32x2 nz, long long* __restrict__ part,
+                                                                   df::f32x2 nz, double* __restrict__ part,
                                                                    const int* __restrict__ list) {
     __shared__ GramTile sm;
     const int cnt = list[0], nent = list[1];
@@ -400,9 +414,9 @@ __global__ void __launch_bounds__(GTHREADS, GCTAS) k_gram_tc_fixup(Seg2d Z, Seg2
         const int a0 = ta * TG_M + sub * GW, b0 = tb * TG_B;
         if (a0 >= q || a0 > b0) continue;   // tiles above the diagonal only (b0 is a multiple of 32)
         const int64_t r0 = (int64_t)chunk * chunk_rows;
-        long long* out = part + (int64_t)unit * TG_ACC;
+        double* out = part + (int64_t)unit * TG_ACC;
         gram_df64_tile(sm, Z, ZH, ZS, q, a0, b0, GW / 4, false, r0, min(n, r0 + chunk_rows), nz,
-                       [&](int m, int a, int b, double v) { out[(m * TG_B + b - b0) * TG_M + (a - ta * TG_M)] = tag_double(v); });
+                       [&](int m, int a, int b, double v) { out[(m * TG_B + b - b0) * TG_M + (a - ta * TG_M)] = v; });
         __syncthreads();
     }
     double* red = &sm.acc[0][0];
@@ -422,20 +436,14 @@ __global__ void __launch_bounds__(GTHREADS, GCTAS) k_gram_tc_fixup(Seg2d Z, Seg2
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
         __syncthreads();
-        if (threadIdx.x == 0) part[(int64_t)unit * TG_ACC + (m * TG_B + cb) * TG_M + ca] = tag_double((red[0] + red[1]) + (red[2] + red[3]));
+        if (threadIdx.x == 0) part[(int64_t)unit * TG_ACC + (m * TG_B + cb) * TG_M + ca] = (red[0] + red[1]) + (red[2] + red[3]);
         __syncthreads();
     }
 }
 
-// A unit's sum, or a tagged FP64 value
-__device__ __forceinline__ double unit_value(long long v, int e) {
-    return (v >> 62) == 1 ? __longlong_as_double(v << 2) : scaled_double(v, e);
-}
-
 // Sum of the chunks in order; the entry (a, b), a <= b, is used for (b, a) too.
-__global__ void __launch_bounds__(256) k_gram_tc_final(const long long* __restrict__ part, const int* __restrict__ cexp,
-                                                       int nchunks, int npair, int nb, int q, double* __restrict__ HR,
-                                                       double* __restrict__ SR) {
+__global__ void __launch_bounds__(256) k_gram_tc_final(const double* __restrict__ part, int nchunks, int npair, int nb, int q,
+                                                       double* __restrict__ HR, double* __restrict__ SR) {
     __shared__ double rh[8][33], rs[8][33];
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
     const int64_t idx = (int64_t)blockIdx.x * 32 + lane;
@@ -447,10 +455,9 @@ __global__ void __launch_bounds__(256) k_gram_tc_final(const long long* __restri
         const int pair = ta * nb - 2 * ta * (ta - 1) + tb - 4 * ta;
         const int64_t o = (int64_t)(b - tb * TG_B) * TG_M + (a - ta * TG_M);
         for (int c = g; c < nchunks; c += 8) {
-            const long long* p = part + ((int64_t)c * npair + pair) * TG_ACC + o;
-            const int* ce = cexp + (int64_t)c * 3 * q;
-            h += unit_value(p[0], ce[a] + ce[q + b] - 2056 - FRAC);
-            s += unit_value(p[(int64_t)TG_B * TG_M], ce[a] + ce[2 * q + b] - 2056 - FRAC);
+            const double* p = part + ((int64_t)c * npair + pair) * TG_ACC + o;
+            h += p[0];
+            s += p[TG_B * TG_M];
         }
     }
     rh[g][lane] = h;
@@ -494,10 +501,10 @@ int gram2_tc(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1
     const int nch = ceil_div(n, chunk_rows);
     const int64_t units = (int64_t)nch * npair;
     const int64_t rpad = round_up(n, TG_BLK);
-    // workspace: integer sums | row exponents | column exponents | guard rows | lists
+    // workspace: sums | row exponents | column exponents | guard rows | lists
     const size_t ints = (size_t)rpad + (size_t)nch * 3 * q + (size_t)rpad / 16 + 2 + (size_t)units * (1 + TG_UNIT_FIX);
     HBSD_TRY(s->ws.alloc((size_t)units * TG_ACC + ints / 2 + 64));
-    long long* part = reinterpret_cast<long long*>(s->ws.p);
+    double* part = s->ws.p;
     int* rexp = reinterpret_cast<int*>(part + units * TG_ACC);   // 16-byte aligned: TG_ACC is even
     int* cexp = rexp + rpad;
     int* sel = cexp + (size_t)nch * 3 * q;
@@ -518,7 +525,7 @@ int gram2_tc(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1
     k_gram_tc_fixup<<<152 * GCTAS, GTHREADS, 0, st>>>(Z, ZH, ZS, q, n, chunk_rows, nb, npair, (int)units, df::NEG_ZERO2, part,
                                                       list);
     HBSD_LAUNCHED(s);
-    k_gram_tc_final<<<ceil_div((int64_t)q * q, 32), 256, 0, st>>>(part, cexp, nch, npair, nb, q, HR, SR);
+    k_gram_tc_final<<<ceil_div((int64_t)q * q, 32), 256, 0, st>>>(part, nch, npair, nb, q, HR, SR);
     HBSD_LAUNCHED(s);
     return 0;
 }

@@ -16,7 +16,8 @@ constexpr int COLS = 64;                  // columns of a B slice; level L's acc
 constexpr int A_SLICE = ROWS * 16 * 2;    // bytes of one 128 x 16 slice
 constexpr int B_SLICE = COLS * 16 * 2;    // bytes of one 64 x 16 slice
 constexpr int FLUSH_STEPS = 16;           // steps of 16 between readings of the accumulators: levels 0-4 stay exact
-constexpr int FRAC = 37;                  // fraction bits of the integer sums, in units of the leading digit product
+constexpr int FRAC = 37;                  // fraction bits of the 64-bit sums, in units of the leading digit product
+constexpr int FRAC_LOW = 8;               // further fraction bits, kept beside the sums (fold_levels)
 constexpr int BAD_EXP = 0x40000000;       // exponent of a row or column with a non-finite entry
 constexpr uint64_t WAIT_NS = 2000000000ull;
 
@@ -39,25 +40,27 @@ __device__ __forceinline__ void mma_window(uint32_t tbase, uint64_t a, uint64_t 
         mma<ACC>(tbase + S * COLS + 256, a + S * (A_SLICE >> 4), b + 4 * (B_SLICE >> 4), tc::idesc_f16_f32(ROWS, N - 256));
 }
 
-// |x| as a 62-bit fixed-point integer plus 0x8080808080808080: byte 7 - s is the digit d_s of |x| plus
-// 128.  off: the column's exponent plus or minus the row's; off - exponent field >= 0 is the shift below
-// the maximum.  About 12 integer instructions; the digits of the sign are taken in digits2.
+// |x| as a 62-bit fixed-point integer, rounded to nearest, plus 0x0080808080808080: byte 7 - s is the digit d_s of
+// |x| plus 128, the leading byte d_0 itself.  off: the column's exponent plus or minus the row's; off - exponent
+// field >= 0 is the shift below the maximum.  The rounding takes one more bit, halved after the bias and a half are
+// added; cut instead, same-signed columns lose up to a unit per row, all one way: 2^-44 of sum|z||h| over 8192 rows at
+// the guard's line, 2^-48 rounded.  The digits of the sign are taken in digits2.
 __device__ __forceinline__ unsigned long long fixed62(double x, int off) {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
     const int ex = (int)((hi >> 20) & 0x7FFu);
     const unsigned sh = ex ? (unsigned)(off - ex) : 64u;   // zeros and subnormals enter as zero
-    const unsigned mh = __funnelshift_l(lo, (hi & 0xFFFFFu) | 0x100000u, 9), ml = lo << 9;
-    const unsigned t = __funnelshift_rc(ml, mh, sh);   // shifts by at most 32
-    unsigned rl;
-    asm("shr.b32 %0, %1, %2;" : "=r"(rl) : "r"(t), "r"(sh > 32u ? sh - 32u : 0u));   // 0 from 32 on
-    const unsigned rh = __funnelshift_rc(mh, 0u, sh);
-    return (((unsigned long long)rh << 32) | rl) + 0x8080808080808080ull;
+    const unsigned mh = __funnelshift_l(lo, (hi & 0xFFFFFu) | 0x100000u, 10), ml = lo << 10;
+    unsigned long long v;
+    asm("shr.b64 %0, %1, %2;" : "=l"(v) : "l"(((unsigned long long)mh << 32) | ml), "r"(sh));   // 0 from 64 on
+    return (v + 0x0101010101010101ull) >> 1;
 }
 
-// FP16 digits of two values from one byte of each biased word: 1024 + byte by its bits, then
-// (1024 + byte) sg - 1152 sg = +-d exactly, with sg = +-1 the values' signs and csg = -1152 sg
-__device__ __forceinline__ uint32_t digits2(unsigned w0, unsigned w1, int byte, uint32_t sg, uint32_t csg) {
-    const unsigned z = (__byte_perm(w0, w1, (unsigned)(byte | ((4 + byte) << 8))) & 0x00FF00FFu) | 0x64006400u;
+// FP16 digits s of two values from one byte of each biased integer: 1024 + byte by its bits (the leading byte, at most
+// 64, with its bias put in here), then (1024 + byte) sg - 1152 sg = +-d exactly, with sg = +-1 the values' signs and
+// csg = -1152 sg
+__device__ __forceinline__ uint32_t digits2(unsigned long long u0, unsigned long long u1, int s, uint32_t sg, uint32_t csg) {
+    const unsigned w0 = (unsigned)(s < 4 ? u0 >> 32 : u0), w1 = (unsigned)(s < 4 ? u1 >> 32 : u1), byte = 3 - (s & 3);
+    const unsigned z = (__byte_perm(w0, w1, byte | ((4 + byte) << 8)) & 0x00FF00FFu) | (s == 0 ? 0x64806480u : 0x64006400u);
     uint32_t d;
     asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(z), "r"(sg), "r"(csg));
     return d;
@@ -77,7 +80,7 @@ __device__ __forceinline__ void slice8(const double (&x)[8], const int (&off)[8]
         asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(csg) : "r"(sg), "r"(0xE480E480u));
 #pragma unroll
         for (int s = 0; s < DIG; ++s)
-            w[s][c >> 1] = digits2((unsigned)(s < 4 ? u0 >> 32 : u0), (unsigned)(s < 4 ? u1 >> 32 : u1), 3 - (s & 3), sg, csg);
+            w[s][c >> 1] = digits2(u0, u1, s, sg, csg);
     }
 #pragma unroll
     for (int s = 0; s < DIG; ++s)
@@ -110,20 +113,25 @@ __device__ __forceinline__ void tmem_ld4(uint32_t addr, uint32_t (&v)[4]) {
                  : "r"(addr));
 }
 
-// One output's levels as a 64-bit integer in units of 2^-37 of the leading digit product: levels 0 and 1 (within
-// 2^22) by adding 1.5 * 2^23, whose bits then hold the integer; levels 2-4 by conversion; levels 5-7 together,
-// rounded to 2^-37 of level 0 (2^3 of level 5)
-__device__ __forceinline__ long long fold_levels(const uint32_t (&l)[8]) {
+// One output's levels as a 64-bit integer in units of 2^-37 of the leading digit product, to be added to the output's sum,
+// and its fraction in units of 2^-45, added to byte i of low (the sum's own fraction) with the carry in the result: levels
+// 0 and 1 (within 2^22) by adding 1.5 * 2^23, whose bits then hold the integer; levels 2-5 by conversion; levels 6 and
+// 7 together, rounded to 2^-45 of level 0 (2^3 of level 6).  With levels 5-7 rounded to 2^-37 at every reading, entries
+// that the guard accepts at its line were off by 2^-41 of sum|z||h|, now 2^-48; the fraction and the rounded operands
+// take 2% of the Gram (n = 334,272, q = 538: 9.69 -> 9.89 ms) and 3% of the update (k = 282: 7.00 -> 7.19).
+__device__ __forceinline__ long long fold_levels(const uint32_t (&l)[8], uint32_t& low, int i) {
     const int m0 = __float_as_int(__fadd_rn(__uint_as_float(l[0]), 12582912.0f)) - 0x4B400000;
     const int m1 = __float_as_int(__fadd_rn(__uint_as_float(l[1]), 12582912.0f)) - 0x4B400000;
     const int m2 = __float2int_rn(__uint_as_float(l[2]));
     const int m3 = __float2int_rn(__uint_as_float(l[3]));
     const int m4 = __float2int_rn(__uint_as_float(l[4]));
-    const float g = __fmaf_rn(__fmaf_rn(__uint_as_float(l[7]), 0.00390625f, __uint_as_float(l[6])), 0.00390625f,
-                              __uint_as_float(l[5]));
-    const int m5 = __float_as_int(__fmaf_rn(g, 0.125f, 12582912.0f)) - 0x4B400000;
+    const int m5 = __float2int_rn(__uint_as_float(l[5]));
+    const float g = __fmaf_rn(__uint_as_float(l[7]), 0.00390625f, __uint_as_float(l[6]));
+    const int m6 = __float_as_int(__fmaf_rn(g, 0.125f, 12582912.0f)) - 0x4B400000;
+    const int w = m5 * 32 + m6 + (int)((low >> (8 * i)) & 255u);   // below 2^30
+    low = __byte_perm(low, (uint32_t)w, 0x3210u + ((4u - i) << (4 * i)));
     return (((long long)m0 << 37) + ((long long)m1 << 29)) + (long long)m2 * (1 << 21) + (long long)m3 * (1 << 13) +
-           (long long)m4 * 32 + (long long)m5;
+           (long long)m4 * 32 + (long long)(w >> FRAC_LOW);
 }
 
 // v 2^e without the FP64 pipe (normalise, round to nearest, set the exponent); results outside the normal
@@ -137,6 +145,11 @@ __device__ __forceinline__ double scaled_double(long long v, int e) {
     const unsigned long long f = m << z;   // leading bit 63; the fraction is the next 52, rounded half up
     const unsigned long long bits = ((unsigned long long)ex << 52) + ((f << 1) >> 12) + ((f >> 10) & 1ull);
     return __longlong_as_double((long long)(bits | (v < 0 ? 0x8000000000000000ull : 0ull)));
+}
+// (v + byte i of low 2^-8) 2^e, rounded once: the fraction counts while v has fewer than 55 bits
+__device__ __forceinline__ double scaled_sum(long long v, uint32_t low, int i, int e) {
+    const bool small = v + (1ll << 54) >= 0 && v < (1ll << 54);
+    return scaled_double(small ? (long long)(((unsigned long long)v << FRAC_LOW) | ((low >> (8 * i)) & 255u)) : v, small ? e - FRAC_LOW : e);
 }
 
 }  // namespace slices

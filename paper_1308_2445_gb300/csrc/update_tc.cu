@@ -1,19 +1,20 @@
 // Block update of steps 10-11 on the tensor cores by exact digit slices (slices.h), with the accuracy of the
-// double-float form kept entry by entry (mixed form: Z0(:, 0:k) := [Z0 Z1] W in place).
+// double-float form checked entry by entry (mixed form: Z0(:, 0:k) := [Z0 Z1] W in place).
 //
 // Column c of Z and row c of W are scaled by 2^(e_c) and 2^(-e_c), e_c the exponent of the largest entry of W's
 // row: the search directions are large where their coefficients are small.  Then each row of Z and each column
 // of W is a 62-bit fixed point against its own largest entry, and an output is the sum of the digit products,
-// as in the Gram (gram_tc.cu).  The truncations leave about sqrt(q) 2^-61.7 of the product of the two maxima,
-// below the double-float form's 2^-48 sum|z||w| wherever sum|z||w| >= sqrt(q) 2^-13 of it.  k_tu_guard
-// evaluates sum|z||w| for every output (FP16 magnitudes, one MMA per 16 columns and 256 outputs of a row) and
-// lists the entries below that line -- rows of a search block span many decades, and on the 16^3 case 0.4 to 1% of
-// the outputs are that far below their row's largest term -- which k_tu_fix computes in FP64.  When more than a
-// sixteenth of a slab's entries fail, the slab is computed by the double-float kernels.
+// as in the Gram (gram_tc.cu).  With P the product of the row's and the column's leading powers of two, that leaves
+// about sqrt(q) 2^-60 P and at most 2^-56 P per 256 terms, within the double-float form's 2^-48 sum|z||w| wherever
+// sum|z||w| >= sqrt(q) 2^-11 P (for errors that do not all go one way, as there).  k_tu_guard evaluates
+// sum|z||w| for every output (FP16 magnitudes, one MMA per 16 columns and 256 outputs of a row) and lists the entries
+// below that line -- rows of a search block span many decades, and on the 16^3 case 0.4 to 1% of the outputs are that
+// far below their row's largest term -- which k_tu_fix computes in FP64.  When more than a sixteenth of a slab's
+// entries fail, the slab is computed by the double-float kernels.
 //
 // The rows are worked off in slabs: results go to a scratch block, since the tiles of a row read all of it, and
 // are copied over Z0 when the slab is done.  One slab of 19,456 rows with q = 538, k = 282: exponents 26 us, guard
-// 103, digits and products 230, entries in FP64 14, copy 15.  All 334,272 rows: 6.98 ms, 22.67 with pairs.  Bound
+// 103, digits and products 230, entries in FP64 14, copy 15.  All 334,272 rows: 7.19 ms, 22.67 with pairs.  Bound
 // by cutting Z (once per 64 columns; 16 clocks of four warps per value) and, in the guard, by the latency of the
 // loads of one CTA per SM; the digit products alone are 1.8 ms.
 #include <algorithm>
@@ -35,7 +36,7 @@ constexpr int TU_MTHREADS = 576;                     // main kernel: 8 warps rea
 constexpr int TU_SLICERS = 256;                      // the same of the guard
 constexpr int TU_THREADS = TU_SLICERS + 64;
 constexpr int TU_OUT_LD = 17;                        // doubles per row of a warp's 32 x 16 outputs in shared memory
-constexpr size_t TU_SMEM = (size_t)TU_NS * TU_STAGE + (size_t)8 * 32 * TU_OUT_LD * 8 + 1024;
+constexpr size_t TU_SMEM = (size_t)TU_NS * TU_STAGE + (size_t)8 * 32 * (TU_OUT_LD + 4) * 8 + 1024;
 constexpr int64_t TU_WAVE = 152 * ROWS;              // rows of one tile per SM
 constexpr int64_t TU_SLAB_BYTES = 88 << 20;          // Z rows of a slab: they stay in L2 between the passes
 constexpr int64_t TU_SLAB_ROWS = 65536;              // a list entry holds 16 bits of row
@@ -403,12 +404,16 @@ __global__ void __launch_bounds__(TU_MTHREADS, 1) k_update_tc(Steps S, int64_t r
         const int fr = r0 + (warp & 3) * 32 + lane;
         const int fer = fr < rows ? rowexp[fr] : 0;
         double* o = reinterpret_cast<double*>(base + TU_NS * TU_STAGE) + (int64_t)warp * 32 * TU_OUT_LD;
+        // [8][32]: fractions of this row's 32 sums, four columns in a word (in registers they would spill)
+        uint32_t* low = reinterpret_cast<uint32_t*>(base + TU_NS * TU_STAGE + 8 * 32 * TU_OUT_LD * 8) + warp * 256 + lane;
         bool ok = true;
         int p = 0;
         for (int tile = 0; ok && tile < jt; ++tile) {
             long long acc[32];
 #pragma unroll
             for (int c = 0; c < 32; ++c) acc[c] = 0;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) low[32 * c] = 0;
             for (int u = 0; u < nph; ++u, ++p) {
                 ok = tc::mbar_wait(&phasedone, (uint32_t)(p & 1), WAIT_NS);
                 ok = __all_sync(0xffffffffu, ok);
@@ -420,11 +425,13 @@ __global__ void __launch_bounds__(TU_MTHREADS, 1) k_update_tc(Steps S, int64_t r
 #pragma unroll
                     for (int l = 0; l < 8; ++l) tmem_ld4(taddr + (uint32_t)(COLS * l + c0), v[l]);
                     asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+                    uint32_t w = low[8 * c0];
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
                         const uint32_t l[8] = {v[0][c], v[1][c], v[2][c], v[3][c], v[4][c], v[5][c], v[6][c], v[7][c]};
-                        acc[c0 + c] += fold_levels(l);
+                        acc[c0 + c] += fold_levels(l, w, c);
                     }
+                    low[8 * c0] = w;
                 }
                 tc::fence_before_sync();
                 __syncwarp();
@@ -437,7 +444,8 @@ __global__ void __launch_bounds__(TU_MTHREADS, 1) k_update_tc(Steps S, int64_t r
                 const int j0 = tile * COLS + (warp >> 2) * 32 + 16 * h;
 #pragma unroll
                 for (int c = 0; c < 16; ++c)
-                    o[lane * TU_OUT_LD + c] = j0 + c < k ? scaled_double(acc[16 * h + c], fer + cw[j0 + c] - 2056 - FRAC) : 0.0;
+                    o[lane * TU_OUT_LD + c] =
+                        j0 + c < k ? scaled_sum(acc[16 * h + c], low[32 * (4 * h + c / 4)], c & 3, fer + cw[j0 + c] - 2056 - FRAC) : 0.0;
                 __syncwarp();
                 const int oc = lane & 15;
                 if (j0 + oc < k)
@@ -495,8 +503,7 @@ __global__ void __launch_bounds__(TU_MTHREADS, 1) k_update_tc(Steps S, int64_t r
                     uint32_t d[2];
 #pragma unroll
                     for (int h = 0; h < 2; ++h)
-                        d[h] = digits2((unsigned)(s < 4 ? w[2 * h] >> 32 : w[2 * h]), (unsigned)(s < 4 ? w[2 * h + 1] >> 32 : w[2 * h + 1]),
-                                       3 - (s & 3), sg[h], csg[h]);
+                        d[h] = digits2(w[2 * h], w[2 * h + 1], s, sg[h], csg[h]);
                     *reinterpret_cast<uint2*>(dst + s * A_SLICE) = make_uint2(d[0], d[1]);
                 }
             }

@@ -121,3 +121,44 @@ def test_gram_fp64_tiles_and_chunks(q, n):
         assert np.array_equal(out, out.T)
         exact, mag = Z.T @ B, np.abs(Z).T @ np.abs(B)
         assert np.all(np.abs(out - 0.5 * (exact + exact.T)) <= 2.0 ** -53 * (n + 4) * (mag + mag.T))
+
+
+def rows_at_the_line(n, q, most, tail, seed):
+    """Columns with one entry of about 1 in every block of 256 rows, in another row for Z than for ZH and ZS, and entries
+    of 2^-1 .. 2^-most in one row in 16, where alone Z and ZH, ZS meet: sum |z||h| then goes down to the guard's line,
+    sqrt(rows) 2^-11 of the product of the maxima.  The last columns fix the rows' scales and make these rows those that
+    the guard looks at.  Half of the columns have one sign.  tail: the other rows hold large entries of Z against
+    2^-50 ones of ZH, ZS, whose rounding to 62 bits all go the same way if they are cut."""
+    rng = np.random.default_rng(seed)
+    i = np.arange(n)
+    heavy = i % 16 == 3
+    mag = np.exp2(-np.linspace(1.0, most, q))
+    out = []
+    for m in range(3):
+        A = np.zeros((n, q))
+        if tail:
+            A[:] = 1.9 if m == 0 else 2.0 ** -50 * rng.uniform(0.5, 1.0, (n, q))
+        A[heavy] = mag * rng.uniform(0.5, 1.5, (int(heavy.sum()), q))
+        A[heavy] *= np.where(np.arange(q) % 2, 1.0, rng.choice([-1.0, 1.0], (int(heavy.sum()), q)))
+        A[i % 256 == (0 if m == 0 else 1)] = 1.3 if m == 0 else 1.7
+        A[i % 256 == (1 if m == 0 else 0)] = 0.0
+        A[:, -1] = 1.9 if m == 0 else np.where(heavy, 64.0, 1.0)
+        out.append(A)
+    return out
+
+
+# most: where 16 of 256 rows (128 of 2,048) leave sum |z||h| at about the line for the smallest pair of columns
+@pytest.mark.parametrize("n,most,tail", [(6000, 5.4, False), (48000, 6.2, False), (48000, 6.2, True)])
+def test_gram_tensor_core_entries_just_above_the_guard(n, most, tail):
+    """Entries that the guard accepts at its line.  Bound 2^-46 of |Z|^T |ZH|: with P the product of the columns' leading
+    powers of two and R rows, the sums of the lowest levels are rounded to 2^-56 P once per 256 rows, and rounding
+    the operands to 2^-62 of their maxima leaves sqrt(R) 2^-60 P; against the line that is 2^-49, and the largest of
+    some ten thousand entries may be 6 times the usual one.  Pairs stay within 2^-47 on such columns."""
+    q = 130
+    Z, ZH, ZS = rows_at_the_line(n, q, most, tail, 77)
+    HR, SR = gram(Z, ZH, ZS)
+    iu = np.triu_indices(q - 1)
+    for out, B in ((HR, ZH), (SR, ZS)):
+        mag = np.abs(Z).T @ np.abs(B)
+        rel = (np.abs(out - Z.T @ B) / mag)[iu]
+        assert rel.max() <= 2.0 ** -46, np.log2(rel.max())

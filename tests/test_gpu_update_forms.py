@@ -110,3 +110,23 @@ def test_update_fp64_columns(n, q, k):
     out = t.cpu().numpy()
     assert np.array_equal(out[:, k:], Z[:, k:])
     assert np.all(np.abs(out[:, :k] - Z @ W) <= 2.0 ** -53 * 2 * (q + 2) * (np.abs(Z) @ np.abs(W)))
+
+
+@pytest.mark.parametrize("n,q,k,most", [(12288, 170, 100, 7.2), (6144, 538, 282, 7.6)])
+def test_update_entries_just_above_the_guard(n, q, k, most):
+    """sum |z||w| from 2^2 down to the guard's line, sqrt(q) 2^-11 of the product P of the row's and the column's leading
+    powers of two: one entry of about 1 in each row of Z and each column of W, at indices that do not meet, the
+    others smaller by up to 2^most, half of the rows and columns of one sign.  Bound 2^-46 of |Z| |W|: the sums of the
+    lowest levels are rounded to 2^-56 P once per 256 terms and the operands to 2^-62 of their maxima, 2^-49 of the
+    line, and the largest of a million entries may be 8 times the usual one."""
+    rng = np.random.default_rng(q)
+    m, w = np.exp2(-np.linspace(1.0, most, n)), np.exp2(-np.linspace(1.0, most, k))
+    Z = m[:, None] * rng.uniform(0.5, 1.5, (n, q)) * np.where(np.arange(n) % 2, 1.0, rng.choice([-1.0, 1.0], (q, n))).T
+    W = w * rng.uniform(0.5, 1.5, (q, k)) * np.where(np.arange(k) % 2, 1.0, rng.choice([-1.0, 1.0], (q, k)))
+    Z[:, 0], Z[:, 1] = 1.3, 0.0
+    W[0], W[1] = 0.0, 1.7
+    W[:, 0] = 1.0     # the same scale for every row of W
+    out = update(Z, W)[:, 1:k]
+    exact, mag = (Z @ W)[:, 1:], (np.abs(Z) @ np.abs(W))[:, 1:]
+    rel = (np.abs(out - exact) / mag).max()
+    assert rel <= 2.0 ** -46, np.log2(rel)
