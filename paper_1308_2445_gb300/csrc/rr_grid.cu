@@ -43,7 +43,8 @@ constexpr int RG_TRI_THREADS = 512;
 constexpr size_t RG_SMEM_MAX = 225 * 1024;
 
 // info[3] set: a pivot of S_R failed, nothing below is wanted.  gate (nullable): max |G - I| of the first
-// CholeskyQR pass; the kernels of the second return unless it is needed.
+// CholeskyQR pass; the kernels of the second return unless it is needed.  Every thread may ask for itself, except in
+// k_rg_panel, which sets info[3].
 __device__ __forceinline__ bool rg_stop(const int* info, const unsigned long long* gate) {
     if (__ldcg(info + 3)) return true;
     return gate && !(__longlong_as_double((long long)__ldcg(gate)) > RG_SECOND_PASS);
@@ -73,16 +74,21 @@ __global__ void __launch_bounds__(256) k_rg_scale(const double* __restrict__ S, 
 __global__ void __launch_bounds__(256) k_rg_panel(const double* __restrict__ A, int n, int p0, int clamp,
                                                   double* __restrict__ L, double* __restrict__ LT, double* __restrict__ rl,
                                                   int* __restrict__ info, const unsigned long long* gate) {
-    if (rg_stop(info, gate)) return;
     __shared__ double D[RG_NB][RG_NB + 1], ri[RG_NB];   // D[j][i]: column j of the block's factor
-    __shared__ int s_bad;
+    __shared__ int s_bad, s_stop;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nb = min(RG_NB, n - p0), p1 = p0 + nb;
     // this warp's row is on its way while the block is factored
     const int row = p1 + (int)blockIdx.x * 8 + warp;
     double a = row < n && lane < nb ? A[(int64_t)row * n + p0 + lane] : 0.0;
-    if (tid == 0) s_bad = 0;
+    // one reading for the CTA: another CTA of this launch may set info[3] meanwhile, and warps that left would be
+    // missed at the barriers below
+    if (tid == 0) {
+        s_bad = 0;
+        s_stop = rg_stop(info, gate);
+    }
     __syncthreads();
+    if (s_stop) return;
     if (warp < 4) {
         // columns 4 t + warp in this warp's registers, lane = row; columns and rows beyond nb are those of I
         double r[8];

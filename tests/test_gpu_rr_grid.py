@@ -74,3 +74,20 @@ def test_dependent_columns_reach_the_rank_revealing_branch(q, k, ndep):
     g, _, fb = L.rayleigh_ritz(HR, SR, k)
     assert fb and info[0] == 1 and info[1] == q - ndep
     assert np.abs(th - g).max() <= 1e-8 * np.abs(g).max()
+
+
+@pytest.mark.parametrize("q,first,later", [(260, 5, 120), (150, 31, 40), (400, 1, 399)])
+def test_dependent_columns_in_an_early_panel(q, first, later):
+    """The first failing pivot lies in a panel that many CTAs factor at once: all of them leave it, and the rank-revealing
+    branch takes over."""
+    HR, SR = pencil(q, 10.0, 7 * q)
+    C = np.eye(q)
+    C[:, first] = C[:, 0] if first == 1 else C[:, 2] - 0.5 * C[:, 3]
+    C[:, later] = C[:, 8] + C[:, 9]
+    HR, SR = C.T @ HR @ C, C.T @ SR @ C
+    HR, SR = 0.5 * (HR + HR.T), 0.5 * (SR + SR.T)
+    k = 20
+    th, _, info = run(HR, SR, k)
+    g, _, fb = L.rayleigh_ritz(HR, SR, k)
+    assert fb and info[0] == 1 and info[1] == q - 2
+    assert np.abs(th - g).max() <= 1e-8 * np.abs(g).max()
