@@ -36,8 +36,8 @@
 //
 // Bound: the integer pipe of the slicers (about 30 integer instructions per value and tile it meets; the
 // tensor core waits for them).  n = 334,272, q = 538: 9.9 ms against 40.5 ms for the FP32 pipes;
-// n = 47,620, q = 149: 0.28 against 0.64 ms.  Error against 64 bits on such blocks 5e-16 (q = 538: 1.9e-15, most of it the
-// 64-bit reference's own), float pairs 2e-15.
+// n = 47,620, q = 149: 0.28 against 0.64 ms.  Error against 64 bits on such blocks 5e-16 (q = 538: 1.9e-15),
+// float pairs 2e-15.
 #include <algorithm>
 #include <mutex>
 #include <string>
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
                                                            const int* __restrict__ cexp, const int* __restrict__ sel,
                                                            double* __restrict__ part, int* __restrict__ list) {
     extern __shared__ __align__(1024) uint8_t tg_smem[];
-    __shared__ __align__(8) uint64_t full[TG_NS], empty[TG_NS], phasedone, accfree;
+    __shared__ __align__(8) uint64_t full[TG_NS], empty[TG_NS], phasedone, accfree, drain;
     __shared__ uint32_t tslot;
     __shared__ int s_flag, s_cnt, s_base, s_ent[TG_UNIT_FIX];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -177,6 +177,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
         }
         tc::mbar_init(&phasedone, 1);
         tc::mbar_init(&accfree, TG_ATHREADS / 32);
+        tc::mbar_init(&drain, 1);
         s_flag = 0;
         s_cnt = 0;
     }
@@ -232,6 +233,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
                 if (ok) tc::mma_commit(&phasedone);
             }
             if (!ok) s_flag = 1;
+            tc::mma_drain(&drain, WAIT_NS);
         }
     } else {   // ---- slicers, and (warps 0-7) the reading of the accumulators
         // a thread without a column reads column 0 of its block, with an exponent that shifts it to zero
@@ -252,8 +254,9 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
                 facc[c * TG_M] = 0;
                 if (c < TG_B / 4) flow[c * TG_M] = 0;
             }
-        auto read_phase = [&](int ph) -> bool {
-            if (!tc::mbar_wait(&phasedone, (uint32_t)(ph & 1), WAIT_NS)) return false;
+        auto read_phase = [&](int ph) {
+            tc::warp_wait(&phasedone, (uint32_t)(ph & 1), WAIT_NS, &s_flag);
+            __syncwarp();
             tc::fence_after_sync();
             if (ph == 0) {
                 // the guard sums against the chunk's rows (see the head of the file); a column without
@@ -298,7 +301,6 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
             tc::fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(&accfree);
-            return true;
         };
         // the values and row exponents of the next two steps are on their way while one is sliced
         double x[2][8];
@@ -338,13 +340,12 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
         fetch(1, x[1], e[1]);
         int st = 0, done = 0, ended = 0, since = 0, next_end = nblk;
         uint32_t ph = 1;
-        bool ok = true;
-        auto step = [&](int t, double (&xs)[8], int4 (&es)[2]) -> bool {
+        auto step = [&](int t, double (&xs)[8], int4 (&es)[2]) {
             const int sg = isa ? 1 : -1;
             const int off[8] = {ebase + sg * es[0].x, ebase + sg * es[0].y, ebase + sg * es[0].z, ebase + sg * es[0].w,
                                 ebase + sg * es[1].x, ebase + sg * es[1].y, ebase + sg * es[1].z, ebase + sg * es[1].w};
             // the first pass over the stages finds them empty (parity 1 of a fresh barrier is complete)
-            if (!tc::mbar_wait(&empty[st], ph, WAIT_NS)) return false;
+            tc::warp_wait(&empty[st], ph, WAIT_NS, &s_flag);
             if (t < nblk) slice8_guard(xs, off, base + st * TG_STAGE + soff);
             else slice8(xs, off, base + st * TG_STAGE + soff, stride);
             tc::fence_proxy_async();
@@ -354,28 +355,20 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
             if (++st == TG_NS) { st = 0; ph ^= 1u; }
             if (isa) {
                 ++since;
-                if (done < ended && since >= 2) {
-                    if (!read_phase(done)) return false;
-                    ++done;
-                }
+                if (done < ended && since >= 2) read_phase(done++);
                 if (t + 1 == next_end) {   // a phase's last step
                     ++ended;
                     since = 0;
                     next_end = min(total, next_end + TG_STEPS);
                 }
             }
-            return true;
         };
-        for (int t = 0; ok && t < total; t += 2) {
-            ok = step(t, x[0], e[0]);
-            if (ok && t + 1 < total) ok = step(t + 1, x[1], e[1]);
+        for (int t = 0; t < total; t += 2) {
+            step(t, x[0], e[0]);
+            if (t + 1 < total) step(t + 1, x[1], e[1]);
         }
         if (isa)
-            while (ok && done < ended) {
-                ok = read_phase(done);
-                ++done;
-            }
-        if (!ok) s_flag = 1;
+            while (done < ended) read_phase(done++);
     }
     tc::fence_before_sync();
     __syncthreads();

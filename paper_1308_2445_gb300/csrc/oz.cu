@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_update_oz(OzSeg s0, OzSeg s1,
                                                               double* __restrict__ Y, int64_t ldy,
                                                               int* __restrict__ status) {
     extern __shared__ __align__(1024) uint8_t oz_smem[];
-    __shared__ __align__(8) uint64_t full[OZ_NS], empty[OZ_NS], segdone, accfree;
+    __shared__ __align__(8) uint64_t full[OZ_NS], empty[OZ_NS], segdone, accfree, drain;
     __shared__ uint32_t tslot;
     __shared__ int s_fail;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -156,6 +156,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_update_oz(OzSeg s0, OzSeg s1,
         }
         tc::mbar_init(&segdone, 1);
         tc::mbar_init(&accfree, OZ_SLICERS);
+        tc::mbar_init(&drain, 1);
         s_fail = 0;
     }
     if (warp == 0) tc::tmem_alloc(&tslot, OZ_TMEM_COLS);
@@ -169,13 +170,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_update_oz(OzSeg s0, OzSeg s1,
         if (lane == 0) {
             const uint32_t idesc = tc::idesc_bf16_f32(128, OZ_N);
             uint32_t init_mask = 0;
+            bool ok = true;
             for (int t = 0; t < total; ++t) {
                 const int st = t % OZ_NS;
                 if (t == n0) {   // the slicers have read segment 0's accumulators
-                    if (!tc::mbar_wait(&accfree, 0u, OZ_WAIT_NS)) { s_fail = 1; break; }
+                    ok = tc::mbar_wait(&accfree, 0u, OZ_WAIT_NS);
                     init_mask = 0;
                 }
-                if (!tc::mbar_wait(&full[st], (uint32_t)((t / OZ_NS) & 1), OZ_WAIT_NS)) { s_fail = 1; break; }
+                ok = ok && tc::mbar_wait(&full[st], (uint32_t)((t / OZ_NS) & 1), OZ_WAIT_NS);
+                if (!ok) break;
                 tc::fence_after_sync();
                 uint8_t* stA = base + st * OZ_STAGE;
                 uint8_t* stB = stA + OZ_DIG * OZ_A_SLICE;
@@ -193,6 +196,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_update_oz(OzSeg s0, OzSeg s1,
                 tc::mma_commit(&empty[st]);
                 if (t == n0 - 1 || t == total - 1) tc::mma_commit(&segdone);
             }
+            if (!ok) s_fail = 1;
+            tc::mma_drain(&drain, OZ_WAIT_NS);
         }
     } else {   // ---- slicers and epilogue
         const int arow = tid >> 1, ahalf = tid & 1;
@@ -211,10 +216,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_update_oz(OzSeg s0, OzSeg s1,
             const int kk = (g ? t - n0 : t) * 16;
             uint8_t* stA = base + st * OZ_STAGE;
             uint8_t* stB = stA + OZ_DIG * OZ_A_SLICE;
-            if (t >= OZ_NS && !tc::mbar_wait(&empty[st], (uint32_t)((t / OZ_NS - 1) & 1), OZ_WAIT_NS)) {
-                s_fail = 1;
-                break;
-            }
+            if (t >= OZ_NS) tc::warp_wait(&empty[st], (uint32_t)((t / OZ_NS - 1) & 1), OZ_WAIT_NS, &s_fail);
             {   // A slices: the 8 digits of the thread's 8 entries of its row
                 const int emax_a = agrow < n ? sg.rowexp[agrow] : 0;
                 double x[8];
@@ -251,10 +253,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_update_oz(OzSeg s0, OzSeg s1,
                 // fold the segment in: levels 0-5 are exact multiples of 2^-30 (summed as integers),
                 // the shared 6-8 accumulator is added in FP64; z w = 2^(E_r + E_c - 12) sum_L D_L,
                 // E = exponent field - 1022
-                if (!tc::mbar_wait(&segdone, (uint32_t)(segs & 1), OZ_WAIT_NS)) {
-                    s_fail = 1;
-                    break;
-                }
+                tc::warp_wait(&segdone, (uint32_t)(segs & 1), OZ_WAIT_NS, &s_fail);
+                __syncwarp();
                 tc::fence_after_sync();
                 const int e_row = egrow < n ? sg.rowexp[egrow] : 0;
 #pragma unroll

@@ -85,6 +85,30 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, uint6
     }
 }
 
+// the same for a whole warp, which goes on in step whatever comes: tcgen05.ld and the warp barriers after a wait need all
+// lanes, and a limit that only some of them reached would split the warp for good.  A lane that gives up sets *failed
+// (shared memory), which also ends every later wait of the CTA that has to spin; the caller drops its results.  (A
+// vote after each wait instead: the Gram 1.6% slower; the spin inlined: 1.3%.)
+static __device__ __noinline__ void warp_wait_spin(uint64_t* mbar, uint32_t parity, uint64_t limit_ns, int* failed) {
+    uint64_t t0;
+    asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t0));
+    for (;;) {
+        if (mbar_try_wait(mbar, parity) || *reinterpret_cast<volatile int*>(failed) != 0) return;
+        uint64_t t;
+        asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t));
+        if (t - t0 > limit_ns) *reinterpret_cast<volatile int*>(failed) = 1;
+    }
+}
+__device__ __forceinline__ void warp_wait(uint64_t* mbar, uint32_t parity, uint64_t limit_ns, int* failed) {
+    if (!mbar_try_wait(mbar, parity)) warp_wait_spin(mbar, parity, limit_ns, failed);
+}
+// by the issuing thread, when it is done or has given up: its MMAs end (a fresh mbarrier of one arrival) before the CTA
+// frees tensor memory and leaves its shared memory, whatever the other warps still wait for
+__device__ __forceinline__ void mma_drain(uint64_t* mbar, uint64_t limit_ns) {
+    mma_commit(mbar);
+    (void)mbar_wait(mbar, 0u, limit_ns);
+}
+
 // 32 lanes (this warp's quarter of TMEM) x 16 columns of 32-bit values starting at taddr
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     uint32_t r[16];

@@ -160,6 +160,14 @@ __device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t b
 __device__ __forceinline__ void expect_bytes(uint64_t* full, uint32_t bytes) {   // with this thread's arrival
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(tc::smem_u32(full)), "r"(bytes) : "memory");
 }
+// the first `copies` copies, one after another into NS stages, have landed: the CTA may leave its shared memory
+template <int NS>
+__device__ __forceinline__ void drain_copies(uint64_t (&full)[NS], int copies) {
+    for (int i = 0; i < NS; ++i) {
+        const int c = (copies - i + NS - 1) / NS;   // into stage i
+        if (c > 0) (void)tc::mbar_wait(&full[i], (uint32_t)((c - 1) & 1), WAIT_NS);
+    }
+}
 
 // One CTA: sum|z||w| of 128 rows and all outputs, 32 columns of Z per stage (warps 0-7 the magnitudes of Z, warp
 // 9 those of W, warp 8 the MMAs).  Entries below the line, and those of rows and columns with a non-finite
@@ -170,7 +178,7 @@ __global__ void __launch_bounds__(TU_THREADS, 1) k_tu_guard(Steps S, int64_t rba
                                                             const uint8_t* __restrict__ Wg, const int* __restrict__ rowexp,
                                                             unsigned* __restrict__ list, unsigned cap) {
     extern __shared__ __align__(1024) uint8_t tu_smem[];
-    __shared__ __align__(8) uint64_t full[TU_GUARD_NS], empty[TU_GUARD_NS], done;
+    __shared__ __align__(8) uint64_t full[TU_GUARD_NS], wfull[TU_GUARD_NS], empty[TU_GUARD_NS], done, drain;
     __shared__ uint32_t tslot;
     __shared__ int s_fail;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -178,10 +186,12 @@ __global__ void __launch_bounds__(TU_THREADS, 1) k_tu_guard(Steps S, int64_t rba
     uint8_t* base = tu_smem + ((1024 - (tc::smem_u32(tu_smem) & 1023)) & 1023);
     if (tid == 0) {
         for (int i = 0; i < TU_GUARD_NS; ++i) {
-            tc::mbar_init(&full[i], TU_SLICERS / 32 + 1);
+            tc::mbar_init(&full[i], TU_SLICERS / 32);
+            tc::mbar_init(&wfull[i], 1);
             tc::mbar_init(&empty[i], 1);
         }
         tc::mbar_init(&done, 1);
+        tc::mbar_init(&drain, 1);
         s_fail = 0;
     }
     if (warp == 0) tc::tmem_alloc(&tslot, 512);
@@ -192,17 +202,18 @@ __global__ void __launch_bounds__(TU_THREADS, 1) k_tu_guard(Steps S, int64_t rba
     const int pairs = (S.total + 1) / 2;
     if (warp == 9) {
         if (lane == 0) {
-            int st = 0;
+            int st = 0, p = 0;
             uint32_t ph = 1;
-            for (int p = 0; p < pairs; ++p) {
+            for (; p < pairs; ++p) {
                 if (!tc::mbar_wait(&empty[st], ph, WAIT_NS)) { s_fail = 1; break; }
                 const int nt = min(2, S.total - 2 * p);
-                expect_bytes(&full[st], (uint32_t)(nt * kp64 * 32));
+                expect_bytes(&wfull[st], (uint32_t)(nt * kp64 * 32));
                 for (int h = 0; h < nt; ++h)
                     bulk_copy(base + st * TU_GUARD_STAGE + 2 * A_SLICE + h * UPDATE_TC_MAX_K * 32,
-                              Wg + (int64_t)(2 * p + h) * kp64 * 32, (uint32_t)(kp64 * 32), &full[st]);
+                              Wg + (int64_t)(2 * p + h) * kp64 * 32, (uint32_t)(kp64 * 32), &wfull[st]);
                 if (++st == TU_GUARD_NS) { st = 0; ph ^= 1u; }
             }
+            drain_copies(wfull, p);
         }
     } else if (warp == 8) {
         if (lane == 0) {
@@ -210,7 +221,7 @@ __global__ void __launch_bounds__(TU_THREADS, 1) k_tu_guard(Steps S, int64_t rba
             uint32_t ph = 0;
             bool ok = true;
             for (int p = 0; p < pairs; ++p) {
-                ok = tc::mbar_wait(&full[st], ph, WAIT_NS);
+                ok = tc::mbar_wait(&full[st], ph, WAIT_NS) && tc::mbar_wait(&wfull[st], ph, WAIT_NS);
                 if (!ok) break;
                 tc::fence_after_sync();
                 const int nt = min(2, S.total - 2 * p);
@@ -229,6 +240,7 @@ __global__ void __launch_bounds__(TU_THREADS, 1) k_tu_guard(Steps S, int64_t rba
             }
             if (ok) tc::mma_commit(&done);
             else s_fail = 1;
+            tc::mma_drain(&drain, WAIT_NS);
         }
     } else {
         const int quarter = lane & 3, row8 = warp * 16 + (lane >> 2);
@@ -258,8 +270,8 @@ __global__ void __launch_bounds__(TU_THREADS, 1) k_tu_guard(Steps S, int64_t rba
         fetch(1, x[1], e[1]);
         int st = 0;
         uint32_t ph = 1;
-        auto step = [&](int p, double (&xs)[2][2][4], int4 (&es)[2]) -> bool {
-            if (!tc::mbar_wait(&empty[st], ph, WAIT_NS)) return false;
+        auto step = [&](int p, double (&xs)[2][2][4], int4 (&es)[2]) {
+            tc::warp_wait(&empty[st], ph, WAIT_NS, &s_fail);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 if (2 * p + h >= S.total) break;
@@ -277,41 +289,35 @@ __global__ void __launch_bounds__(TU_THREADS, 1) k_tu_guard(Steps S, int64_t rba
             if (lane == 0) mbar_arrive(&full[st]);
             fetch(p + 2, xs, es);
             if (++st == TU_GUARD_NS) { st = 0; ph ^= 1u; }
-            return true;
         };
-        bool ok = true;
-        for (int p = 0; ok && p < pairs; p += 2) {
-            ok = step(p, x[0], e[0]);
-            if (ok && p + 1 < pairs) ok = step(p + 1, x[1], e[1]);
+        for (int p = 0; p < pairs; p += 2) {
+            step(p, x[0], e[0]);
+            if (p + 1 < pairs) step(p + 1, x[1], e[1]);
         }
-        if (ok) ok = tc::mbar_wait(&done, 0u, WAIT_NS);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) {
-            s_fail = 1;
-        } else {
-            tc::fence_after_sync();
-            const int r = (warp & 3) * 32 + lane;
-            const int er = r0 + r < rows ? rowexp[r0 + r] : (int)0x80808080;
-            const float need = sqrtf((float)(S.q0 + S.q1)) * 0x1p-11f;   // in units of the leading powers of two
-            const bool row_on = er != (int)0x80808080, row_bad = er == BAD_EXP;
-            for (int c0 = (warp >> 2) * 8; c0 < kp64; c0 += 16) {
-                uint32_t v[8];
-                tmem_ld8(tbase + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0, v);
-                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+        tc::warp_wait(&done, 0u, WAIT_NS, &s_fail);
+        __syncwarp();
+        tc::fence_after_sync();
+        const int r = (warp & 3) * 32 + lane;
+        const int er = r0 + r < rows ? rowexp[r0 + r] : (int)0x80808080;
+        const float need = sqrtf((float)(S.q0 + S.q1)) * 0x1p-11f;   // in units of the leading powers of two
+        const bool row_on = er != (int)0x80808080, row_bad = er == BAD_EXP;
+        for (int c0 = (warp >> 2) * 8; c0 < kp64; c0 += 16) {
+            uint32_t v[8];
+            tmem_ld8(tbase + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0, v);
+            asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const int j = c0 + c;
-                    const int w = j < k ? cw[j] : (int)0x80808080;
-                    // a zero row or column gives exact zeros -- unless the other holds a non-finite entry
-                    const bool fail = j < k && r0 + r < rows &&
-                                      (row_bad || w == BAD_EXP || (row_on && w != (int)0x80808080 && !(__uint_as_float(v[c]) >= need)));
-                    const unsigned m = __ballot_sync(0xffffffffu, fail);
-                    if (m) {
-                        unsigned pos = 0;
-                        if (lane == 0) pos = atomicAdd(list, __popc(m));
-                        pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(m & ((1u << lane) - 1u));
-                        if (fail && pos < cap) list[2 + pos] = ((unsigned)(r0 + r) << 16) | (unsigned)j;
-                    }
+            for (int c = 0; c < 8; ++c) {
+                const int j = c0 + c;
+                const int w = j < k ? cw[j] : (int)0x80808080;
+                // a zero row or column gives exact zeros -- unless the other holds a non-finite entry
+                const bool fail = j < k && r0 + r < rows &&
+                                  (row_bad || w == BAD_EXP || (row_on && w != (int)0x80808080 && !(__uint_as_float(v[c]) >= need)));
+                const unsigned m = __ballot_sync(0xffffffffu, fail);
+                if (m) {
+                    unsigned pos = 0;
+                    if (lane == 0) pos = atomicAdd(list, __popc(m));
+                    pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(m & ((1u << lane) - 1u));
+                    if (fail && pos < cap) list[2 + pos] = ((unsigned)(r0 + r) << 16) | (unsigned)j;
                 }
             }
         }
@@ -333,7 +339,7 @@ __global__ void __launch_bounds__(TU_MTHREADS, 1) k_update_tc(Steps S, int64_t r
                                                              const uint8_t* __restrict__ Wsl, const int* __restrict__ rowexp,
                                                              double* __restrict__ Y, unsigned* __restrict__ list, unsigned cap) {
     extern __shared__ __align__(1024) uint8_t tu_smem[];
-    __shared__ __align__(8) uint64_t full[TU_NS], empty[TU_NS], phasedone, accfree;
+    __shared__ __align__(8) uint64_t full[TU_NS], wfull[TU_NS], empty[TU_NS], phasedone, accfree, drain;
     __shared__ uint32_t tslot;
     __shared__ int s_fail;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -345,11 +351,13 @@ __global__ void __launch_bounds__(TU_MTHREADS, 1) k_update_tc(Steps S, int64_t r
     uint8_t* base = tu_smem + ((1024 - (tc::smem_u32(tu_smem) & 1023)) & 1023);
     if (tid == 0) {
         for (int i = 0; i < TU_NS; ++i) {
-            tc::mbar_init(&full[i], 9);
+            tc::mbar_init(&full[i], 8);
+            tc::mbar_init(&wfull[i], 1);
             tc::mbar_init(&empty[i], 1);
         }
         tc::mbar_init(&phasedone, 1);
         tc::mbar_init(&accfree, 8);
+        tc::mbar_init(&drain, 1);
     }
     if (warp == 0) tc::tmem_alloc(&tslot, 512);
     tc::fence_before_sync();
@@ -360,14 +368,15 @@ __global__ void __launch_bounds__(TU_MTHREADS, 1) k_update_tc(Steps S, int64_t r
 
     if (warp == 17) {   // ---- W slices: one bulk copy per step, in the order of the steps
         if (lane == 0) {
-            int st = 0;
+            int st = 0, v = 0;
             uint32_t ph = 1;
-            for (int v = 0; v < all; ++v) {
+            for (; v < all; ++v) {
                 if (!tc::mbar_wait(&empty[st], ph, WAIT_NS)) { s_fail = 1; break; }
-                expect_bytes(&full[st], DIG * B_SLICE);
-                bulk_copy(base + st * TU_STAGE + DIG * A_SLICE, Wsl + (int64_t)v * (DIG * B_SLICE), DIG * B_SLICE, &full[st]);
+                expect_bytes(&wfull[st], DIG * B_SLICE);
+                bulk_copy(base + st * TU_STAGE + DIG * A_SLICE, Wsl + (int64_t)v * (DIG * B_SLICE), DIG * B_SLICE, &wfull[st]);
                 if (++st == TU_NS) { st = 0; ph ^= 1u; }
             }
+            drain_copies(wfull, v);
         }
     } else if (warp == 16) {   // ---- MMA issuer
         if (lane == 0) {
@@ -378,7 +387,7 @@ __global__ void __launch_bounds__(TU_MTHREADS, 1) k_update_tc(Steps S, int64_t r
                 const int steps = min(FLUSH_STEPS, total - (p % nph) * FLUSH_STEPS);
                 if (p > 0) ok = tc::mbar_wait(&accfree, (uint32_t)((p - 1) & 1), WAIT_NS);
                 for (int t = 0; ok && t < steps; ++t) {
-                    ok = tc::mbar_wait(&full[st], ph, WAIT_NS);
+                    ok = tc::mbar_wait(&full[st], ph, WAIT_NS) && tc::mbar_wait(&wfull[st], ph, WAIT_NS);
                     if (!ok) break;
                     tc::fence_after_sync();
                     const uint64_t a = tc::smem_desc(tc::smem_u32(base + st * TU_STAGE), 128, 256);
@@ -398,6 +407,7 @@ __global__ void __launch_bounds__(TU_MTHREADS, 1) k_update_tc(Steps S, int64_t r
                 if (ok) tc::mma_commit(&phasedone);
             }
             if (!ok) s_fail = 1;
+            tc::mma_drain(&drain, WAIT_NS);
         }
     } else if (warp < 8) {   // ---- the accumulators: 32 rows and 32 columns per warp, kept over the phases of a column tile
         const uint32_t taddr = tbase + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * 32);
@@ -406,18 +416,16 @@ __global__ void __launch_bounds__(TU_MTHREADS, 1) k_update_tc(Steps S, int64_t r
         double* o = reinterpret_cast<double*>(base + TU_NS * TU_STAGE) + (int64_t)warp * 32 * TU_OUT_LD;
         // [8][32]: fractions of this row's 32 sums, four columns in a word (in registers they would spill)
         uint32_t* low = reinterpret_cast<uint32_t*>(base + TU_NS * TU_STAGE + 8 * 32 * TU_OUT_LD * 8) + warp * 256 + lane;
-        bool ok = true;
         int p = 0;
-        for (int tile = 0; ok && tile < jt; ++tile) {
+        for (int tile = 0; tile < jt; ++tile) {
             long long acc[32];
 #pragma unroll
             for (int c = 0; c < 32; ++c) acc[c] = 0;
 #pragma unroll
             for (int c = 0; c < 8; ++c) low[32 * c] = 0;
             for (int u = 0; u < nph; ++u, ++p) {
-                ok = tc::mbar_wait(&phasedone, (uint32_t)(p & 1), WAIT_NS);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
+                tc::warp_wait(&phasedone, (uint32_t)(p & 1), WAIT_NS, &s_fail);
+                __syncwarp();
                 tc::fence_after_sync();
 #pragma unroll
                 for (int c0 = 0; c0 < 32; c0 += 4) {
@@ -437,7 +445,6 @@ __global__ void __launch_bounds__(TU_MTHREADS, 1) k_update_tc(Steps S, int64_t r
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&accfree);
             }
-            if (!ok) break;
             // through shared memory, 16 columns of two rows per store
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -456,7 +463,6 @@ __global__ void __launch_bounds__(TU_MTHREADS, 1) k_update_tc(Steps S, int64_t r
                 __syncwarp();
             }
         }
-        if (!ok) s_fail = 1;
     } else {   // ---- slicers: rows row8 and row8 + 8, four columns of each step
         const int quarter = lane & 3, row8 = (warp - 8) * 16 + (lane >> 2);
         bool on[2];
@@ -483,8 +489,8 @@ __global__ void __launch_bounds__(TU_MTHREADS, 1) k_update_tc(Steps S, int64_t r
         fetch(x[1], e[1]);
         int st = 0;
         uint32_t ph = 1;
-        auto step = [&](double (&xs)[2][4], int4& es) -> bool {
-            if (!tc::mbar_wait(&empty[st], ph, WAIT_NS)) return false;
+        auto step = [&](double (&xs)[2][4], int4& es) {
+            tc::warp_wait(&empty[st], ph, WAIT_NS, &s_fail);
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 uint8_t* dst = base + st * TU_STAGE + soff + u * 256;
@@ -512,14 +518,11 @@ __global__ void __launch_bounds__(TU_MTHREADS, 1) k_update_tc(Steps S, int64_t r
             if (lane == 0) mbar_arrive(&full[st]);
             fetch(xs, es);
             if (++st == TU_NS) { st = 0; ph ^= 1u; }
-            return true;
         };
-        bool ok = true;
-        for (int v = 0; ok && v < all; v += 2) {
-            ok = step(x[0], e[0]);
-            if (ok && v + 1 < all) ok = step(x[1], e[1]);
+        for (int v = 0; v < all; v += 2) {
+            step(x[0], e[0]);
+            if (v + 1 < all) step(x[1], e[1]);
         }
-        if (!ok) s_fail = 1;
     }
     tc::fence_before_sync();
     __syncthreads();
