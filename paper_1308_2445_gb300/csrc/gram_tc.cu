@@ -69,6 +69,14 @@ constexpr size_t TG_SMEM = (size_t)TG_NS * TG_STAGE + (size_t)TG_ACC * 9 + 1024;
 constexpr int TG_UNIT_FIX = 256;                // failing entries of a unit that are computed one by one
 constexpr int TG_EXP_ROWS = 32;                 // rows per CTA of the exponent pass
 
+// a failing entry on the list: its unit (any int), matrix (0: ZH, 1: ZS), columns b and a of the tile
+__host__ __device__ constexpr long long tg_entry(int unit, int m, int cb, int ca) {
+    return ((long long)unit << 13) | (m << 12) | (cb << 7) | ca;
+}
+__host__ __device__ constexpr int tg_entry_unit(long long e) { return (int)(e >> 13); }
+static_assert(tg_entry_unit(tg_entry(0x7FFFFFFF, 1, TG_B - 1, TG_M - 1)) == 0x7FFFFFFF && tg_entry(1 << 18, 0, 0, 0) > 0,
+              "an entry holds every unit");
+
 // rexp[i] = exponent field of max_a |Z(i, a)|; cexp[chunk][0][c] = max over the chunk's rows of the
 // exponent field of Z(i, c) minus rexp[i]; cexp[chunk][1..2][c] the same of ZH, ZS plus rexp[i] (memset
 // below every real value before); sel[g] = the row of group g (16 rows) with the largest scaled ZH entry, by
@@ -148,12 +156,12 @@ __device__ __forceinline__ void tg_pair(int p, int nb, int& ta, int& tb) {
 // stage s, empty[s] when the MMAs that read it are done, phasedone when a phase's MMAs are done, accfree
 // when its accumulators have been read.  The reading of a phase waits until the slicers are two steps into
 // the next one, so that the MMAs find filled stages afterwards.  list[0] counts the units left to k_gram_tc_fixup
-// (a wait that gives up leaves its unit there too) and list[1] the single entries: units from list[2] on,
-// entries (unit << 13 | matrix << 12 | column b << 7 | column a) from list[2 + units] on.
+// (a wait that gives up leaves its unit there too; units from list[2] on) and list[1] the single entries, in ents.
 __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Seg2d ZS, int q, int64_t n,
                                                            int64_t chunk_rows, int nb, const int* __restrict__ rexp,
                                                            const int* __restrict__ cexp, const int* __restrict__ sel,
-                                                           double* __restrict__ part, int* __restrict__ list) {
+                                                           double* __restrict__ part, long long* __restrict__ ents,
+                                                           int* __restrict__ list) {
     extern __shared__ __align__(1024) uint8_t tg_smem[];
     __shared__ __align__(8) uint64_t full[TG_NS], empty[TG_NS], phasedone, accfree, drain;
     __shared__ uint32_t tslot;
@@ -382,8 +390,8 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
     if (nfix > 0) {
         if (tid == 0) s_base = atomicAdd(list + 1, nfix);
         __syncthreads();
-        int* ents = list + 2 + gridDim.x * gridDim.y + s_base;
-        for (int t = tid; t < nfix; t += TG_THREADS) ents[t] = (unit << 13) | s_ent[t];
+        for (int t = tid; t < nfix; t += TG_THREADS)
+            ents[s_base + t] = tg_entry(unit, s_ent[t] >> 12, (s_ent[t] >> 7) & (TG_B - 1), s_ent[t] & (TG_M - 1));
     }
     double* out = part + (int64_t)unit * TG_ACC;
     for (int t = tid; t < TG_ACC; t += TG_THREADS) {
@@ -394,8 +402,8 @@ __global__ void __launch_bounds__(TG_THREADS, 1) k_gram_tc(Seg2d Z, Seg2d ZH, Se
 
 // The listed units in double-float, four 32 x 32 tiles each, and the listed entries in FP64, one CTA each
 __global__ void __launch_bounds__(GTHREADS, GCTAS) k_gram_tc_fixup(Seg2d Z, Seg2d ZH, Seg2d ZS, int q, int64_t n,
-                                                                   int64_t chunk_rows, int nb, int npair, int units,
-                                                                   df::f32x2 nz, double* __restrict__ part,
+                                                                   int64_t chunk_rows, int nb, int npair, df::f32x2 nz,
+                                                                   double* __restrict__ part, const long long* __restrict__ ents,
                                                                    const int* __restrict__ list) {
     __shared__ GramTile sm;
     const int cnt = list[0], nent = list[1];
@@ -414,7 +422,8 @@ __global__ void __launch_bounds__(GTHREADS, GCTAS) k_gram_tc_fixup(Seg2d Z, Seg2
     }
     double* red = &sm.acc[0][0];
     for (int w = blockIdx.x; w < nent; w += gridDim.x) {
-        const int code = list[2 + units + w], unit = code >> 13, m = (code >> 12) & 1;
+        const long long ent = ents[w];
+        const int unit = tg_entry_unit(ent), code = (int)ent, m = (code >> 12) & 1;
         const int chunk = unit / npair;
         int ta, tb;
         tg_pair(unit - chunk * npair, nb, ta, tb);
@@ -494,11 +503,12 @@ int gram2_tc(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1
     const int nch = ceil_div(n, chunk_rows);
     const int64_t units = (int64_t)nch * npair;
     const int64_t rpad = round_up(n, TG_BLK);
-    // workspace: sums | row exponents | column exponents | guard rows | lists
-    const size_t ints = (size_t)rpad + (size_t)nch * 3 * q + (size_t)rpad / 16 + 2 + (size_t)units * (1 + TG_UNIT_FIX);
-    HBSD_TRY(s->ws.alloc((size_t)units * TG_ACC + ints / 2 + 64));
+    // workspace: sums | listed entries | row exponents | column exponents | guard rows | listed units
+    const size_t ints = (size_t)rpad + (size_t)nch * 3 * q + (size_t)rpad / 16 + 2 + (size_t)units;
+    HBSD_TRY(s->ws.alloc((size_t)units * (TG_ACC + TG_UNIT_FIX) + ints / 2 + 64));
     double* part = s->ws.p;
-    int* rexp = reinterpret_cast<int*>(part + units * TG_ACC);   // 16-byte aligned: TG_ACC is even
+    long long* ents = reinterpret_cast<long long*>(part + units * TG_ACC);
+    int* rexp = reinterpret_cast<int*>(ents + units * TG_UNIT_FIX);   // 16-byte aligned: both strides are even
     int* cexp = rexp + rpad;
     int* sel = cexp + (size_t)nch * 3 * q;
     int* list = sel + rpad / 16;
@@ -513,9 +523,10 @@ int gram2_tc(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1
     Seg2d Z{Z0, ld0, q0, Z1, ld1}, ZH{H0, ldh0, q0, H1, ldh1}, ZS{S0, lds0, q0, S1, lds1};
     k_gram_tc_exps<<<ceil_div(n, TG_EXP_ROWS), 256, 0, st>>>(Z, ZH, ZS, q, n, chunk_rows, rexp, cexp, sel);
     HBSD_LAUNCHED(s);
-    k_gram_tc<<<dim3(npair, nch), TG_THREADS, TG_SMEM, st>>>(Z, ZH, ZS, q, n, chunk_rows, nb, rexp, cexp, sel, part, list);
+    k_gram_tc<<<dim3(npair, nch), TG_THREADS, TG_SMEM, st>>>(Z, ZH, ZS, q, n, chunk_rows, nb, rexp, cexp, sel, part, ents,
+                                                              list);
     HBSD_LAUNCHED(s);
-    k_gram_tc_fixup<<<152 * GCTAS, GTHREADS, 0, st>>>(Z, ZH, ZS, q, n, chunk_rows, nb, npair, (int)units, df::NEG_ZERO2, part,
+    k_gram_tc_fixup<<<152 * GCTAS, GTHREADS, 0, st>>>(Z, ZH, ZS, q, n, chunk_rows, nb, npair, df::NEG_ZERO2, part, ents,
                                                       list);
     HBSD_LAUNCHED(s);
     k_gram_tc_final<<<ceil_div((int64_t)q * q, 32), 256, 0, st>>>(part, nch, npair, nb, q, HR, SR);
