@@ -10,6 +10,7 @@
 #include <mutex>
 
 #include "common.h"
+#include "rr_math.h"
 
 namespace hbsd {
 
@@ -524,13 +525,13 @@ __device__ double block_sum(double v, double* red) {
 __device__ void tridiagonalize(double* A, int nn, int lda, double* Q, double* d, double* e,
                                double* tau, double* pv, double* red) {
     for (int kk = 0; kk + 2 < nn; ++kk) {
-        double s2 = 0.0;
-        for (int i = kk + 1 + threadIdx.x; i < nn; i += blockDim.x) s2 += A[(int64_t)i * lda + kk] * A[(int64_t)i * lda + kk];
-        s2 = block_sum(s2, red);
+        double tail = 0.0;   // without x0: see rr_grid.cu
+        for (int i = kk + 2 + threadIdx.x; i < nn; i += blockDim.x) tail += A[(int64_t)i * lda + kk] * A[(int64_t)i * lda + kk];
+        tail = block_sum(tail, red);
         const double x0 = A[(int64_t)(kk + 1) * lda + kk];
-        const double tail = s2 - x0 * x0;
+        const double s2 = tail + x0 * x0;
         if (threadIdx.x == 0) d[kk] = A[(int64_t)kk * lda + kk];
-        if (tail <= 0.0 || s2 == 0.0) {
+        if (tail < rrm::RR_TAIL_MIN) {
             if (threadIdx.x == 0) { e[kk] = x0; tau[kk] = 0.0; }
             for (int i = kk + 1 + threadIdx.x; i < nn; i += blockDim.x) A[(int64_t)i * lda + kk] = 0.0;
             __syncthreads();

@@ -364,13 +364,12 @@ __global__ void __launch_bounds__(RR_THREADS_C, 1)
         double* vbk = vb2 + (kk & 1) * (q + 1);
         const double* row = A + (int64_t)(kk - r0) * q;
         if (warp == 0) {
-            double s2 = 0.0;
-            for (int j = kk + 1 + lane; j < q; j += 32) s2 = fma(row[j], row[j], s2);
-            s2 = wsum(s2);
-            const double x0 = row[kk + 1];
-            const double tail = s2 - x0 * x0;
+            double tail = 0.0;   // without x0: see rr_grid.cu
+            for (int j = kk + 2 + lane; j < q; j += 32) tail = fma(row[j], row[j], tail);
+            tail = wsum(tail);
+            const double x0 = row[kk + 1], s2 = fma(x0, x0, tail);
             double alpha, t;
-            if (tail <= 0.0 || s2 == 0.0) {
+            if (tail < RR_TAIL_MIN) {
                 alpha = x0;
                 t = 0.0;
             } else {

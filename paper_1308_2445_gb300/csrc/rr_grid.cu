@@ -279,13 +279,15 @@ __global__ void __launch_bounds__(RG_TRI_THREADS, 1) k_rg_tridiag(const double* 
     // reflector of row i from its entries rb[i ..] (warps 0-3 of every CTA); rank 0 records it
     auto make_v = [&](int i) {
         double* vb = vb2 + (i & 1) * (q + 1);
-        double s2 = 0.0;
-        for (int j = i + tid; j < q; j += 128) s2 = fma(j > i ? rb[j] : 0.0, rb[j], s2);
-        s2 = sum4(s2);
+        // the squares behind x0 on their own: taken from the whole sum by subtraction, entries below 1e-8 |x0| would
+        // be lost, and dropped from T instead of eliminated
+        double tail = 0.0;
+        for (int j = i + tid; j < q; j += 128) tail = fma(j > i + 1 ? rb[j] : 0.0, rb[j], tail);
+        tail = sum4(tail);
         const double x0 = rb[i + 1];   // thread 1's entry: visible after sum4's barriers
-        const double tail = fma(-x0, x0, s2);
+        const double s2 = fma(x0, x0, tail);
         double alpha = x0, t = 0.0;
-        if ((long long)__double_as_longlong(tail) > 0) {   // tail > 0
+        if (mag(tail) >= mag(RR_TAIL_MIN)) {   // NaN too
             alpha = -copysign(s2 * rsqrt(s2), x0);
             t = rcp64(fma(-alpha, x0, s2));   // 2 / v^T v with v^T v = 2 (s2 - alpha x0)
         }

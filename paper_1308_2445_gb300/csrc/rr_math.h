@@ -16,6 +16,9 @@ __device__ __forceinline__ double wsum(double v) {
     return v;
 }
 
+// Squares of a reflector's entries below this are zero: their reciprocal would not be finite.
+constexpr double RR_TAIL_MIN = 0x1p-1000;
+
 // magnitude of a double as an integer that orders like it
 __device__ __forceinline__ unsigned long long mag(double x) {
     return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;

@@ -91,3 +91,51 @@ def test_dependent_columns_in_an_early_panel(q, first, later):
     g, _, fb = L.rayleigh_ritz(HR, SR, k)
     assert fb and info[0] == 1 and info[1] == q - 2
     assert np.abs(th - g).max() <= 1e-8 * np.abs(g).max()
+
+
+@pytest.mark.parametrize("q,small,dep", [(12, 5e-9, 0), (20, 3e-9, 0), (40, 1e-9, 0), (150, 5e-10, 0), (40, 1e-9, 1)])
+def test_nearly_tridiagonal(q, small, dep):
+    """A nearly tridiagonal pencil: what lies outside the three diagonals is below 1e-8 of a row's largest entry, and has
+    to be eliminated, not dropped.  The vectors diagonalise H_R and S_R to the rounding of a few hundred FP64
+    operations (1e-12 of the largest entry).  S_R = I; dep: nearly tridiagonal as well, with one column twice, which the
+    rank-revealing kernel reduces first."""
+    rng = np.random.default_rng(q)
+
+    def matrix(off, diag):
+        A = np.triu(small * rng.uniform(0.5, 1.0, (q, q)), 2) + np.diag(np.full(q - 1, off), 1)
+        return A + A.T + np.diag(diag)
+
+    H, S, C = matrix(1.0, np.arange(q) / 4.0), np.eye(q), np.eye(q)
+    if dep:
+        S, C = matrix(0.3, np.ones(q)), np.hstack([C, C[:, -1:]])
+    k = q // 2
+    th, W, info = run(C.T @ H @ C, C.T @ S @ C, k)
+    scale = np.abs(np.linalg.eigvalsh(H)).max()
+    assert info[0] == dep and info[1] == q
+    Li = np.linalg.inv(np.linalg.cholesky(S))
+    g = np.linalg.eigvalsh(Li @ H @ Li.T)[:k]
+    V = C @ W
+    assert np.abs(th - g).max() <= 1e-12 * scale
+    assert np.abs(V.T @ S @ V - np.eye(k)).max() <= 1e-12
+    assert np.abs(V.T @ H @ V - np.diag(th)).max() <= 1e-12 * scale
+    assert np.abs(H @ V - S @ V * th).max() <= 1e-12 * scale
+
+
+def test_entries_too_small_to_square():
+    """Rows whose remaining entries have squares below the normal range, and a NaN among them: zeros to the first, and the
+    second is not lost (the call must not return finite pairs)."""
+    q = 40
+    H = np.diag(np.arange(q) / 4.0) + np.diag(np.ones(q - 1), 1) + np.diag(np.ones(q - 1), -1)
+    tiny = np.triu(np.full((q, q), 1e-160), 2)
+    th, W, _ = run(H + tiny + tiny.T, np.eye(q), 10)
+    assert np.abs(th - np.linalg.eigvalsh(H)[:10]).max() <= 1e-12 * 11
+    assert np.abs(W.T @ W - np.eye(10)).max() <= 1e-12
+    th, W, _ = run(np.diag(np.arange(q) / 4.0) + tiny + tiny.T, np.eye(q), 10)   # x0 = 0 as well
+    assert np.abs(th - np.arange(10) / 4.0).max() <= 1e-12 * 11
+    H[20, 30] = H[30, 20] = np.nan
+    from paper_1308_2445_gb300 import hbsd
+    try:
+        th, W, _ = run(H, np.eye(q), 10)
+    except hbsd.HbsdError:
+        return
+    assert not (np.isfinite(th).all() and np.isfinite(W).all())
