@@ -229,6 +229,7 @@ int gram_skew(Session* s, const double* Z, int64_t ldz, const double* V1, int64_
               int64_t ldv2, int64_t n, int q, double* A1, double* A2, cudaStream_t st);
 // largest q the allocation-free Gram's static scratch holds (2 q^2 doubles per row chunk, 2^21 in all)
 constexpr int GRAM_NOALLOC_MAX_Q = 1024;
+size_t gram_scratch_doubles(int q);   // that gram2 needs at most for q columns, whatever the rows (dense.cu)
 int gram_noalloc(const double* Z, int64_t ldz, const double* ZH, int64_t ldzh, const double* ZS, int64_t ldzs,
                  int64_t n, int q, double* HR, double* SR, cudaStream_t st);
 template <class T>

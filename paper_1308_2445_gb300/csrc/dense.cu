@@ -288,6 +288,7 @@ __global__ void __launch_bounds__(64) k_gram_partial24(Seg2<T> Z, Seg2<T> ZH, Se
 // the width decides by padding: 24 x 24 tiles where they leave a tenth less than 32 x 32 ones -- q = 71, n = 20,613:
 // 405 us against 764; q = 35: 211 against 396.  Chunks of at least 32 rows, enough for 8 (16) CTAs per SM: with
 // 128 rows or more, q = 64 of 646 rows took 84 us, now 31.
+constexpr int GRAM_CTAS24 = 2432, GRAM_CTAS32 = 1216;
 struct GramPlan {
     int w, tiles, nch;
     int64_t rpc;
@@ -297,12 +298,20 @@ static GramPlan gram_plan(int64_t n, int q, size_t most) {
     const int64_t w24 = (int64_t)ceil_div(q, 24) * 24, w32 = (int64_t)ceil_div(q, 32) * 32;
     g.w = 11 * w24 * w24 < 10 * w32 * w32 ? 24 : 32;
     g.tiles = ceil_div(q, g.w);
-    int64_t nch = std::max<int64_t>(1, std::min<int64_t>((n + 31) / 32, ceil_div(g.w == 24 ? 2432 : 1216, g.tiles * g.tiles)));
+    int64_t nch = std::max<int64_t>(1, std::min<int64_t>((n + 31) / 32, ceil_div(g.w == 24 ? GRAM_CTAS24 : GRAM_CTAS32, g.tiles * g.tiles)));
     nch = std::min<int64_t>(nch, (int64_t)most);
     g.rpc = (n + nch - 1) / nch;
     if (g.w == 32) g.rpc = round_up(g.rpc, 32);   // that kernel works in whole row tiles
     g.nch = (int)((n + g.rpc - 1) / g.rpc);
     return g;
+}
+// Scratch that holds the partial sums of any number of rows: chunks x 2 q^2, with at most GRAM_CTAS / tiles^2 + 1 chunks
+// and q at most tiles times the tile width.  By 32-column steps of the width, so that a call of another width of as
+// many steps, or fewer, finds it large enough: a caller that made one call may capture such calls into a graph.
+size_t gram_scratch_doubles(int q) {
+    static_assert(24 * 24 * GRAM_CTAS24 >= 32 * 32 * GRAM_CTAS32, "the larger of the two plans");
+    const size_t w = (size_t)round_up(q, 32);
+    return 2 * ((size_t)24 * 24 * GRAM_CTAS24 + w * w) + 64;
 }
 template <class T>
 static void gram_partials(const GramPlan& g, Seg2<T> Z, Seg2<T> ZH, Seg2<T> ZS, int q, int64_t n, double* partial, cudaStream_t st) {

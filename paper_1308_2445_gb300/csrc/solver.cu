@@ -1129,8 +1129,7 @@ int hbsd_gram(const double* Z, int64_t ldz, const double* ZH, int64_t ldzh, cons
         if (!Z || !ZH || !ZS || !HR || !SR || n <= 0 || q <= 0) return fail(HBSD_ERR_ARG, "bad arguments");
         if (!ld_ok(ldz, q) || !ld_ok(ldzh, q) || !ld_ok(ldzs, q)) return fail(HBSD_ERR_ARG, "leading dimension below the block width");
         Session* S = scratch_session();
-        const int tiles = ceil_div(q, 32);
-        HBSD_TRY(S->ws.alloc((size_t)2 * 1024 * (1216 + tiles * tiles) + 1024));
+        HBSD_TRY(S->ws.alloc(gram_scratch_doubles(q)));
         return gram2<double>(S, Z, ldz, q, nullptr, 0, 0, ZH, ldzh, nullptr, 0, ZS, ldzs, nullptr, 0, n, HR, SR,
                              (cudaStream_t)stream);
     });

@@ -162,3 +162,36 @@ def test_gram_tensor_core_entries_just_above_the_guard(n, most, tail):
         mag = np.abs(Z).T @ np.abs(B)
         rel = (np.abs(out - Z.T @ B) / mag)[iu]
         assert rel.max() <= 2.0 ** -46, np.log2(rel.max())
+
+
+def test_gram_scratch_covers_every_row_count():
+    """hbsd_gram's scratch depends on the width alone: after one call of a few rows, calls of any height at
+    widths of as many 32-column tiles can be captured (nothing is allocated)."""
+    import threading
+    from paper_1308_2445_gb300 import hbsd
+    errors = []
+
+    def work():   # a thread of its own: the scratch of these calls is kept per thread
+        try:
+            side = torch.cuda.Stream()
+            with torch.cuda.stream(side):
+                for q in (24, 72, 144, 358):
+                    dev = lambda n: torch.randn(n, q, dtype=torch.float64, device="cuda")
+                    HR, SR = (torch.zeros(q, q, dtype=torch.float64, device="cuda") for _ in range(2))
+                    small, Z = dev(64), dev(90000 if q < 300 else 20000)
+                    hbsd.gram(small, small, small, HR, SR, stream=side.cuda_stream)
+                    side.synchronize()
+                    g = torch.cuda.CUDAGraph()
+                    with torch.cuda.graph(g, stream=side):
+                        hbsd.gram(Z, Z, Z, HR, SR, stream=side.cuda_stream)
+                    g.replay()
+                    side.synchronize()
+                    exact = Z.T @ Z
+                    assert (HR - exact).abs().max() <= 1e-12 * exact.abs().max()
+        except Exception as e:   # noqa: BLE001 - handed to the test
+            errors.append(e)
+
+    t = threading.Thread(target=work)
+    t.start()
+    t.join()
+    assert not errors, errors[0]
