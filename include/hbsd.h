@@ -482,9 +482,10 @@ void hbsd_server_destroy(hbsd_server* sv);
  * Autotuner: for one session and block width w, times the candidate launch shapes of the two
  * steps whose best shape depends on the problem's size, on seeded data on the session's stream,
  * and keeps the fastest for the session's later solves:
- *   - the fused SpMM of steps 3/7 (in the session's precision form; w columns): the most lanes
- *     per matrix row, 4, 8, 16 or 32 (fewer lanes per row put more rows in a CTA and take more
- *     passes over the columns; double-float products use at most 4 whatever the limit);
+ *   - the fused SpMM of steps 3/7 (the FP64 product, w columns): the most lanes per matrix row, 4, 8,
+ *     16 or 32 (fewer lanes per row put more rows in a CTA and take more passes over the columns).  The
+ *     limit holds for FP64 and FP32 products, in the mixed form the convergence checks among them;
+ *     double-float products use at most 4 lanes whatever the limit;
  *   - the cooperative MINRES launch of step 6(b) (min(w, 32) columns, 10 steps): its CTA count,
  *     the whole GPU or 1/2 ... 1/32 of it; the smallest count within 10% of the fastest is kept
  *     (cheaper grid barriers, and SMs left to the other sessions of a batch).

@@ -104,19 +104,19 @@ int autotune(Session* s, int width, hbsd_tune* out) {
         k_tune_fill<<<1024, 256, 0, st>>>(X.p, n * ld, 0x5EEDull);
         HBSD_CUDA(cudaGetLastError());
         HBSD_CUDA(cudaMemsetAsync(e.p, 0, 64 * sizeof(double), st));
-        const bool df = s->opt.precision == HBSD_PRECISION_MIXED && s->opt_df64 && s->opt.spmm_df64 && s->A.hsdf.p;
         const int saved_lpr = s->tune_spmm_lpr, saved_grid = s->tune_mr_grid;
-        // 1. fused SpMM: most lanes per row
+        // 1. fused SpMM: most lanes per row.  Of the FP64 product, in the mixed form too: the limit binds it and the FP32
+        // one, while the double-float product has lanes of its own.  (Timed with that one, the four candidates were
+        // the same launch, and noise or the order chose for the FP64 products.  85 columns with 4, 8, 16 and 32 lanes:
+        // 82, 82, 74, 76 us on the 16^3 problem, 918, 930, 981, 984 on the 32^3 one.)
         static const int lanes[4] = {4, 8, 16, 32};
         double best = 1e300;
         int best_l = 32;
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 3; c >= 0; --c) {
             s->tune_spmm_lpr = lanes[c];
             double ms = 0.0;
-            int rc = time_best(st, 3, &ms, [&]() -> int {
-                return df ? spmm_pair_df64(s, s->A, X.p, ld, w, Y0.p, ld, Y1.p, ld, st)
-                          : spmm_pair<double>(s, s->A, X.p, ld, w, Y0.p, ld, Y1.p, ld, st);
-            });
+            int rc = time_best(st, 3, &ms,
+                               [&]() -> int { return spmm_pair<double>(s, s->A, X.p, ld, w, Y0.p, ld, Y1.p, ld, st); });
             if (rc) {
                 s->tune_spmm_lpr = saved_lpr;
                 return rc;

@@ -5,6 +5,8 @@ deterministic, and tuning fixes a session's launch shapes before its solves, so 
 batch must equal, bit for bit, the same tuned session solved alone; one instance is also checked
 against the FP64 oracle at the solver's bar (|dlambda| <= 1e-9 max|lambda|, angles at the gaps).
 """
+import time
+
 import numpy as np
 import pytest
 
@@ -190,3 +192,29 @@ def test_mixed_form_escalates_a_stalled_solve_to_fp64_and_converges():
     H, S = p.scipy_pair()
     R = (H - sm.sigma0 * S) @ X - (S @ X) * (lam_m - sm.sigma0)[None, :]
     assert (np.linalg.norm(R, axis=0) / np.linalg.norm((H - sm.sigma0 * S) @ X, axis=0)).max() <= 1e-8 * 1.001
+
+
+def test_tuned_lanes_do_not_slow_the_products_they_limit():
+    """The tuner's lane limit binds the FP64 product, also of a mixed session (its convergence checks): with the limit it is
+    no slower than without, to 8% of timing noise."""
+    p = pi.generate(16, 6, 2, 0.15, 1)
+    w = 85
+    X = torch.randn(p.n, 86, dtype=torch.float64, device="cuda")[:, :w]
+    Y = [torch.zeros(p.n, 86, dtype=torch.float64, device="cuda")[:, :w] for _ in range(2)]
+
+    def best(s):
+        out = []
+        for _ in range(12):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            for _ in range(50):
+                s.spmm_pair(X, *Y)
+            torch.cuda.synchronize()
+            out.append(time.perf_counter() - t0)
+        return min(out)
+
+    s = hb().Session.from_problem(p, precision=hb().PRECISION_MIXED)
+    before = best(s)
+    s.autotune(77)   # 77 + 8 columns
+    assert best(s) <= 1.08 * before
+    s.close()
