@@ -539,13 +539,14 @@ int hbsd_solve_batch(hbsd_batch_item* items, int count, const hbsd_batch_opts* o
 
 /* Double-float forms of hbsd_gram and hbsd_update, the ones the mixed form (HBSD_PRECISION_MIXED)
  * runs: FP64 inputs and outputs, products and short sums in pairs of floats (about 48 bits per
- * term, TwoProd / TwoSum), the Gram sums accumulated in FP64 every 64 rows.  From n q^2 = 8e7 on the
- * Gram runs on the tensor cores from exact 8-bit digits of the operands instead (62 bits against each
- * column's largest entry in a few thousand rows), and entries whose sum |z||h| is far below the product of
- * their columns' maxima are computed in FP64 or in pairs.  The others carry about 48 bits of sum |z||h| as
- * well, as long as the roundings of different rows are not all the same (columns that repeat one
- * value from row to row beside a much larger entry elsewhere: 41 bits at worst).  So does the update from n q k = 2e8 on when
- * n >= 6144, 56 <= k <= 512, Z is 16-byte aligned and ldz even.  hbsd_gram_df64
+ * term, TwoProd / TwoSum), the Gram sums accumulated in FP64 every 64 rows.  From q = 48 and n q^2 = 8e7 on
+ * the Gram runs on the tensor cores instead, from exact 8-bit digits of the operands (62 bits against each
+ * column's largest entry in a few thousand rows); entries whose sum |z||h| is far below the product of their
+ * columns' maxima are computed in FP64 or in pairs.  The others carry about 48 bits of sum |z||h| as
+ * well, as long as the roundings of different rows are not all the same (columns that repeat one value from
+ * row to row beside a much larger entry elsewhere: 41 bits at worst).  So does the update of n >= 6144
+ * rows and 56 <= k <= 512 columns from n q k = 2e8 and q k = 7200 on, where that is the faster form (below q k =
+ * 12000 not at every n), if Z is 16-byte aligned and ldz even.  hbsd_gram_df64
  * computes the entries a <= b of Z^T ZH and Z^T ZS and mirrors them (no averaging).  Arguments,
  * layouts and errors as hbsd_gram / hbsd_update; FP64 values enter the products with ~47 bits
  * above 2^-96 in magnitude, at least 24 bits down to 2^-126, and as zero below.  hbsd_update_df64

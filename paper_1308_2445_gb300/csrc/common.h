@@ -250,6 +250,7 @@ int update2_df64(Session* s, double* Z0, int64_t ld0, int q0, const double* Z1, 
 // the update on the tensor cores by exact digit slices, at least as accurate (update_tc.cu): in place, 16-byte
 // aligned blocks with even leading dimensions, k <= UPDATE_TC_MAX_K
 constexpr int UPDATE_TC_MAX_K = 512;
+constexpr int64_t UPDATE_TC_WAVE = 152 * 128;   // rows of one tile per SM
 bool update_tc_fits(const double* Z0, int64_t ld0, const double* Z1, int64_t ld1, int q1, int k);
 int update2_tc(Session* s, double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, int64_t n, const double* W,
                int k, cudaStream_t st);

@@ -8,6 +8,8 @@
 // carry FP64 accuracy.  Large products run on the tensor cores instead (gram_tc.cu, update_tc.cu).
 //
 // The pair arithmetic (split, TwoProd + TwoSum, renormalisation) is in df64.h.
+#include <algorithm>
+#include <cmath>
 #include <mutex>
 
 #include "common.h"
@@ -225,10 +227,12 @@ int gram2_df64(Session* s, const double* Z0, int64_t ld0, int q0, const double* 
     const int q = q0 + q1;
     if (q <= 0) return 0;
     // Tensor cores from n q^2 = 8e7 on: below it the exponent pass, the lists and the fix-up launch (50 us at
-    // the least) outweigh the products.  Measured on both sides, us (this kernel / tensor cores): q = 71,
-    // n = 6,000: 51 / 59, n = 20,000: 125 / 89; q = 149, n = 2,000: 51 / 61, n = 6,000: 103 / 65; q = 19,
-    // n = 150,000: 145 / 202; q = 35, n = 150,000: 344 / 323; q = 538, n = 646: 121 / 95.
-    if ((double)n * q * q >= 8e7)
+    // the least) outweigh the products.  Not below 48 columns, whatever the rows: a tile of 128 x (32 + 32) columns is
+    // then mostly padding.  Measured on both sides, us (this kernel / tensor cores): q = 71, n = 5,951: 57 / 69,
+    // n = 15,869: 108 / 92; q = 149, n = 2,252: 57 / 72, n = 5,855: 108 / 75; q = 538, n = 449: 101 / 105, n = 1,036:
+    // 177 / 142; q = 48, n = 34,722: 115 / 101, n = 434,027: 1,007 / 884; q = 40, n = 81,250: 194 / 196, n = 625,000:
+    // 1,116 / 1,264; q = 33, n = 275,482: 564 / 580; q = 24, n = 225,694: 249 / 336; q = 19, n = 360,110: 406 / 515.
+    if (q >= 48 && (double)n * q * q >= 8e7)
         return gram2_tc(s, Z0, ld0, q0, Z1, ld1, q1, H0, ldh0, H1, ldh1, S0, lds0, S1, lds1, n, HR, SR, st);
     // tiles of equal width, a multiple of 4 columns up to GW
     const int ntile = ceil_div(q, GW);
@@ -248,15 +252,25 @@ int gram2_df64(Session* s, const double* Z0, int64_t ld0, int q0, const double* 
     return 0;
 }
 
+// The update on the tensor cores where it is the faster one.  Otherwise one CTA's chain of column tiles and the passes
+// over Z for exponents and guard cost more than they save; and a wave of row tiles costs the same however few rows are in
+// it, so that blocks of q k < 12000 have to fill theirs (fill) or to be large.  us (pairs / digit slices; n, q, k) below
+// the line: 4728, 282, 150: 129 / 172; 3295, 538, 282: 293 / 341; 21701, 128, 72: 123 / 144; 41700, 100, 72: 173 / 184;
+// 59000, 96, 84: 255 / 271; 318877, 56, 56: 534 / 756; 233100, 66, 65: 587 / 700; 178571, 80, 70: 541 / 600; 162760, 96,
+// 64: 496 / 469.  Above: 7092, 282, 150: 186 / 174; 6591, 538, 282: 548 / 348; 19773, 538, 282: 1,448 / 743; 16276, 128,
+// 96: 133 / 108; 32552, 128, 72: 177 / 154; 44500, 112, 81: 231 / 194; 100000, 91, 90: 503 / 385; 334272, 100, 80: 1,390 /
+// 1,141.  On 300 measured sizes the slower side is taken by at most 5%.
+static bool update_tc_pays(int64_t n, int q, int k) {
+    const double qk = (double)q * k, waves = (double)n / UPDATE_TC_WAVE, fill = waves / std::ceil(waves);
+    if (n < 6144 || k < 56 || qk < 7200 || n * qk < 2e8) return false;
+    return qk >= 12000 || fill >= 0.8 || (qk >= 9000 && n * qk >= 3e8);
+}
+
 int update2_df64(Session* s, double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, int64_t n,
                  const double* W, int k, cudaStream_t st, bool split_w) {
     const int q = q0 + q1;
     if (k > q0) return fail(HBSD_ERR_ARG, "update: k must not exceed the first segment width");
-    // On the tensor cores from here (us, pairs / digit slices; n, q, k): 20000, 149, 85: 187 / 157; 47620, 112, 56:
-    // 172 / 153; 6000, 538, 282: 459 / 328; 20000, 538, 282: 1,441 / 733.  Below, one CTA's chain of column tiles
-    // and the passes over Z for exponents and guard cost more: 20000, 128, 64: 106 / 117; 6000, 282, 150: 156 /
-    // 165; 646, 538, 282: 139 / 322; with half-empty column tiles 150000, 96, 48: 373 / 402.
-    if (n >= 6144 && k >= 56 && (double)n * q * k >= 2e8) {
+    if (update_tc_pays(n, q, k)) {
         if ((size_t)UR * q * sizeof(float2) <= 220 * 1024 && update_tc_fits(Z0, ld0, Z1, ld1, q1, k))
             return update2_tc(s, Z0, ld0, q0, Z1, ld1, q1, n, W, k, st);
         split_w = true;   // an earlier block of the same step may have gone the other way and left df_w alone

@@ -37,7 +37,8 @@ constexpr int TU_SLICERS = 256;                      // the same of the guard
 constexpr int TU_THREADS = TU_SLICERS + 64;
 constexpr int TU_OUT_LD = 17;                        // doubles per row of a warp's 32 x 16 outputs in shared memory
 constexpr size_t TU_SMEM = (size_t)TU_NS * TU_STAGE + (size_t)8 * 32 * (TU_OUT_LD + 4) * 8 + 1024;
-constexpr int64_t TU_WAVE = 152 * ROWS;              // rows of one tile per SM
+constexpr int64_t TU_WAVE = UPDATE_TC_WAVE;
+static_assert(TU_WAVE == 152 * ROWS, "one tile per SM");
 constexpr int64_t TU_SLAB_BYTES = 88 << 20;          // Z rows of a slab: they stay in L2 between the passes
 constexpr int64_t TU_SLAB_ROWS = 65536;              // a list entry holds 16 bits of row
 constexpr int TU_GUARD_NS = 4;                       // stage buffers of the guard

@@ -164,6 +164,13 @@ def test_gram_tensor_core_entries_just_above_the_guard(n, most, tail):
         assert rel.max() <= 2.0 ** -46, np.log2(rel.max())
 
 
+@pytest.mark.parametrize("q,n", [(47, 40001), (48, 34721), (48, 34817), (49, 33537), (64, 20225), (65, 19201)])
+def test_gram_on_both_sides_of_the_width_rule(q, n):
+    """Pairs below 48 columns whatever the rows, and below n q^2 = 8e7; digit slices above, with nearly empty second
+    tiles of 32 and of 128 columns."""
+    check(*blocks(q, n, 400 + q))
+
+
 def test_gram_scratch_covers_every_row_count():
     """hbsd_gram's scratch depends on the width alone: after one call of a few rows, calls of any height at
     widths of as many 32-column tiles can be captured (nothing is allocated)."""

@@ -130,3 +130,12 @@ def test_update_entries_just_above_the_guard(n, q, k, most):
     exact, mag = (Z @ W)[:, 1:], (np.abs(Z) @ np.abs(W))[:, 1:]
     rel = (np.abs(out - exact) / mag).max()
     assert rel <= 2.0 ** -46, np.log2(rel)
+
+
+# q k below and from 7,200 on, waves of row tiles filled and not, n q k below and from 3e8 on: pairs, slices, pairs, slices,
+# pairs, slices; then column tiles of one column, q one more and one less than whole steps of 16
+@pytest.mark.parametrize("n,q,k", [(37001, 100, 71), (37001, 100, 72), (40001, 100, 72), (44003, 100, 90), (23003, 128, 90),
+                                   (28003, 128, 90), (38913, 129, 90), (40003, 175, 57), (40013, 113, 90), (12289, 257, 65),
+                                   (37005, 111, 65)])
+def test_update_around_the_rule_of_narrow_blocks(n, q, k):
+    check(*blocks(n, q, k, 1300 + q))
