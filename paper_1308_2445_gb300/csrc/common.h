@@ -264,10 +264,13 @@ int update_df64_rows(Session* s, const double* Z0, int64_t ld0, int q0, const do
 int update_oz(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, int64_t n,
               const double* W, int k, double* Y, int64_t ldy, cudaStream_t st, int* status = nullptr);
 constexpr int OZ_MAX_Q_SEG = 640;   // largest block width update_oz takes
-// the same over the whole GPU (rr_grid.cu); ws: rr_grid_ws_doubles(q, k)
+// the Rayleigh-Ritz step over the whole GPU (rr_grid.cu); ws: rr_grid_ws_doubles(q, k), its per-vector diagnostics at
+// rr_grid_vdiag; ev: 8 events around its 7 phases, or NULL
 size_t rr_grid_ws_doubles(int q, int k);
+size_t rr_grid_vdiag(int q, int k);
 int rayleigh_ritz_grid(Session* s, const double* HR, const double* SR, int q, int k, double* theta, double* W, double* ws,
-                       int* info, cudaStream_t st, bool* launched);
+                       int* info, cudaStream_t st, bool* launched, cudaEvent_t* ev = nullptr);
+// the same on one cluster, or by the form above
 int rayleigh_ritz_cluster(Session* s, const double* HR, const double* SR, int q, int k, double* theta,
                           double* W, int* info_host, cudaStream_t st, double drop_tol = 0.0);
 template <class T>

@@ -733,10 +733,11 @@ int rayleigh_ritz_cluster(Session* s, const double* HR, const double* SR, int q,
     const bool grid = drop_tol == 0.0 && q >= RR_GRID_MIN_Q;
     if (grid) HBSD_TRY(s->rr_ws.alloc(rr_grid_ws_doubles(q, k)));
     static const bool trace = std::getenv("HBSD_TRACE") != nullptr || std::getenv("HBSD_RRDBG") != nullptr;
-    static thread_local cudaEvent_t tev[4];
+    static thread_local cudaEvent_t tev[4], gev[8];   // gev: phases of the form over the whole GPU
     static thread_local bool tev_made = false;
     if (trace && !tev_made) {
         for (auto& e : tev) cudaEventCreate(&e);
+        for (auto& e : gev) cudaEventCreate(&e);
         tev_made = true;
     }
     if (trace) cudaEventRecord(tev[0], st);
@@ -749,7 +750,8 @@ int rayleigh_ritz_cluster(Session* s, const double* HR, const double* SR, int q,
     bool launched = false, on_grid = false;
     int used_nc = 0, used_stage = 0;
     if (grid) {
-        HBSD_TRY(rayleigh_ritz_grid(s, HR, SR, q, k, theta, W, s->rr_ws.p, s->rr_info.p, st, &launched));
+        HBSD_TRY(rayleigh_ritz_grid(s, HR, SR, q, k, theta, W, s->rr_ws.p, s->rr_info.p, st, &launched,
+                                    trace ? gev : nullptr));
         on_grid = launched;
         if (trace && launched) cudaEventRecord(tev[1], st);
     }
@@ -815,10 +817,10 @@ int rayleigh_ritz_cluster(Session* s, const double* HR, const double* SR, int q,
     HBSD_CUDA(cudaMemcpyAsync(info, s->rr_info.p, 4 * sizeof(int), cudaMemcpyDeviceToHost, st));
     {
         static const char* dbg = std::getenv("HBSD_RRDBG");
-        if (dbg && dbg[0] == '2' && !on_grid) {
+        if (dbg && dbg[0] == '2') {
             std::vector<double> vd(3 * (size_t)k);
-            HBSD_CUDA(cudaMemcpyAsync(vd.data(), s->rr_ws.p + rr_cluster_ws_doubles(q, k, 16, 1) - 3 * k,
-                                      3 * k * sizeof(double), cudaMemcpyDeviceToHost, st));
+            const size_t at = on_grid ? rr_grid_vdiag(q, k) : (size_t)rr_cluster_ws_doubles(q, k, 16, 1) - 3 * k;
+            HBSD_CUDA(cudaMemcpyAsync(vd.data(), s->rr_ws.p + at, 3 * k * sizeof(double), cudaMemcpyDeviceToHost, st));
             HBSD_CUDA(cudaStreamSynchronize(st));
             for (int j = 0; j < k; ++j)
                 std::fprintf(stderr, "[hbsd]   RR vec %d solves-after-first %d theta %.12e coarse %.12e\n", j, (int)vd[j],
@@ -842,6 +844,13 @@ int rayleigh_ritz_cluster(Session* s, const double* HR, const double* SR, int q,
     if (on_grid) {   // no column dropped
         info[0] = 0;
         info[1] = q;
+    }
+    if (std::getenv("HBSD_TRACE") && !info[3] && on_grid) {
+        float ms[7];
+        for (int i = 0; i < 7; ++i) HBSD_CUDA(cudaEventElapsedTime(&ms[i], gev[i], gev[i + 1]));
+        std::fprintf(stderr,
+                     "[hbsd]   RR q %d k %d whole GPU us: chol %.0f C %.0f tridiag %.0f eig %.0f rqi %.0f cholqr %.0f back %.0f\n",
+                     q, k, ms[0] * 1e3, ms[1] * 1e3, ms[2] * 1e3, ms[3] * 1e3, ms[4] * 1e3, ms[5] * 1e3, ms[6] * 1e3);
     }
     if (std::getenv("HBSD_TRACE") && !info[3] && !on_grid) {
         uint64_t t[10];

@@ -454,10 +454,11 @@ __global__ void __launch_bounds__(128) k_rg_bisect(const double* __restrict__ dg
     if (lane == 0) lam[j] = 0.5 * (lo + hi);
 }
 
-// Eigenvector j of T on one warp (rr_math.h), to Vt[j q + i]
+// Eigenvector j of T on one warp (rr_math.h), to Vt[j q + i].  vdiag[3][k]: solves after the first, last shift, coarse
+// eigenvalue (read by the host under HBSD_RRDBG=2)
 __global__ void __launch_bounds__(32) k_rg_invit(const double* __restrict__ dg, const double* __restrict__ eg, int q, int k,
                                                  const double* __restrict__ lam, double* __restrict__ Vt, double* gscr,
-                                                 const int* __restrict__ info) {
+                                                 double* __restrict__ vdiag, const int* __restrict__ info) {
     if (rg_stop(info, nullptr)) return;
     extern __shared__ double ism[];
     const int lane = threadIdx.x, j = (int)blockIdx.x;
@@ -471,9 +472,14 @@ __global__ void __launch_bounds__(32) k_rg_invit(const double* __restrict__ dg, 
     __syncwarp();
     const TriBounds tb = tri_bounds(dd, ee, q, lane);
     double th;
-    tri_eigenvector(dd, ee, q, k, j, lam, tb.tnorm, tb.pivmin, scr, lane, [&](const double* x) {
+    const int solves = tri_eigenvector(dd, ee, q, k, j, lam, tb.tnorm, tb.pivmin, scr, lane, [&](const double* x) {
         for (int i = lane; i < q; i += 32) Vt[(int64_t)j * q + i] = x[i];
     }, &th);
+    if (lane == 0) {
+        vdiag[j] = (double)solves;
+        vdiag[k + j] = th;
+        vdiag[2 * k + j] = lam[j];
+    }
 }
 
 // G = V^T V (lower triangle) from the rows of Vt (k x q), one 16 x 16 tile per CTA; off = max |G - I|
@@ -704,14 +710,18 @@ __global__ void __launch_bounds__(128) k_rg_back(const double* __restrict__ VH, 
 size_t rr_grid_ws_doubles(int q, int k) {
     const int lda = q + 20, maxrows = (q + RG_CLUSTER - 1) / RG_CLUSTER;
     return (size_t)6 * q * q + (size_t)RG_CLUSTER * maxrows * lda + (size_t)2 * q * k + (size_t)3 * k * k +
-           (size_t)4 * q * k + 42 * (size_t)q + 4 * (size_t)k + 1200;
+           (size_t)4 * q * k + 42 * (size_t)q + 7 * (size_t)k + 1200;
 }
+size_t rr_grid_vdiag(int q, int k) { return rr_grid_ws_doubles(q, k) - 3 * (size_t)k; }
 
-// Launches the whole reduced solve (info must be zero); false: the cluster cannot be scheduled here and
-// nothing was launched.
+// Launches the whole reduced solve (info must be zero); *launched = false: the cluster cannot be scheduled here and
+// nothing was launched.  ev (nullable): 8 events, recorded before the first launch and after each phase.
 int rayleigh_ritz_grid(Session* s, const double* HR, const double* SR, int q, int k, double* theta, double* W, double* ws,
-                       int* info, cudaStream_t st, bool* launched) {
+                       int* info, cudaStream_t st, bool* launched, cudaEvent_t* ev) {
     *launched = false;
+    auto mark = [&](int i) {
+        if (ev) (void)cudaEventRecord(ev[i], st);
+    };
     const size_t qq = (size_t)q * q, kk = (size_t)k * k, qk = (size_t)q * k;
     double* A = ws;
     double* L = A + qq;
@@ -795,22 +805,28 @@ int rayleigh_ritz_grid(Session* s, const double* HR, const double* SR, int q, in
     };
     HBSD_CUDA(cudaMemsetAsync(off, 0, 2 * sizeof(*off), st));
     *launched = true;
+    mark(0);
     const int tq = ceil_div(q, 32);
     k_rg_scale<<<dim3(tq, tq), 256, 0, st>>>(SR, q, A, dv);
     HBSD_LAUNCHED(s);
     HBSD_TRY(cholesky(A, q, 0, L, LT, rl, nullptr));
+    mark(1);
     // T(:, j) = L^{-1} Hd(:, j) at T[j q + i]; C(:, j) = L^{-1} T(j, :)^T, rows up to j's block, at C[j q + i]
     k_rg_fwd<<<ceil_div(q, 4), 128, fwd_sm, st>>>(LT, rl, q, q, HR, 1, q, dv, T, 1, q, 0, info, nullptr);
     HBSD_LAUNCHED(s);
     k_rg_fwd<<<ceil_div(q, 4), 128, fwd_sm, st>>>(LT, rl, q, q, T, q, 1, nullptr, C, 1, q, 1, info, nullptr);
     HBSD_LAUNCHED(s);
+    mark(2);
     HBSD_CUDA(cudaLaunchKernelEx(&cfg, k_rg_tridiag, (const double*)C, q, lda, in_sm ? (double*)nullptr : arows, rowbuf, VH, tau, dg, eg,
                                  (const int*)info));
     HBSD_LAUNCHED(s);
+    mark(3);
     k_rg_bisect<<<ceil_div(k, 4), 128, bis_sm, st>>>(dg, eg, q, k, lam, info);
     HBSD_LAUNCHED(s);
-    k_rg_invit<<<k, 32, inv_sm, st>>>(dg, eg, q, k, lam, V1, inv_in ? nullptr : scr, info);
+    mark(4);
+    k_rg_invit<<<k, 32, inv_sm, st>>>(dg, eg, q, k, lam, V1, inv_in ? nullptr : scr, ws + rr_grid_vdiag(q, k), info);
     HBSD_LAUNCHED(s);
+    mark(5);
     // CholeskyQR: V1 -> V2, and V2 -> V1 when the first pass found the vectors far from orthonormal
     const int tk = ceil_div(k, 16);
     for (int pass = 0; pass < 2; ++pass) {
@@ -824,6 +840,7 @@ int rayleigh_ritz_grid(Session* s, const double* HR, const double* SR, int q, in
                                                                             gate);
         HBSD_LAUNCHED(s);
     }
+    mark(6);
     // the vectors are in V2, or in V1 after a second pass (rg_stop(info, off) chooses)
     k_rg_quotients<<<ceil_div(k, 4), 128, 0, st>>>(dg, eg, q, k, V2, V1, lamr, info, off);
     HBSD_LAUNCHED(s);
@@ -831,6 +848,7 @@ int rayleigh_ritz_grid(Session* s, const double* HR, const double* SR, int q, in
     HBSD_LAUNCHED(s);
     k_rg_back<<<k, 128, back_sm, st>>>(VH, GV, tau, L, rl, q, k, V2, V1, lamr, dv, theta, W, info, off);
     HBSD_LAUNCHED(s);
+    mark(7);
     return 0;
 }
 

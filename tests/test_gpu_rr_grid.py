@@ -139,3 +139,26 @@ def test_entries_too_small_to_square():
     except hbsd.HbsdError:
         return
     assert not (np.isfinite(th).all() and np.isfinite(W).all())
+
+
+def test_trace_output():
+    """HBSD_TRACE prints the phases of a call and HBSD_RRDBG=2 a line per vector, whichever kernels ran."""
+    import os
+    import subprocess
+    import sys
+    code = ("import numpy as np, torch\nfrom paper_1308_2445_gb300 import hbsd\n"
+            "for q in (12, 64):\n"
+            "    H = torch.diag(torch.arange(q, dtype=torch.float64)).cuda() + 0.01\n"
+            "    S = torch.eye(q, dtype=torch.float64, device='cuda')\n"
+            "    th, W = (torch.zeros(s, dtype=torch.float64, device='cuda') for s in ((9,), (q, 9)))\n"
+            "    hbsd.rayleigh_ritz(H, S, 9, th, W, torch.zeros(2, dtype=torch.int32, device='cuda'))\n")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, env=dict(os.environ, HBSD_TRACE="1", HBSD_RRDBG="2"),
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    assert r.stderr.count("RR vec") == 2 * 9
+    for q in (12, 64):
+        line = [x for x in r.stderr.splitlines() if f"RR q {q} k 9" in x]
+        assert len(line) == 1
+        for phase in ("chol", "C", "tridiag", "eig", "rqi", "cholqr", "back"):
+            assert f" {phase} " in line[0]
