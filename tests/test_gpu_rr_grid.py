@@ -162,3 +162,22 @@ def test_trace_output():
         assert len(line) == 1
         for phase in ("chol", "C", "tridiag", "eig", "rqi", "cholqr", "back"):
             assert f" {phase} " in line[0]
+
+
+@pytest.mark.parametrize("q,k", [(640, 40), (2200, 24)])
+def test_rows_and_iterates_in_global_memory(q, k):
+    """From 625 columns on the rows of the tridiagonalisation leave shared memory, from 2,134 on the inverse iteration's
+    scratch does.  S_R diagonal, so that the reference is one standard eigenproblem; tolerances as above."""
+    rng = np.random.default_rng(q)
+    B = rng.standard_normal((q, q))
+    B = np.diag(np.arange(q) * 1.0) + (B + B.T) / np.sqrt(q)
+    d = 10.0 ** rng.uniform(-2, 2, q)
+    HR, SR = d[:, None] * B * d, np.diag(d * d)
+    HR = 0.5 * (HR + HR.T)
+    th, W, info = run(HR, SR, k)
+    g = np.linalg.eigvalsh(B)
+    scale = np.abs(g).max()
+    assert info[0] == 0 and info[1] == q
+    assert np.abs(th - g[:k]).max() <= 1e-11 * scale
+    assert np.abs(W.T @ SR @ W - np.eye(k)).max() <= 1e-10
+    assert np.abs(W.T @ HR @ W - np.diag(th)).max() <= 1e-10 * scale
