@@ -546,7 +546,10 @@ int hbsd_solve_batch(hbsd_batch_item* items, int count, const hbsd_batch_opts* o
  * well, as long as the roundings of different rows are not all the same (columns that repeat one value from
  * row to row beside a much larger entry elsewhere: 41 bits at worst).  So does the update of n >= 6144
  * rows and 56 <= k <= 512 columns from n q k = 2e8 and q k = 7200 on, where that is the faster form (below q k =
- * 12000 not at every n), if Z is 16-byte aligned and ldz even.  hbsd_gram_df64
+ * 12000 not at every n), if Z is 16-byte aligned and ldz even.  Calls under stream capture run in pairs whatever
+ * their size: after one call of as many columns they allocate nothing, and later calls leave a graph's scratch
+ * where it is (of the Gram, if that call had as many rows or more than 311,000 / p, p = t (t + 1) / 2, t = ceil(q / 32)).
+ * hbsd_gram_df64
  * computes the entries a <= b of Z^T ZH and Z^T ZS and mirrors them (no averaging).  Arguments,
  * layouts and errors as hbsd_gram / hbsd_update; FP64 values enter the products with ~47 bits
  * above 2^-96 in magnitude, at least 24 bits down to 2^-126, and as zero below.  hbsd_update_df64

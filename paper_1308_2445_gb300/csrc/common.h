@@ -241,6 +241,8 @@ int rayleigh_ritz(Session* s, const double* HR, const double* SR, int q, int k, 
 int gram2_df64(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1,
                const double* H0, int64_t ldh0, const double* H1, int64_t ldh1, const double* S0, int64_t lds0,
                const double* S1, int64_t lds1, int64_t n, double* HR, double* SR, cudaStream_t st);
+// leaves scratch for calls of gram2_df64 under capture: of no more rows, or of any number once n gives every SM its CTAs
+int gram_df64_reserve(Session* s, int64_t n, int q);
 // the Gram on the tensor cores by exact digit slices, at least as accurate (gram_tc.cu)
 int gram2_tc(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, const double* H0,
              int64_t ldh0, const double* H1, int64_t ldh1, const double* S0, int64_t lds0, const double* S1, int64_t lds1,
@@ -357,7 +359,7 @@ struct Session {
     DBuf<int> mr_any, mr_steps; // grid barrier + error flag; per-column step counts
     DBuf<unsigned long long> mr_stamps;   // MINRES phase times when tracing
     DBuf<int64_t> mr_blk;       // per-block SELL slot ranges of the fused MINRES kernel
-    DBuf<double> ut_ws;         // tensor-core update (update_tc.cu): slab results, slices of W, exponents, list
+    DBuf<double> df_ws;         // double-float Gram and update: sums, results of a slab, slices of W, exponents, lists
     DBuf<float2> df_w;          // double-float copy of the Rayleigh-Ritz coefficients W
     DBuf<double> oz_ws;         // split-slice update: exponents and bf16 slices of W (oz.cu)
     DBuf<int> oz_status;        // set by a timed-out MMA wait of the solve's tensor-core updates

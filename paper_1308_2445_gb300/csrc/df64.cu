@@ -221,6 +221,26 @@ __global__ void __launch_bounds__(512) k_update_df64_kt(const double* Z0, int64_
 
 }  // namespace
 
+// Under capture nothing may be allocated, and a graph keeps the address of its scratch.  The tensor-core forms' scratch
+// grows with the rows, so captured calls run the pairs, with scratch that a call of fewer rows has left and a call of
+// more rows does not move: the update's copy of W, and for the Gram s->ws, which stops growing at CAPTURED_CTAS CTAs
+// per SM and which other calls of the Gram reserve without using it.
+static bool stream_captured(cudaStream_t st) {
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &c) != cudaSuccess) {   // the legacy stream beside another thread's capture
+        (void)cudaGetLastError();
+        return false;
+    }
+    return c != cudaStreamCaptureStatusNone;
+}
+constexpr int CAPTURED_CTAS = 8;
+static int captured_chunks(int64_t n, int q) {
+    const int ntile = ceil_div(q, GW), npair = ntile * (ntile + 1) / 2;
+    return (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, ceil_div(152 * CAPTURED_CTAS, npair)));
+}
+
+int gram_df64_reserve(Session* s, int64_t n, int q) { return s->ws.alloc((size_t)captured_chunks(n, q) * 2 * q * q + 64); }
+
 int gram2_df64(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1,
                const double* H0, int64_t ldh0, const double* H1, int64_t ldh1, const double* S0, int64_t lds0,
                const double* S1, int64_t lds1, int64_t n, double* HR, double* SR, cudaStream_t st) {
@@ -232,7 +252,8 @@ int gram2_df64(Session* s, const double* Z0, int64_t ld0, int q0, const double* 
     // n = 15,869: 108 / 92; q = 149, n = 2,252: 57 / 72, n = 5,855: 108 / 75; q = 538, n = 449: 101 / 105, n = 1,036:
     // 177 / 142; q = 48, n = 34,722: 115 / 101, n = 434,027: 1,007 / 884; q = 40, n = 81,250: 194 / 196, n = 625,000:
     // 1,116 / 1,264; q = 33, n = 275,482: 564 / 580; q = 24, n = 225,694: 249 / 336; q = 19, n = 360,110: 406 / 515.
-    if (q >= 48 && (double)n * q * q >= 8e7)
+    const bool captured = stream_captured(st);
+    if (!captured && q >= 48 && (double)n * q * q >= 8e7)
         return gram2_tc(s, Z0, ld0, q0, Z1, ld1, q1, H0, ldh0, H1, ldh1, S0, lds0, S1, lds1, n, HR, SR, st);
     // tiles of equal width, a multiple of 4 columns up to GW
     const int ntile = ceil_div(q, GW);
@@ -240,14 +261,16 @@ int gram2_df64(Session* s, const double* Z0, int64_t ld0, int q0, const double* 
     const int npair = ntile * (ntile + 1) / 2;
     // chunks of rows: several waves of CTAs, at least 128 rows each
     int nch = (int)std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, ceil_div(GWAVES * 152 * GCTAS, npair)));
+    if (captured) nch = captured_chunks(n, q);
     int64_t rpc = round_up((n + nch - 1) / nch, GR);
     nch = (int)((n + rpc - 1) / rpc);
-    HBSD_TRY(s->ws.alloc((size_t)nch * 2 * q * q + 64));
+    DBuf<double>& ws = captured ? s->ws : s->df_ws;
+    HBSD_TRY(ws.alloc((size_t)nch * 2 * q * q + 64));
     Seg2d Z{Z0, ld0, q0, Z1, ld1}, ZH{H0, ldh0, q0, H1, ldh1}, ZS{S0, lds0, q0, S1, lds1};
-    k_gram_df64<<<dim3(npair, nch), GTHREADS, 0, st>>>(Z, ZH, ZS, q, n, rpc, ntile, nb, df::NEG_ZERO2, s->ws.p);
+    k_gram_df64<<<dim3(npair, nch), GTHREADS, 0, st>>>(Z, ZH, ZS, q, n, rpc, ntile, nb, df::NEG_ZERO2, ws.p);
     HBSD_LAUNCHED(s);
     const int64_t qq = (int64_t)q * q;
-    k_gram_final_upper<<<ceil_div(qq, 32), 256, 0, st>>>(s->ws.p, nch, q, HR, SR);
+    k_gram_final_upper<<<ceil_div(qq, 32), 256, 0, st>>>(ws.p, nch, q, HR, SR);
     HBSD_LAUNCHED(s);
     return 0;
 }
@@ -271,7 +294,7 @@ int update2_df64(Session* s, double* Z0, int64_t ld0, int q0, const double* Z1, 
     const int q = q0 + q1;
     if (k > q0) return fail(HBSD_ERR_ARG, "update: k must not exceed the first segment width");
     if (update_tc_pays(n, q, k)) {
-        if ((size_t)UR * q * sizeof(float2) <= 220 * 1024 && update_tc_fits(Z0, ld0, Z1, ld1, q1, k))
+        if (!stream_captured(st) && (size_t)UR * q * sizeof(float2) <= 220 * 1024 && update_tc_fits(Z0, ld0, Z1, ld1, q1, k))
             return update2_tc(s, Z0, ld0, q0, Z1, ld1, q1, n, W, k, st);
         split_w = true;   // an earlier block of the same step may have gone the other way and left df_w alone
     }

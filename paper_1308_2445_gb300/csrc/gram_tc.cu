@@ -505,8 +505,8 @@ int gram2_tc(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1
     const int64_t rpad = round_up(n, TG_BLK);
     // workspace: sums | listed entries | row exponents | column exponents | guard rows | listed units
     const size_t ints = (size_t)rpad + (size_t)nch * 3 * q + (size_t)rpad / 16 + 2 + (size_t)units;
-    HBSD_TRY(s->ws.alloc((size_t)units * (TG_ACC + TG_UNIT_FIX) + ints / 2 + 64));
-    double* part = s->ws.p;
+    HBSD_TRY(s->df_ws.alloc((size_t)units * (TG_ACC + TG_UNIT_FIX) + ints / 2 + 64));
+    double* part = s->df_ws.p;
     long long* ents = reinterpret_cast<long long*>(part + units * TG_ACC);
     int* rexp = reinterpret_cast<int*>(ents + units * TG_UNIT_FIX);   // 16-byte aligned: both strides are even
     int* cexp = rexp + rpad;

@@ -582,8 +582,8 @@ int update2_tc(Session* s, double* Z0, int64_t ld0, int q0, const double* Z1, in
     const size_t y_b = (size_t)slab * k * 8, sl_b = (size_t)jt * S.total * DIG * B_SLICE, g_b = (size_t)S.total * kp64 * 32;
     const size_t ints = (size_t)slab + 16 * S.total + kp64 + 2 + cap;
     const size_t a_y = (y_b + 1023) / 1024 * 1024, a_sl = (sl_b + 1023) / 1024 * 1024, a_g = (g_b + 1023) / 1024 * 1024;
-    HBSD_TRY(s->ut_ws.alloc((a_y + a_sl + a_g + ints * 4 + 64) / 8 + 1));
-    uint8_t* ws = reinterpret_cast<uint8_t*>(s->ut_ws.p);
+    HBSD_TRY(s->df_ws.alloc((a_y + a_sl + a_g + ints * 4 + 64) / 8 + 1));
+    uint8_t* ws = reinterpret_cast<uint8_t*>(s->df_ws.p);
     double* Y = reinterpret_cast<double*>(ws);
     uint8_t* Wsl = ws + a_y;
     uint8_t* Wg = Wsl + a_sl;

@@ -202,3 +202,38 @@ def test_gram_scratch_covers_every_row_count():
     t.start()
     t.join()
     assert not errors, errors[0]
+
+
+def test_gram_df64_captured_after_fewer_rows():
+    """A captured call allocates nothing after a call of fewer rows -- of either form, with as many rows as give every
+    SM its CTAs --, and an uncaptured call of more rows leaves the graph's scratch where it is.  Bound as above."""
+    import threading
+    from paper_1308_2445_gb300 import hbsd
+    errors = []
+
+    def work():   # a thread of its own: the scratch of these calls is kept per thread
+        try:
+            side = torch.cuda.Stream()
+            with torch.cuda.stream(side):
+                for q, n0, n1, n2 in ((149, 25000, 47620, 90000), (40, 104000, 120000, 160000), (149, 3000, 2900, 30000)):
+                    dev = lambda n: torch.randn(n, q, dtype=torch.float64, device="cuda")
+                    HR, SR, H2, S2 = (torch.zeros(q, q, dtype=torch.float64, device="cuda") for _ in range(4))
+                    small, Z, large = dev(n0), dev(n1), dev(n2)
+                    hbsd.gram_df64(small, small, small, HR, SR, stream=side.cuda_stream)
+                    side.synchronize()
+                    g = torch.cuda.CUDAGraph()
+                    with torch.cuda.graph(g, stream=side):
+                        hbsd.gram_df64(Z, Z, Z, HR, SR, stream=side.cuda_stream)
+                    hbsd.gram_df64(large, large, large, H2, S2, stream=side.cuda_stream)
+                    g.replay()
+                    side.synchronize()
+                    for A, B, C in ((Z, HR, SR), (large, H2, S2)):
+                        exact, bound = A.T @ A, 2.0 ** -44 * (A.abs().T @ A.abs())
+                        assert ((B - exact).abs() <= bound).all() and ((C - exact).abs() <= bound).all()
+        except Exception as e:   # noqa: BLE001 - handed to the test
+            errors.append(e)
+
+    t = threading.Thread(target=work)
+    t.start()
+    t.join()
+    assert not errors, errors[0]

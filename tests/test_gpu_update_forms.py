@@ -139,3 +139,37 @@ def test_update_entries_just_above_the_guard(n, q, k, most):
                                    (37005, 111, 65)])
 def test_update_around_the_rule_of_narrow_blocks(n, q, k):
     check(*blocks(n, q, k, 1300 + q))
+
+
+def test_update_captured_after_fewer_rows():
+    """A captured call allocates nothing after a call of fewer rows, of either form, and an uncaptured call of more rows
+    leaves the graph's scratch where it is.  Bound as above."""
+    import threading
+    from paper_1308_2445_gb300 import hbsd
+    errors = []
+
+    def work():   # a thread of its own: the scratch of these calls is kept per thread
+        try:
+            side = torch.cuda.Stream()
+            with torch.cuda.stream(side):
+                for q, k, n0, n1, n2 in ((160, 140, 100, 9000, 30000), (160, 140, 9000, 9500, 40000)):
+                    W = torch.randn(q, k, dtype=torch.float64, device="cuda")
+                    small, Z, large = (torch.randn(n, q, dtype=torch.float64, device="cuda") for n in (n0, n1, n2))
+                    Z0, L0 = Z.clone(), large.clone()
+                    hbsd.update_df64(small, W, k, stream=side.cuda_stream)
+                    side.synchronize()
+                    g = torch.cuda.CUDAGraph()
+                    with torch.cuda.graph(g, stream=side):
+                        hbsd.update_df64(Z, W, k, stream=side.cuda_stream)
+                    hbsd.update_df64(large, W, k, stream=side.cuda_stream)
+                    g.replay()
+                    side.synchronize()
+                    for A, B in ((Z0, Z), (L0, large)):
+                        assert ((B[:, :k] - A @ W).abs() <= 2.0 ** -44 * (A.abs() @ W.abs())).all()
+        except Exception as e:   # noqa: BLE001 - handed to the test
+            errors.append(e)
+
+    t = threading.Thread(target=work)
+    t.start()
+    t.join()
+    assert not errors, errors[0]
