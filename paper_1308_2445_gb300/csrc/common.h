@@ -256,6 +256,10 @@ constexpr int64_t UPDATE_TC_WAVE = 152 * 128;   // rows of one tile per SM
 bool update_tc_fits(const double* Z0, int64_t ld0, const double* Z1, int64_t ld1, int q1, int k);
 int update2_tc(Session* s, double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, int64_t n, const double* W,
                int k, cudaStream_t st);
+size_t gram_tc_doubles(int64_t n, int q);   // of s->df_ws
+size_t update_tc_doubles(int64_t n, int q0, int q1, int k);
+// the most of s->df_ws that the Grams and updates of a solve take, for q_lo to q_hi columns (df64.cu)
+size_t df64_solve_doubles(int64_t n, int q_lo, int q_hi, int k);
 // Y = [Z0 Z1] W in double-float (df64.cu); with cnt, only when *cnt > cap on the device
 int update_df64_rows(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, int64_t n,
                      const double* W, int k, double* Y, int64_t ldy, const unsigned* cnt, unsigned cap, cudaStream_t st,

@@ -241,27 +241,33 @@ static int captured_chunks(int64_t n, int q) {
 
 int gram_df64_reserve(Session* s, int64_t n, int q) { return s->ws.alloc((size_t)captured_chunks(n, q) * 2 * q * q + 64); }
 
+// Tensor cores from n q^2 = 8e7 on: below it the exponent pass, the lists and the fix-up launch (50 us at
+// the least) outweigh the products.  Not below 48 columns, whatever the rows: a tile of 128 x (32 + 32) columns is
+// then mostly padding.  Measured on both sides, us (k_gram_df64 / tensor cores): q = 71, n = 5,951: 57 / 69,
+// n = 15,869: 108 / 92; q = 149, n = 2,252: 57 / 72, n = 5,855: 108 / 75; q = 538, n = 449: 101 / 105, n = 1,036:
+// 177 / 142; q = 48, n = 34,722: 115 / 101, n = 434,027: 1,007 / 884; q = 40, n = 81,250: 194 / 196, n = 625,000:
+// 1,116 / 1,264; q = 33, n = 275,482: 564 / 580; q = 24, n = 225,694: 249 / 336; q = 19, n = 360,110: 406 / 515.
+static bool gram_tc_pays(int64_t n, int q) { return q >= 48 && (double)n * q * q >= 8e7; }
+
+// chunks of rows for the pairs: several waves of CTAs, at least 128 rows each
+static int gram_chunks(int64_t n, int q) {
+    const int ntile = ceil_div(q, GW), npair = ntile * (ntile + 1) / 2;
+    return (int)std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, ceil_div(GWAVES * 152 * GCTAS, npair)));
+}
+
 int gram2_df64(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1,
                const double* H0, int64_t ldh0, const double* H1, int64_t ldh1, const double* S0, int64_t lds0,
                const double* S1, int64_t lds1, int64_t n, double* HR, double* SR, cudaStream_t st) {
     const int q = q0 + q1;
     if (q <= 0) return 0;
-    // Tensor cores from n q^2 = 8e7 on: below it the exponent pass, the lists and the fix-up launch (50 us at
-    // the least) outweigh the products.  Not below 48 columns, whatever the rows: a tile of 128 x (32 + 32) columns is
-    // then mostly padding.  Measured on both sides, us (this kernel / tensor cores): q = 71, n = 5,951: 57 / 69,
-    // n = 15,869: 108 / 92; q = 149, n = 2,252: 57 / 72, n = 5,855: 108 / 75; q = 538, n = 449: 101 / 105, n = 1,036:
-    // 177 / 142; q = 48, n = 34,722: 115 / 101, n = 434,027: 1,007 / 884; q = 40, n = 81,250: 194 / 196, n = 625,000:
-    // 1,116 / 1,264; q = 33, n = 275,482: 564 / 580; q = 24, n = 225,694: 249 / 336; q = 19, n = 360,110: 406 / 515.
     const bool captured = stream_captured(st);
-    if (!captured && q >= 48 && (double)n * q * q >= 8e7)
+    if (!captured && gram_tc_pays(n, q))
         return gram2_tc(s, Z0, ld0, q0, Z1, ld1, q1, H0, ldh0, H1, ldh1, S0, lds0, S1, lds1, n, HR, SR, st);
     // tiles of equal width, a multiple of 4 columns up to GW
     const int ntile = ceil_div(q, GW);
     const int nb = ceil_div(ceil_div(q, ntile), 4);
     const int npair = ntile * (ntile + 1) / 2;
-    // chunks of rows: several waves of CTAs, at least 128 rows each
-    int nch = (int)std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, ceil_div(GWAVES * 152 * GCTAS, npair)));
-    if (captured) nch = captured_chunks(n, q);
+    int nch = captured ? captured_chunks(n, q) : gram_chunks(n, q);
     int64_t rpc = round_up((n + nch - 1) / nch, GR);
     nch = (int)((n + rpc - 1) / rpc);
     DBuf<double>& ws = captured ? s->ws : s->df_ws;
@@ -287,6 +293,22 @@ static bool update_tc_pays(int64_t n, int q, int k) {
     const double qk = (double)q * k, waves = (double)n / UPDATE_TC_WAVE, fill = waves / std::ceil(waves);
     if (n < 6144 || k < 56 || qk < 7200 || n * qk < 2e8) return false;
     return qk >= 12000 || fill >= 0.8 || (qk >= 9000 && n * qk >= 3e8);
+}
+
+// The scratch of one call, and the most of a solve whose Grams and updates have q_lo to q_hi columns, the first q_lo of
+// them in one block and k of them updated: reserved before the loop, so that nothing is reallocated (and the
+// device synchronised) while other sessions run.  Uncaptured calls.
+size_t gram_df64_doubles(int64_t n, int q) {
+    return gram_tc_pays(n, q) ? gram_tc_doubles(n, q) : (size_t)gram_chunks(n, q) * 2 * q * q + 64;
+}
+size_t update_df64_doubles(int64_t n, int q0, int q1, int k) {
+    return update_tc_pays(n, q0 + q1, k) && k <= UPDATE_TC_MAX_K ? update_tc_doubles(n, q0, q1, k) : 0;
+}
+size_t df64_solve_doubles(int64_t n, int q_lo, int q_hi, int k) {
+    size_t most = 0;
+    for (int q = q_lo; q <= q_hi; ++q)
+        most = std::max({most, gram_df64_doubles(n, q), update_df64_doubles(n, q_lo, q - q_lo, k)});
+    return most;
 }
 
 int update2_df64(Session* s, double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, int64_t n,

@@ -481,31 +481,46 @@ __global__ void __launch_bounds__(256) k_gram_tc_final(const double* __restrict_
 
 }  // namespace
 
-int gram2_tc(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, const double* H0,
-             int64_t ldh0, const double* H1, int64_t ldh1, const double* S0, int64_t lds0, const double* S1, int64_t lds1,
-             int64_t n, double* HR, double* SR, cudaStream_t st) {
-    const int q = q0 + q1;
-    const int nb = ceil_div(q, TG_B);
-    int npair = 0;
-    for (int ta = 0; ta * TG_M < q; ++ta) npair += nb - 4 * ta;
-    // chunks of whole 256-row blocks: the height that ends the last wave of units soonest
+// tile pairs, and chunks of whole 256-row blocks: the height that ends the last wave of units soonest
+struct TgPlan {
+    int nb, npair, nch;
+    int64_t chunk_rows, units, rpad;
+    size_t ints, doubles;   // of the workspace
+};
+static TgPlan tg_plan(int64_t n, int q) {
+    TgPlan g;
+    g.nb = ceil_div(q, TG_B);
+    g.npair = 0;
+    for (int ta = 0; ta * TG_M < q; ++ta) g.npair += g.nb - 4 * ta;
     const int nblk = ceil_div(n, TG_BLK);
     int bpc = 1;
     double best = 1e300;
     for (int k = 1; k <= std::min(nblk, TG_MAX_BLKS); ++k) {
-        const double cost = (double)ceil_div((int64_t)npair * ceil_div(nblk, k), 152) * (k + 0.4);
+        const double cost = (double)ceil_div((int64_t)g.npair * ceil_div(nblk, k), 152) * (k + 0.4);
         if (cost < best) {
             best = cost;
             bpc = k;
         }
     }
-    const int64_t chunk_rows = (int64_t)bpc * TG_BLK;
-    const int nch = ceil_div(n, chunk_rows);
-    const int64_t units = (int64_t)nch * npair;
-    const int64_t rpad = round_up(n, TG_BLK);
+    g.chunk_rows = (int64_t)bpc * TG_BLK;
+    g.nch = ceil_div(n, g.chunk_rows);
+    g.units = (int64_t)g.nch * g.npair;
+    g.rpad = round_up(n, TG_BLK);
     // workspace: sums | listed entries | row exponents | column exponents | guard rows | listed units
-    const size_t ints = (size_t)rpad + (size_t)nch * 3 * q + (size_t)rpad / 16 + 2 + (size_t)units;
-    HBSD_TRY(s->df_ws.alloc((size_t)units * (TG_ACC + TG_UNIT_FIX) + ints / 2 + 64));
+    g.ints = (size_t)g.rpad + (size_t)g.nch * 3 * q + (size_t)g.rpad / 16 + 2 + (size_t)g.units;
+    g.doubles = (size_t)g.units * (TG_ACC + TG_UNIT_FIX) + g.ints / 2 + 64;
+    return g;
+}
+size_t gram_tc_doubles(int64_t n, int q) { return tg_plan(n, q).doubles; }
+
+int gram2_tc(Session* s, const double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, const double* H0,
+             int64_t ldh0, const double* H1, int64_t ldh1, const double* S0, int64_t lds0, const double* S1, int64_t lds1,
+             int64_t n, double* HR, double* SR, cudaStream_t st) {
+    const int q = q0 + q1;
+    const TgPlan g = tg_plan(n, q);
+    const int nb = g.nb, npair = g.npair, nch = g.nch;
+    const int64_t chunk_rows = g.chunk_rows, units = g.units, rpad = g.rpad;
+    HBSD_TRY(s->df_ws.alloc(g.doubles));
     double* part = s->df_ws.p;
     long long* ents = reinterpret_cast<long long*>(part + units * TG_ACC);
     int* rexp = reinterpret_cast<int*>(ents + units * TG_UNIT_FIX);   // 16-byte aligned: both strides are even

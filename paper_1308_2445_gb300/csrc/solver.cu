@@ -588,11 +588,10 @@ static int labpsd_solve(Session* S, int m, double tol, const double* X0, int64_t
     HBSD_TRY(C.HR.alloc((size_t)qmax * qmax)); HBSD_TRY(C.SR.alloc((size_t)qmax * qmax));
     HBSD_TRY(C.W.alloc((size_t)qmax * w));
     HBSD_TRY(C.Ulist.alloc(m)); HBSD_TRY(C.Llist.alloc(m)); HBSD_TRY(C.steps.alloc(m));
-    {   // scratch of the reductions and the Gram partials, sized once (no reallocation mid-solve)
-        const int tiles = ceil_div(qmax, 32);
-        HBSD_TRY(S->ws.alloc((size_t)2 * 1024 * (1216 + tiles * tiles) + (size_t)304 * 2 * qmax + 1024));
-        HBSD_TRY(S->rr_info.alloc(4));
-    }
+    // scratch of the reductions, the Grams and the updates, sized once (no reallocation mid-solve)
+    HBSD_TRY(S->ws.alloc(gram_scratch_doubles(qmax) + (size_t)304 * 2 * qmax + 1024));
+    HBSD_TRY(S->rr_info.alloc(4));
+    if (mixed && S->opt_df64) HBSD_TRY(S->df_ws.alloc(df64_solve_doubles(n, w, qmax, w)));
     HBSD_TRY(S->oz_status.alloc(1));
     HBSD_CUDA(cudaMemsetAsync(S->oz_status.p, 0, sizeof(int), st));
     hbsd_stats& stt = S->stats;

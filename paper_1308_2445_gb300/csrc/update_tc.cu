@@ -569,25 +569,43 @@ bool update_tc_fits(const double* Z0, int64_t ld0, const double* Z1, int64_t ld1
     return k <= UPDATE_TC_MAX_K && ok(Z0, ld0) && (q1 == 0 || ok(Z1, ld1));
 }
 
+// slabs of whole waves whose Z rows stay in L2 from one pass to the next
+struct TuPlan {
+    int64_t slab;
+    unsigned cap;                // entries of the list
+    size_t y_b, sl_b, g_b;       // bytes of the workspace: results of a slab | slices of W | guard magnitudes of W
+    size_t doubles;              // ... | exponents of rows, W's rows and columns | list
+};
+static TuPlan tu_plan(int64_t n, int q0, int q1, int k) {
+    TuPlan p;
+    const int total = ceil_div(q0, 16) + ceil_div(q1, 16), jt = ceil_div(k, COLS), kp64 = jt * COLS;
+    const int64_t waves = std::max<int64_t>(1, std::min<int64_t>(TU_SLAB_BYTES / (TU_WAVE * (q0 + q1) * 8), TU_SLAB_ROWS / TU_WAVE));
+    p.slab = std::min<int64_t>(waves * TU_WAVE, round_up(n, ROWS));
+    p.cap = (unsigned)std::max<int64_t>(4096, p.slab * k / 16);
+    auto kib = [](size_t b) { return (b + 1023) / 1024 * 1024; };
+    p.y_b = kib((size_t)p.slab * k * 8);
+    p.sl_b = kib((size_t)jt * total * DIG * B_SLICE);
+    p.g_b = kib((size_t)total * kp64 * 32);
+    const size_t ints = (size_t)p.slab + 16 * total + kp64 + 2 + p.cap;
+    p.doubles = (p.y_b + p.sl_b + p.g_b + ints * 4 + 64) / 8 + 1;
+    return p;
+}
+size_t update_tc_doubles(int64_t n, int q0, int q1, int k) { return tu_plan(n, q0, q1, k).doubles; }
+
 int update2_tc(Session* s, double* Z0, int64_t ld0, int q0, const double* Z1, int64_t ld1, int q1, int64_t n, const double* W,
                int k, cudaStream_t st) {
     Steps S{Z0, ld0, q0, Z1, ld1, q1, ceil_div(q0, 16), 0};
     S.total = S.t0 + ceil_div(q1, 16);
     const int jt = ceil_div(k, COLS), kp64 = jt * COLS;
-    // slabs of whole waves whose Z rows stay in L2 from one pass to the next
-    const int64_t waves = std::max<int64_t>(1, std::min<int64_t>(TU_SLAB_BYTES / (TU_WAVE * (q0 + q1) * 8), TU_SLAB_ROWS / TU_WAVE));
-    const int64_t slab = std::min<int64_t>(waves * TU_WAVE, round_up(n, ROWS));
-    const unsigned cap = (unsigned)std::max<int64_t>(4096, slab * k / 16);
-    // workspace: results of a slab | slices of W | guard magnitudes of W | exponents of rows, W's rows and columns | list
-    const size_t y_b = (size_t)slab * k * 8, sl_b = (size_t)jt * S.total * DIG * B_SLICE, g_b = (size_t)S.total * kp64 * 32;
-    const size_t ints = (size_t)slab + 16 * S.total + kp64 + 2 + cap;
-    const size_t a_y = (y_b + 1023) / 1024 * 1024, a_sl = (sl_b + 1023) / 1024 * 1024, a_g = (g_b + 1023) / 1024 * 1024;
-    HBSD_TRY(s->df_ws.alloc((a_y + a_sl + a_g + ints * 4 + 64) / 8 + 1));
+    const TuPlan p = tu_plan(n, q0, q1, k);
+    const int64_t slab = p.slab;
+    const unsigned cap = p.cap;
+    HBSD_TRY(s->df_ws.alloc(p.doubles));
     uint8_t* ws = reinterpret_cast<uint8_t*>(s->df_ws.p);
     double* Y = reinterpret_cast<double*>(ws);
-    uint8_t* Wsl = ws + a_y;
-    uint8_t* Wg = Wsl + a_sl;
-    int* ek = reinterpret_cast<int*>(Wg + a_g);          // 16-byte aligned, a multiple of 16 entries
+    uint8_t* Wsl = ws + p.y_b;
+    uint8_t* Wg = Wsl + p.sl_b;
+    int* ek = reinterpret_cast<int*>(Wg + p.g_b);          // 16-byte aligned, a multiple of 16 entries
     int* rowexp = ek + 16 * S.total;
     int* cw = rowexp + slab;
     unsigned* list = reinterpret_cast<unsigned*>(cw + kp64);
