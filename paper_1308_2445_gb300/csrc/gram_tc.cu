@@ -35,8 +35,8 @@
 // would take at least 50 clocks each).
 //
 // Bound: the integer pipe of the slicers (about 30 integer instructions per value and tile it meets; the
-// tensor core waits for them).  n = 334,272, q = 538: 9.9 ms against 40.5 ms for the FP32 pipes;
-// n = 47,620, q = 149: 0.28 against 0.64 ms.  Error against 64 bits on such blocks 5e-16 (q = 538: 1.9e-15),
+// tensor core waits for them).  n = 334,272, q = 538: 10.0 ms against 40.5 ms for the FP32 pipes;
+// n = 47,620, q = 149: 0.28 against 0.64 ms.  Error against 64 bits on such blocks 3e-16 to 8e-16 (q = 538: 2.3e-15),
 // float pairs 2e-15.
 #include <algorithm>
 #include <mutex>

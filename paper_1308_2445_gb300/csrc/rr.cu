@@ -728,7 +728,7 @@ int rayleigh_ritz_cluster(Session* s, const double* HR, const double* SR, int q,
     HBSD_TRY(s->rr_ws.alloc((size_t)std::max<int64_t>(rr_cluster_ws_doubles(q, k, 16, 1), (int64_t)4 * q * q + 3 * q + 64)));
     HBSD_TRY(s->rr_info.alloc(4));
     // over the whole GPU from 20 columns on, where it is no slower (us, this kernel / whole GPU: q = 20: 349 /
-    // 334, 35: 514 / 471, 64: 847 / 654, 149: 2,450 / 1,396, 538: 44,700 / 8,020); this kernel below, for the
+    // 334, 35: 514 / 471, 64: 847 / 654, 149: 2,464 / 1,428, 538: 44,563 / 7,950); this kernel below, for the
     // column-dropping mode, and where a cluster of 16 cannot be scheduled
     const bool grid = drop_tol == 0.0 && q >= RR_GRID_MIN_Q;
     if (grid) HBSD_TRY(s->rr_ws.alloc(rr_grid_ws_doubles(q, k)));

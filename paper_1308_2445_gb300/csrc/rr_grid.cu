@@ -16,7 +16,7 @@
 //      orthonormal; Rayleigh quotients.
 //   6. W = D L^{-T} H_0 H_1 ... z, one CTA per vector (k_rg_back).
 //
-// One call, one cluster for everything before: q = 149, k = 85: 1.40 ms (2.45), of which tridiagonalisation 0.58,
+// One call, one cluster for everything before: q = 149, k = 85: 1.43 ms (2.46), of which tridiagonalisation 0.58,
 // inverse iteration 0.15, Cholesky panels 0.19; q = 538, k = 282: 8.0 ms (44.7), of which tridiagonalisation 4.8,
 // inverse iteration 0.77, panels 0.62, substitutions 0.6, back-transformation 0.48.
 #include <cooperative_groups.h>

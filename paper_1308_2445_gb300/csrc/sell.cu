@@ -349,7 +349,8 @@ __global__ void k_split_scaled(const double* __restrict__ X, int64_t ldx, int k,
 // Pair mode of k_spmm in double-float: per stored entry the (hi, lo) of D Hs D and of D S D, per column pair one
 // float4 of X2.  Sums by df::dfma's steps on packed column pairs, renormalised every 8 entries; the row result is
 // scaled back by D^-1 in FP64.
-// Bound by the FP32 pipe: 24 packed instructions (48 pipe cycles of a warp) per entry and column pair.  Without the
+// Bound by the FP32 pipe (24 packed instructions, 48 pipe cycles of a warp, per entry and column pair: half of its cycles
+// at 85 columns of the 32^3 problem) and the latency of the gathers.  Without the
 // loads an entry ahead, and with scalar instructions, 85 columns of the 32^3 problem took 583 us (now 404); packed
 // without them 517.
 // nax = -ax; the product is kept negated, which saves negating it for its rounding error

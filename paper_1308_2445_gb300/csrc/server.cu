@@ -74,7 +74,8 @@ size_t estimate_bytes(int64_t n, int64_t nnz, int nev, int nl_k) {
     // fill nnz(L)/nnz measured at 16.5 on the 32^3 workload (n = 47,620) and growing as n^0.35
     // (39 at 64^3), plus a quarter for the factorisation's fronts; ~20 blocks of n x (nev + m0)
     // doubles (the solve's blocks, MINRES vectors, FP32 and double-float copies, start block and
-    // warm-start copy); with a nonlocal term the dense Fhat (FP64 + FP32) and its setup block.
+    // warm-start copy); the Gram's sums and the update's slab are another 2% of those blocks
+    // at most, within the constant on small problems; with a nonlocal term the dense Fhat (FP64 + FP32) and its setup block.
     // The server scales this by the largest measured footprint / estimate seen so far.
     const int64_t w = nev + std::max(3, (nev + 9) / 10);
     const double fill = 16.5 * std::pow((double)std::max<int64_t>(n, 1000) / 47620.0, 0.35);

@@ -14,7 +14,7 @@
 //
 // The rows are worked off in slabs: results go to a scratch block, since the tiles of a row read all of it, and
 // are copied over Z0 when the slab is done.  One slab of 19,456 rows with q = 538, k = 282: exponents 26 us, guard
-// 103, digits and products 230, entries in FP64 14, copy 15.  All 334,272 rows: 7.19 ms, 22.67 with pairs.  Bound
+// 103, digits and products 230, entries in FP64 14, copy 15.  All 334,272 rows: 6.93 ms, 22.65 with pairs.  Bound
 // by cutting Z (once per 64 columns; 16 clocks of four warps per value) and, in the guard, by the latency of the
 // loads of one CTA per SM; the digit products alone are 1.8 ms.
 #include <algorithm>
