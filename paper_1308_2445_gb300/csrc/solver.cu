@@ -1187,9 +1187,10 @@ int hbsd_gram_df64(const double* Z, int64_t ldz, const double* ZH, int64_t ldzh,
         if (!Z || !ZH || !ZS || !HR || !SR || n <= 0 || q <= 0) return fail(HBSD_ERR_ARG, "bad arguments");
         if (!ld_ok(ldz, q) || !ld_ok(ldzh, q) || !ld_ok(ldzs, q)) return fail(HBSD_ERR_ARG, "leading dimension below the block width");
         Session* S = scratch_session();
-        HBSD_TRY(gram_df64_reserve(S, n, q));
-        return gram2_df64(S, Z, ldz, q, nullptr, 0, 0, ZH, ldzh, nullptr, 0, ZS, ldzs, nullptr, 0, n, HR, SR,
-                          (cudaStream_t)stream);
+        HBSD_TRY(gram2_df64(S, Z, ldz, q, nullptr, 0, 0, ZH, ldzh, nullptr, 0, ZS, ldzs, nullptr, 0, n, HR, SR,
+                            (cudaStream_t)stream));
+        (void)gram_df64_reserve(S, n, q);   // without room for it, only a later captured call fails
+        return HBSD_OK;
     });
 }
 
